@@ -460,23 +460,20 @@ geneo_status_t refactor_fp64(geneo_handle_s* h, const AssemblyOut& a, const int3
   GENEO_CUDA(cudaStreamSynchronize(s));
   std::vector<BandDesc> rd;
   int64_t tot = 0;
+  int blk_mask = 0;
   for (int j = 0; j < N; ++j) {
     if (!flag[j]) continue;
     const SubDesc& d = h->hsub[j];
-    const int n = isK ? d.nN : d.nD, w = isK ? d.wK : d.wA;
-    rd.push_back(BandDesc{tot, n, w, j, band_ld(w), 0, -1});
+    const int n = isK ? d.nN : d.nD, w = band_w(isK ? d.wK : d.wA);
+    rd.push_back(BandDesc{tot, n, w, j, band_ld(w), sweep_block(w, true), -1});
+    blk_mask |= rd.back().blk;
     tot += (int64_t)n * band_ld(w);
     r->maxw = std::max(r->maxw, w);
     r->maxn = std::max(r->maxn, n);
   }
   r->count = (int)rd.size();
   if (rd.empty()) return GENEO_OK;
-  int64_t dv = tot;
-  for (BandDesc& b : rd) {
-    b.dinv = dv;
-    dv += dinv_elems(b.n);
-  }
-  GENEO_TRY(mem.get(&r->band, (size_t)dv));
+  GENEO_TRY(mem.get(&r->band, (size_t)tot));
   GENEO_TRY(mem.get(&r->desc, rd.size()));
   GENEO_CUDA(cudaMemsetAsync(r->band, 0, sizeof(double) * tot, s));
   GENEO_CUDA(cudaMemcpyAsync(r->desc, rd.data(), sizeof(BandDesc) * rd.size(), cudaMemcpyHostToDevice, s));
@@ -487,7 +484,7 @@ geneo_status_t refactor_fp64(geneo_handle_s* h, const AssemblyOut& a, const int3
     k_band_fill_A<double><<<R, kT, 0, s>>>(h->dsub, r->desc, h->dpos, h->nToD, a.lrow, a.lcol, a.lA, r->band);
   note_launch();
   GENEO_CUDA(cudaGetLastError());
-  GENEO_TRY(band_potrf<double>(r->band, r->desc, R, r->maxw, r->maxn, h->dstat, s));
+  GENEO_TRY(band_potrf<double>(r->band, r->desc, R, r->maxw, r->maxn, blk_mask, h->dstat, s));
   for (const BandDesc& b : rd) hmain[b.id].n = 0;
   GENEO_CUDA(cudaMemcpyAsync(dmain, hmain.data(), sizeof(BandDesc) * N, cudaMemcpyHostToDevice, s));
   return GENEO_OK;
@@ -702,10 +699,10 @@ geneo_status_t assemble_local(geneo_handle_s* h, const geneo_problem_t* p, Assem
     d.wA = hwA[j];
     d.bandK = bandK_tot;
     d.bandA = bandA_tot;
-    bandK_tot += (int64_t)d.nN * band_ld(d.wK);
-    bandA_tot += (int64_t)d.nD * band_ld(d.wA);
-    out.maxwK = std::max(out.maxwK, d.wK);
-    h->maxwA = std::max(h->maxwA, d.wA);
+    bandK_tot += (int64_t)d.nN * band_ld(band_w(d.wK));
+    bandA_tot += (int64_t)d.nD * band_ld(band_w(d.wA));
+    out.maxwK = std::max(out.maxwK, band_w(d.wK));
+    h->maxwA = std::max(h->maxwA, band_w(d.wA));
     h->maxnD = std::max(h->maxnD, d.nD);
   }
   GENEO_CUDA(cudaMemcpyAsync(h->dsub, h->hsub.data(), sizeof(SubDesc) * N, cudaMemcpyHostToDevice, s));
@@ -739,30 +736,33 @@ geneo_status_t assemble_local(geneo_handle_s* h, const geneo_problem_t* p, Assem
 
   // band storage, descriptors
   const size_t esz = h->fp32 ? sizeof(float) : sizeof(double);
-  // the inverted diagonal blocks follow all bands in the same allocation
   // with FP32 factors the bands are equilibrated (S A S, s = diag^{-1/2}):
   // FP32 Cholesky of the unscaled matrices breaks down at coefficient
-  // contrasts near 1e8; the row scalings follow the inverted blocks
+  // contrasts near 1e8; the row scalings follow the bands
   const bool equil = h->fp32;
-  int64_t dinvK_tot = 0, dinvA_tot = 0;
+  int64_t sclK_tot = 0, sclA_tot = 0;
   int maxnK = 0;
   for (const SubDesc& d : h->hsub) {
-    dinvK_tot += dinv_elems(d.nN) + (equil ? scl_elems(d.nN) : 0);
-    dinvA_tot += dinv_elems(d.nD) + (equil ? scl_elems(d.nD) : 0);
+    sclK_tot += equil ? scl_elems(d.nN) : 0;
+    sclA_tot += equil ? scl_elems(d.nD) : 0;
     maxnK = std::max(maxnK, d.nN);
   }
-  GENEO_TRY(tmp.alloc(&out.bandK, esz * (size_t)std::max<int64_t>(bandK_tot + dinvK_tot, 1)));
-  GENEO_TRY(h->mem.alloc(&h->bandA, esz * (size_t)std::max<int64_t>(bandA_tot + dinvA_tot, 1)));
+  GENEO_TRY(tmp.alloc(&out.bandK, esz * (size_t)std::max<int64_t>(bandK_tot + sclK_tot, 1)));
+  GENEO_TRY(h->mem.alloc(&h->bandA, esz * (size_t)std::max<int64_t>(bandA_tot + sclA_tot, 1)));
   GENEO_CUDA(cudaMemsetAsync(out.bandK, 0, esz * bandK_tot, s));
   GENEO_CUDA(cudaMemsetAsync(h->bandA, 0, esz * bandA_tot, s));
   std::vector<BandDesc> bk(N), ba(N);
   int64_t dK = bandK_tot, dA = bandA_tot;
+  int maskK = 0, maskA = 0;  // block sizes of the sweeps
   for (int j = 0; j < N; ++j) {
     const SubDesc& d = h->hsub[j];
-    bk[j] = BandDesc{d.bandK, d.nN, d.wK, j, band_ld(d.wK), dK, equil ? dK + dinv_elems(d.nN) : -1};
-    ba[j] = BandDesc{d.bandA, d.nD, d.wA, j, band_ld(d.wA), dA, equil ? dA + dinv_elems(d.nD) : -1};
-    dK += dinv_elems(d.nN) + (equil ? scl_elems(d.nN) : 0);
-    dA += dinv_elems(d.nD) + (equil ? scl_elems(d.nD) : 0);
+    const int wK = band_w(d.wK), wA = band_w(d.wA);
+    bk[j] = BandDesc{d.bandK, d.nN, wK, j, band_ld(wK), sweep_block(wK, !h->fp32), equil ? dK : -1};
+    ba[j] = BandDesc{d.bandA, d.nD, wA, j, band_ld(wA), sweep_block(wA, !h->fp32), equil ? dA : -1};
+    dK += equil ? scl_elems(d.nN) : 0;
+    dA += equil ? scl_elems(d.nD) : 0;
+    maskK |= bk[j].blk;
+    maskA |= ba[j].blk;
   }
   // largest factorisations first: blocks are dispatched in index order, so
   // this shortens the tail of the last wave (descriptors carry their id)
@@ -832,15 +832,15 @@ geneo_status_t assemble_local(geneo_handle_s* h, const geneo_problem_t* p, Assem
     // failing the setup
     const float wt = (float)h->opt.fp32_pivot_tol;
     for (const FactorBatch& fb : batK)
-      GENEO_TRY(band_potrf<float>((float*)out.bandK, fb.d, (int)fb.h.size(), fb.maxw, fb.maxn, h->dstat, s, equil,
+      GENEO_TRY(band_potrf<float>((float*)out.bandK, fb.d, (int)fb.h.size(), fb.maxw, fb.maxn, maskK, h->dstat, s, equil,
                                   out.weak, wt, fb.plan.ok ? &fb.plan : nullptr));
     for (const FactorBatch& fb : batA)
-      GENEO_TRY(band_potrf<float>((float*)h->bandA, fb.d, (int)fb.h.size(), fb.maxw, fb.maxn, h->dstat, h->aux,
+      GENEO_TRY(band_potrf<float>((float*)h->bandA, fb.d, (int)fb.h.size(), fb.maxw, fb.maxn, maskA, h->dstat, h->aux,
                                   equil, out.weak + N, wt, fb.plan.ok ? &fb.plan : nullptr));
     h->factor_classes = (int)(batK.size() + batA.size());
   } else {
-    GENEO_TRY(band_potrf<double>((double*)out.bandK, fdK, N, out.maxwK, maxnK, h->dstat, s));
-    GENEO_TRY(band_potrf<double>((double*)h->bandA, fdA, N, h->maxwA, h->maxnD, h->dstat, h->aux));
+    GENEO_TRY(band_potrf<double>((double*)out.bandK, fdK, N, out.maxwK, maxnK, maskK, h->dstat, s));
+    GENEO_TRY(band_potrf<double>((double*)h->bandA, fdA, N, h->maxwA, h->maxnD, maskA, h->dstat, h->aux));
   }
   h->prof.end(pK, s);
   h->prof.end(pA, h->aux);

@@ -411,38 +411,6 @@ __global__ void k_band_scale_x(const T* __restrict__ base, const BandDesc* __res
     X[idx] *= (double)S[idx % d.n];
 }
 
-// Inverses M of the 16 x 16 diagonal blocks of a factored band (FP64
-// arithmetic, rounded to T), stored transposed (M(i, t) at 16 t + i): a
-// half-warp per block, lane c forms column c by forward substitution.  The solves apply these blocks as small products, so
-// no dependent chain of divisions sits on their sequential path.
-template <typename T>
-__global__ void __launch_bounds__(256)
-k_band_dinv(T* __restrict__ base, const BandDesc* __restrict__ descs) {
-  const BandDesc d = descs[blockIdx.y];
-  const int lane = threadIdx.x & 31, c = lane & 15;
-  const int blk = (blockIdx.x * 8 + (threadIdx.x >> 5)) * 2 + (lane >> 4);
-  const int nb = (d.n + 15) / 16;
-  if (blk >= nb || d.dinv < 0) return;
-  const int kb = blk * 16, b = min(16, d.n - kb), w = d.w, ld = d.ld;
-  const T* L = base + d.off;
-  double x[16];
-#pragma unroll
-  for (int r = 0; r < 16; ++r) {
-    double v = 0.0;
-    if (r < b && c < b && r >= c) {
-      v = r == c ? 1.0 : 0.0;
-#pragma unroll
-      for (int t = 0; t < r; ++t)
-        if (t >= c && r - t <= w) v -= (double)L[(int64_t)(kb + r) * ld + (t - r + w)] * x[t];
-      v /= (double)L[(int64_t)(kb + r) * ld + w];
-    }
-    x[r] = v;
-  }
-  T* D = base + d.dinv + (int64_t)blk * 256;
-#pragma unroll
-  for (int r = 0; r < 16; ++r) D[c * 16 + r] = (T)x[r];
-}
-
 // ---------------------------------------------------------------------------
 // Left-looking FP32 band Cholesky on the tensor cores.
 //
@@ -970,865 +938,6 @@ k_band_solve(const T* __restrict__ base, const BandDesc* __restrict__ descs,
       mbar_wait_bounded(&bars[v % kStages], (uint32_t)((v / kStages) & 1), st, d.id, v);
 }
 
-// One right-hand side with the whole vector resident in shared memory (the
-// preconditioner's local solves and the coarse solve).  The vector is read
-// once at the start and written once at the end, so no global access sits on
-// the sequential path of the sweeps; only the factor (band rows and the
-// inverted diagonal block) streams in.  Forward block (left-looking): row i
-// of the block is a dot product over the w solved entries to its left, split
-// over a half-warp (16 segments, shuffle reduction), then the inverted
-// diagonal block is applied.  Backward block (right-looking): the transposed
-// inverse is applied, then every thread updates rows above the block.
-template <typename T, int kStages>
-__global__ void __launch_bounds__(kThreads, sizeof(T) == 4 ? 2 : 1)
-k_band_solve_res(const T* __restrict__ base, const BandDesc* __restrict__ descs,
-                 double* __restrict__ xbase, const int64_t* __restrict__ xoff,
-                 const int32_t* __restrict__ nrhs_dev, const int32_t* __restrict__ skip, DevStatus* st) {
-  constexpr int SNB = 16;
-  const BandDesc d = descs[blockIdx.x];
-  // vectors, counts and skip flags are indexed by the subdomain id (a
-  // batch may hold a subset of the subdomains)
-  const int mi = d.id >= 0 ? d.id : (int)blockIdx.x;
-  if (skip && skip[mi]) return;
-  if (nrhs_dev && nrhs_dev[mi] <= 0) return;
-  const int n = d.n, w = d.w;
-  if (n <= 0) return;
-  const int ld = d.ld;
-  const T* L = base + d.off;
-  const T* Dg = base + d.dinv;
-  double* X = xbase + xoff[mi];
-
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw);             // kStages
-  T* stage = reinterpret_cast<T*>(smem_raw + 128);                    // kStages * SNB * ld
-  T* dstage = stage + (size_t)kStages * SNB * ld;                     // kStages * 256
-  T* vec = dstage + (size_t)kStages * 256;                            // n (padded to 4)
-  T* zb = vec + ((n + 3) & ~3);                                       // SNB
-  const int tid = threadIdx.x;
-  const int nb = (n + SNB - 1) / SNB;
-  const int nvis = 2 * nb;
-
-  if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) mbar_init(&bars[s], 1);
-    fence_barrier_init();
-  }
-  __syncthreads();
-  auto issue = [&](int v) {
-    const int blk = visit_block(v, nb), kb = blk * SNB;
-    const int b = min(SNB, n - kb);
-    const int s = v % kStages;
-    const uint32_t bytes = (uint32_t)((size_t)b * ld * sizeof(T));
-    fence_proxy_async();
-    mbar_arrive_expect_tx(&bars[s], bytes + 256 * (uint32_t)sizeof(T));
-    bulk_load(stage + (size_t)s * SNB * ld, L + (int64_t)kb * ld, bytes, &bars[s]);
-    bulk_load(dstage + (size_t)s * 256, Dg + (int64_t)blk * 256, 256 * sizeof(T), &bars[s]);
-  };
-  int issued = 0;  // copies issued by thread 0
-  if (tid == 0)
-    for (; issued < min(kStages - 1, nvis); ++issued) issue(issued);
-  const T* Sg = d.scl >= 0 ? base + d.scl : nullptr;  // equilibrated band: solve with S A S
-  for (int i = tid; i < n; i += kThreads) vec[i] = Sg ? (T)X[i] * Sg[i] : (T)X[i];
-  __syncthreads();
-  bool ok = true;
-  int waited = 0;  // stages this thread has waited for
-
-  for (int v = 0; v < nvis; ++v) {
-    const int s = v % kStages;
-    const uint32_t parity = (uint32_t)((v / kStages) & 1);
-    if (tid == 0 && ok && issued < nvis) issue(issued++);
-    const int kb = visit_block(v, nb) * SNB;
-    const int b = min(SNB, n - kb);
-    if (ok) {
-      ok = mbar_wait_bounded(&bars[s], parity, st, d.id, v);
-      waited += ok ? 1 : 0;
-    }
-    const T* S = stage + (size_t)s * SNB * ld;
-    const T* D = dstage + (size_t)s * 256;   // M(i, t) at D[16 t + i]
-    if (v < nb) {
-      // ---------------- forward: z_i = b_i - sum_{c < kb} L(kb+i, c) y_c
-      const int i = tid >> 4, sl = tid & 15;
-      T acc = T(0);
-      if (i < b) {
-        const int r = kb + i;
-        const int olo = max(0, w - r), ohi = w - i;  // band offsets of the columns [r - w, kb)
-        const int len = ohi - olo;
-        const T* sp = S + (size_t)i * ld + olo;
-        const T* vp = vec + (r - w + olo);
-        T a1 = T(0);
-        int j = sl;
-        for (; j + 16 < len; j += 32) {
-          acc += sp[j] * vp[j];
-          a1 += sp[j + 16] * vp[j + 16];
-        }
-        if (j < len) acc += sp[j] * vp[j];
-        acc += a1;
-      }
-#pragma unroll
-      for (int off = 8; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off, 16);
-      if (sl == 0 && i < b) zb[i] = vec[kb + i] - acc;
-      __syncthreads();
-      // y = M z
-      if (tid < b) {
-        T y = T(0);
-#pragma unroll
-        for (int t = 0; t < SNB; ++t)
-          if (t <= tid) y += D[t * SNB + tid] * zb[t];
-        vec[kb + tid] = y;
-      }
-    } else {
-      // ---------------- backward: x = M^T y, then rows above the block
-      if (tid < b) {
-        T x = T(0);
-#pragma unroll
-        for (int j = 0; j < SNB; ++j) {
-          const int i = (tid + j) & (SNB - 1);  // rotated: conflict-free reads of M
-          if (i >= tid && i < b) x += D[tid * SNB + i] * vec[kb + i];
-        }
-        zb[tid] = x;
-      }
-      __syncthreads();
-      if (tid < b) vec[kb + tid] = zb[tid];
-      // y_rr -= sum_t L(kb + t, rr) x_{kb+t} for rr in [kb - w, kb)
-      const int lo = max(0, kb - w);
-      for (int rr = lo + tid; rr < kb; rr += kThreads) {
-        const int tmax = min(b - 1, rr - kb + w);
-        T a0 = T(0), a1 = T(0);
-        int t = 0;
-        for (; t + 1 <= tmax; t += 2) {
-          a0 += S[t * ld + (rr - kb - t + w)] * zb[t];
-          a1 += S[(t + 1) * ld + (rr - kb - t - 1 + w)] * zb[t + 1];
-        }
-        if (t <= tmax) a0 += S[t * ld + (rr - kb - t + w)] * zb[t];
-        vec[rr] -= a0 + a1;
-      }
-    }
-    __syncthreads();
-  }
-  // after a timed-out wait, let the copies still in flight land (bounded)
-  if (tid == 0 && !ok)
-    for (int v = waited; v < issued; ++v)
-      mbar_wait_bounded(&bars[v % kStages], (uint32_t)((v / kStages) & 1), st, d.id, v);
-  if (!ok) return;
-  for (int i = tid; i < n; i += kThreads) X[i] = Sg ? (double)(vec[i] * Sg[i]) : (double)vec[i];
-}
-
-// One right-hand side for bands whose whole vector does not fit in shared
-// memory next to the staged rows (wide bands, long subdomains, FP64).  The
-// sweeps are those of k_band_solve_res (forward left-looking with the
-// inverted 16 x 16 diagonal blocks, backward right-looking), with the
-// vector kept as a window of the rows [kb - w - 16, kb + 16) in a ring of
-// `ring` slots (a power of two >= w + 32): the forward results go to X as
-// they are formed and come back into the ring during the backward sweep, one
-// block ahead.  The band rows stream in as half blocks of 8 rows through kHS
-// shared stages; warp 8 (one lane) issues the bulk copies as soon as a stage
-// is released (full / empty mbarriers, the empty ones counted by the 256
-// compute threads), so a stage is refilled while the other half of the
-// block is still being used.  The first half block of every block also
-// carries that block's inverted diagonal block.  Every wait is bounded; a
-// wait that gives up records GENEO_ERR_TIMEOUT and raises a block-wide
-// abort flag, and the copies already issued are waited for before exit.
-template <typename T, int kHS>
-__global__ void __launch_bounds__(kThreads + 32, 1)
-k_band_solve_ring(const T* __restrict__ base, const BandDesc* __restrict__ descs,
-                  double* __restrict__ xbase, const int64_t* __restrict__ xoff,
-                  const int32_t* __restrict__ nrhs_dev, const int32_t* __restrict__ skip, int ring,
-                  DevStatus* st) {
-  constexpr int SNB = 16, HB = 8;
-  const BandDesc d = descs[blockIdx.x];
-  const int mi = d.id >= 0 ? d.id : (int)blockIdx.x;
-  if (skip && skip[mi]) return;
-  if (nrhs_dev && nrhs_dev[mi] <= 0) return;
-  const int n = d.n, w = d.w;
-  if (n <= 0) return;
-  const int ld = d.ld;
-  const T* L = base + d.off;
-  const T* Dg = base + d.dinv;
-  const T* Sg = d.scl >= 0 ? base + d.scl : nullptr;  // equilibrated band: solve with S A S
-  double* X = xbase + xoff[mi];
-  const int rmask = ring - 1;
-
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint64_t* full = reinterpret_cast<uint64_t*>(smem_raw);  // kHS
-  uint64_t* empty = full + kHS;                             // kHS
-  volatile int* abort = reinterpret_cast<volatile int*>(empty + kHS);
-  T* stage = reinterpret_cast<T*>(smem_raw + 256);          // kHS * (HB * ld + 256)
-  const size_t hs_len = (size_t)HB * ld + 256;              // rows, then the diagonal block
-  T* vec = stage + (size_t)kHS * hs_len;                    // ring
-  T* zb = vec + ring;                                       // SNB
-  T* xs = zb + SNB;                                         // SNB
-  T* rhs = xs + SNB;                                        // SNB: right-hand side of the next block
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int nb = (n + SNB - 1) / SNB;
-  const int nvis = 2 * nb;
-  const int nhv = 2 * nvis;
-
-  if (tid == 0) {
-    for (int i = 0; i < kHS; ++i) {
-      mbar_init(&full[i], 1);
-      mbar_init(&empty[i], kThreads);
-    }
-    *abort = 0;
-    fence_barrier_init();
-  }
-  for (int i = tid; i < ring; i += blockDim.x) vec[i] = T(0);
-  for (int i = tid; i < SNB; i += blockDim.x) rhs[i] = (i < n) ? (Sg ? (T)X[i] * Sg[i] : (T)X[i]) : T(0);
-  __syncthreads();
-
-  auto bounded = [&](uint64_t* bar, uint32_t parity, int64_t where) -> bool {
-    for (int it = 0; it < (1 << 22); ++it) {
-      if (mbar_try_wait(bar, parity)) return true;
-      if ((it & 1023) == 1023 && *abort) return false;
-    }
-    *abort = 1;
-    record_error(st, GENEO_ERR_TIMEOUT, d.id, where);
-    return false;
-  };
-
-  if (wid == kThreads / 32) {
-    // ------------------------------------------------------------ copies
-    if (lane == 0) {
-      uint32_t iss[kHS];
-#pragma unroll
-      for (int i = 0; i < kHS; ++i) iss[i] = 0;
-      for (int hv = 0; hv < nhv && !*abort; ++hv) {
-        const int sl = hv % kHS;
-        if (hv >= kHS && !bounded(&empty[sl], (uint32_t)((hv / kHS - 1) & 1), hv)) break;
-        const int v = hv >> 1, h = hv & 1;
-        const int blk = visit_block(v, nb), kb = blk * SNB;
-        const int r0 = kb + HB * h, rows = max(0, min(HB, n - r0));
-        const uint32_t bytes = (uint32_t)((size_t)rows * ld * sizeof(T));
-        const uint32_t dbytes = h == 0 ? 256u * (uint32_t)sizeof(T) : 0u;
-        T* dst = stage + (size_t)sl * hs_len;
-        fence_proxy_async();
-        mbar_arrive_expect_tx(&full[sl], bytes + dbytes);
-        if (bytes) bulk_load(dst, L + (int64_t)r0 * ld, bytes, &full[sl]);
-        if (dbytes) bulk_load(dst + (size_t)HB * ld, Dg + (int64_t)blk * 256, dbytes, &full[sl]);
-        ++iss[sl];
-      }
-      // let every copy issued land before the block exits
-#pragma unroll
-      for (int i = 0; i < kHS; ++i)
-        if (iss[i] > 0)
-          for (int it = 0; it < (1 << 22) && !mbar_try_wait(&full[i], (iss[i] - 1) & 1); ++it) {
-          }
-    }
-    return;
-  }
-
-  // ------------------------------------------------------------ sweeps
-  int lo = n;  // lowest row in the ring during the backward sweep
-  for (int v = 0; v < nvis; ++v) {
-    const int kb = visit_block(v, nb) * SNB;
-    const int b = min(SNB, n - kb);
-    const int hv0 = 2 * v, s0 = hv0 % kHS, s1 = (hv0 + 1) % kHS;
-    const uint32_t p0 = (uint32_t)((hv0 / kHS) & 1), p1 = (uint32_t)(((hv0 + 1) / kHS) & 1);
-    const T* H0 = stage + (size_t)s0 * hs_len;  // rows kb .. kb + 7, then M
-    const T* H1 = stage + (size_t)s1 * hs_len;  // rows kb + 8 .. kb + 15
-    const T* D = H0 + (size_t)HB * ld;           // M(i, t) at D[16 t + i]
-    if (v < nb) {
-      // ---------------- forward: z_i = b_i - sum_{c < kb} L(kb+i, c) y_c
-      T nxt = T(0);  // right-hand side of the next block (thread i < 16)
-      if (tid < SNB && v + 1 < nb && kb + SNB + tid < n) {
-        const int r = kb + SNB + tid;
-        nxt = Sg ? (T)X[r] * Sg[r] : (T)X[r];
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        if (!*abort) bounded(h ? &full[s1] : &full[s0], h ? p1 : p0, v);
-        const T* S = h ? H1 : H0;
-        const int i = HB * h + wid;  // one row per warp
-        T acc = T(0);
-        if (i < b) {
-          const int r = kb + i;
-          const int olo = max(0, w - r), ohi = w - i;  // band offsets of the columns [r - w, kb)
-          const T* sp = S + (size_t)wid * ld;
-          T a1 = T(0);
-          int j = olo + lane;
-          for (; j + 32 < ohi; j += 64) {
-            acc += sp[j] * vec[(r - w + j) & rmask];
-            a1 += sp[j + 32] * vec[(r - w + j + 32) & rmask];
-          }
-          if (j < ohi) acc += sp[j] * vec[(r - w + j) & rmask];
-          acc += a1;
-        }
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-        if (lane == 0 && i < b) zb[i] = rhs[i] - acc;
-        if (h == 1) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[s1])) : "memory");
-      }
-      asm volatile("bar.sync 1, 256;" ::: "memory");
-      // y = M z
-      if (tid < b) {
-        T y = T(0);
-#pragma unroll
-        for (int t = 0; t < SNB; ++t)
-          if (t <= tid) y += D[t * SNB + tid] * zb[t];
-        vec[(kb + tid) & rmask] = y;
-        X[kb + tid] = (double)y;
-      }
-      if (tid < SNB) rhs[tid] = nxt;
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[s0])) : "memory");
-      if (v == nb - 1) lo = max(0, kb - w);
-    } else {
-      // ---------------- backward: x = M^T y, then rows above the block
-      const int nlo = max(0, kb - SNB - w);
-      T er = T(0);  // row entering the ring (forward result)
-      if (tid < lo - nlo) er = (T)X[nlo + tid];
-      if (!*abort) bounded(&full[s0], p0, v);
-      if (!*abort) bounded(&full[s1], p1, v);
-      if (tid < b) {
-        T x = T(0);
-#pragma unroll
-        for (int j = 0; j < SNB; ++j) {
-          const int i = (tid + j) & (SNB - 1);  // rotated: conflict-free reads of M
-          if (i >= tid && i < b) x += D[tid * SNB + i] * vec[(kb + i) & rmask];
-        }
-        xs[tid] = x;
-        X[kb + tid] = Sg ? (double)(x * Sg[kb + tid]) : (double)x;
-      }
-      asm volatile("bar.sync 1, 256;" ::: "memory");
-      // y_rr -= sum_t L(kb + t, rr) x_t for rr in [lo, kb)
-      for (int rr = lo + tid; rr < kb; rr += kThreads) {
-        const int tmax = min(b - 1, rr - kb + w);
-        T a0 = T(0), a1 = T(0);
-        int t = 0;
-        for (; t + 1 <= tmax; t += 2) {
-          const T* r0p = t < HB ? H0 + (size_t)t * ld : H1 + (size_t)(t - HB) * ld;
-          const T* r1p = t + 1 < HB ? H0 + (size_t)(t + 1) * ld : H1 + (size_t)(t + 1 - HB) * ld;
-          a0 += r0p[rr - kb - t + w] * xs[t];
-          a1 += r1p[rr - kb - t - 1 + w] * xs[t + 1];
-        }
-        if (t <= tmax) {
-          const T* r0p = t < HB ? H0 + (size_t)t * ld : H1 + (size_t)(t - HB) * ld;
-          a0 += r0p[rr - kb - t + w] * xs[t];
-        }
-        vec[rr & rmask] -= a0 + a1;
-      }
-      if (tid < lo - nlo) vec[(nlo + tid) & rmask] = er;
-      lo = nlo;
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[s0])) : "memory");
-      asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&empty[s1])) : "memory");
-    }
-    asm volatile("bar.sync 1, 256;" ::: "memory");
-  }
-}
-
-// Several right-hand sides (the eigensolver's K_j^{-1} blocks), at most
-// 2 CT per launch.  The solved rows of the last w + 32 block rows sit in a
-// shared ring stored row-major (row stride KP = 2 CT + 4 values, so rows
-// taken by consecutive threads fall in distinct banks).
-// Forward block: the (16 x w) x (w x k) product with the solved rows is cut
-// into eight ranges of the band, one per warp; lane (i, g) owns row i and
-// columns [g CT, g CT + CT), reads one factor value and CT/4 four-wide ring
-// vectors per band position, and the warps' partial sums are added in a
-// fixed order; the inverted diagonal block is then applied (one output per
-// thread).  Backward block: the transposed inverse is applied, then the ring
-// rows above the block are updated, one (row, four columns) item per thread.
-// Right-hand sides of the next block and the rows that enter the ring are
-// loaded one block ahead.
-template <typename T, typename A, int CT, int kStages>
-__global__ void __launch_bounds__(kThreads, 1)
-k_band_solve_multi(const T* __restrict__ base, const BandDesc* __restrict__ descs,
-                   double* __restrict__ xbase, const int64_t* __restrict__ xoff, int col0, int kcap,
-                   const int32_t* __restrict__ nrhs_dev, const int32_t* __restrict__ skip, int ring,
-                   DevStatus* st) {
-  constexpr int SNB = 16;
-  constexpr int KP = 2 * CT + 4;
-  constexpr int NW = kThreads / 32;
-  const BandDesc d = descs[blockIdx.x];
-  // vectors, counts and skip flags are indexed by the subdomain id (a
-  // batch may hold a subset of the subdomains)
-  const int mi = d.id >= 0 ? d.id : (int)blockIdx.x;
-  if (skip && skip[mi]) return;
-  // column split: block y takes the columns [2 CT y, 2 CT (y + 1)) of the kcap
-  col0 += (int)blockIdx.y * 2 * CT;
-  kcap -= (int)blockIdx.y * 2 * CT;
-  int k = min(kcap, 2 * CT);
-  if (nrhs_dev) k = min(k, nrhs_dev[mi] - col0);
-  if (k <= 0) return;
-  const int n = d.n, w = d.w;
-  if (n <= 0) return;
-  const int ld = d.ld;
-  const T* L = base + d.off;
-  const T* Dg = base + d.dinv;
-  double* X = xbase + xoff[mi] + (int64_t)col0 * n;
-  const int rmask = ring - 1;  // ring: power of two >= w + 2 SNB
-
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw);      // kStages
-  T* stage = reinterpret_cast<T*>(smem_raw + 128);             // kStages * SNB * ld
-  T* dstage = stage + (size_t)kStages * SNB * ld;              // kStages * 256
-  A* win = reinterpret_cast<A*>(dstage + (size_t)kStages * 256);  // ring * KP
-  A* red = win + (size_t)ring * KP;                               // NW * SNB * KP
-  A* zb = red + (size_t)NW * SNB * KP;                            // SNB * KP
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int nb = (n + SNB - 1) / SNB;
-  const int nvis = 2 * nb;
-
-  for (int idx = tid; idx < ring * KP; idx += kThreads) win[idx] = A();
-  if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) mbar_init(&bars[s], 1);
-    fence_barrier_init();
-  }
-  __syncthreads();
-  auto issue = [&](int v) {
-    const int blk = visit_block(v, nb), kb = blk * SNB;
-    const int b = min(SNB, n - kb);
-    const int s = v % kStages;
-    const uint32_t bytes = (uint32_t)((size_t)b * ld * sizeof(T));
-    fence_proxy_async();
-    mbar_arrive_expect_tx(&bars[s], bytes + 256 * (uint32_t)sizeof(T));
-    bulk_load(stage + (size_t)s * SNB * ld, L + (int64_t)kb * ld, bytes, &bars[s]);
-    bulk_load(dstage + (size_t)s * 256, Dg + (int64_t)blk * 256, 256 * sizeof(T), &bars[s]);
-  };
-  int issued = 0;
-  if (tid == 0)
-    for (; issued < min(kStages - 1, nvis); ++issued) issue(issued);
-  // element e of a (16 rows x k columns) block handled by this thread:
-  // idx = tid + e * kThreads, column idx >> 4, row idx & 15
-  auto load_rows = [&](int r0, int cnt, A* out) {
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int idx = tid + e * kThreads, c = idx >> 4, t = idx & 15;
-      out[e] = (c < k && t < cnt) ? to_arith<A>(X[(int64_t)c * n + r0 + t]) : A();
-    }
-  };
-  A xr[2];
-  load_rows(0, min(SNB, n), xr);
-  bool ok = true;
-  int waited = 0;
-  int lo = n;
-
-  for (int v = 0; v < nvis; ++v) {
-    const int s = v % kStages;
-    const uint32_t parity = (uint32_t)((v / kStages) & 1);
-    if (tid == 0 && ok && issued < nvis) issue(issued++);
-    const int kb = visit_block(v, nb) * SNB;
-    const int b = min(SNB, n - kb);
-    const T* S = stage + (size_t)s * SNB * ld;
-    const T* D = dstage + (size_t)s * 256;   // M(i, t) at D[16 t + i]
-    if (v < nb) {
-      // ---------------- forward
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int idx = tid + e * kThreads, c = idx >> 4, t = idx & 15;
-        if (c < k) zb[t * KP + c] = xr[e];
-      }
-      if (v + 1 < nb) load_rows(kb + SNB, min(SNB, n - kb - SNB), xr);
-      if (ok) {
-        ok = mbar_wait_bounded(&bars[s], parity, st, d.id, v);
-        waited += ok ? 1 : 0;
-      }
-      {
-        const int i = lane & 15, g = lane >> 4;
-        A acc[CT];
-#pragma unroll
-        for (int c = 0; c < CT; ++c) acc[c] = A();
-        if (i < b) {
-          const int ua = (int)((int64_t)w * wid / NW), ub = (int)((int64_t)w * (wid + 1) / NW);
-          const int u0 = max(ua, max(i, w - kb));
-          const T* srow = S + (size_t)i * ld - i;   // srow[u] = L(kb + i, kb - w + u)
-          for (int u = u0; u < ub; ++u) {
-            const A a = to_arith<A>(srow[u]);
-            const A* rr = win + (size_t)((kb - w + u) & rmask) * KP + g * CT;
-#pragma unroll
-            for (int q = 0; q < CT / 4; ++q) {
-              A xv[4];
-              load4(rr + 4 * q, xv);
-#pragma unroll
-              for (int z = 0; z < 4; ++z) acc[4 * q + z] += a * xv[z];
-            }
-          }
-        }
-        A* rp = red + (size_t)(wid * SNB + i) * KP + g * CT;
-#pragma unroll
-        for (int q = 0; q < CT / 4; ++q) store4(rp + 4 * q, acc + 4 * q);
-      }
-      __syncthreads();
-      for (int idx = tid; idx < SNB * k; idx += kThreads) {
-        const int c = idx >> 4, t = idx & 15;
-        A sum = A();
-#pragma unroll
-        for (int ww = 0; ww < NW; ++ww) sum += red[(size_t)(ww * SNB + t) * KP + c];
-        zb[t * KP + c] -= sum;
-      }
-      __syncthreads();
-      // y = M z: one (row, column) output per thread
-      for (int idx = tid; idx < SNB * k; idx += kThreads) {
-        const int c = idx >> 4, i = idx & 15;
-        if (i < b) {
-          A y = A();
-#pragma unroll
-          for (int t = 0; t < SNB; ++t)
-            if (t <= i) y += to_arith<A>(D[t * SNB + i]) * zb[t * KP + c];
-          win[(size_t)((kb + i) & rmask) * KP + c] = y;
-          X[(int64_t)c * n + kb + i] = to_double(y);
-        }
-      }
-      if (v == nb - 1) lo = max(0, kb - w);
-    } else {
-      // ---------------- backward
-      const int nlo = max(0, kb - SNB - w);
-      A er[2];
-      load_rows(nlo, lo - nlo, er);  // rows entering the ring (forward results)
-      if (ok) {
-        ok = mbar_wait_bounded(&bars[s], parity, st, d.id, v);
-        waited += ok ? 1 : 0;
-      }
-      // x = M^T y into zb (the ring rows of the block are not needed again)
-      for (int idx = tid; idx < SNB * k; idx += kThreads) {
-        const int c = idx >> 4, t = idx & 15;
-        A x = A();
-        if (t < b) {
-#pragma unroll
-          for (int j = 0; j < SNB; ++j) {
-            const int i = (t + j) & (SNB - 1);  // rotated: conflict-free reads of M
-            if (i >= t && i < b) x += to_arith<A>(D[t * SNB + i]) * win[(size_t)((kb + i) & rmask) * KP + c];
-          }
-          X[(int64_t)c * n + kb + t] = to_double(x);
-        }
-        zb[t * KP + c] = x;
-      }
-      __syncthreads();
-      // rows [lo, kb): y_rr -= sum_t L(kb + t, rr) x_{kb+t}, items (row, four columns)
-      const int cnt = kb - lo, nq = (k + 3) >> 2;
-      for (int it = tid; it < cnt * nq; it += kThreads) {
-        const int rr = lo + it % cnt, q = it / cnt;
-        const int tmax = min(b - 1, rr - kb + w);
-        A* yrow = win + (size_t)(rr & rmask) * KP + 4 * q;
-        A acc[4];
-        load4(yrow, acc);
-        for (int t = 0; t <= tmax; ++t) {
-          const A lv = to_arith<A>(S[t * ld + (rr - kb - t + w)]);
-          A xv[4];
-          load4(zb + t * KP + 4 * q, xv);
-#pragma unroll
-          for (int z = 0; z < 4; ++z) acc[z] -= lv * xv[z];
-        }
-        store4(yrow, acc);
-      }
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int idx = tid + e * kThreads, c = idx >> 4, t = idx & 15;
-        if (c < k && t < lo - nlo) win[(size_t)((nlo + t) & rmask) * KP + c] = er[e];
-      }
-      lo = nlo;
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && !ok)
-    for (int v = waited; v < issued; ++v)
-      mbar_wait_bounded(&bars[v % kStages], (uint32_t)((v / kStages) & 1), st, d.id, v);
-}
-
-// Tensor-core variant of the multi-right-hand-side solve for FP32 factors:
-// the same sweeps as k_band_solve_multi, with the two contractions done by
-// m16n8k8 TF32 MMAs in three passes (hi*hi + hi*lo + lo*hi, about FP32
-// accuracy):
-//  forward  (16 x w) x (w x k): rows of the block against the solved ring
-//           rows, the band cut into eight k-ranges (one per warp), partial
-//           sums added in a fixed order;
-//  backward (w x 16) x (16 x k): ring rows above the block minus L^T x, one
-//           16-row tile per warp at a time, the ring values as the MMA's C.
-// k <= 8 NT columns per launch.  The ring holds row r at slot r mod ring
-// (ring a power of two >= w + 2 SNB); its row stride RP puts the four
-// k-rows of a B fragment in distinct eight-bank groups: by padding (8, 24,
-// 40 values for NT = 1, 3, 4) or, for NT = 2, with 16 values and the column
-// halves swapped (column c at c ^ 8) on slots with bit 1 set.  With NT <= 2
-// the block is sized for two resident blocks per SM.
-template <int NT>
-struct MtcKP { static constexpr int v = NT == 1 ? 8 : (NT == 4 ? 40 : 24); };
-template <int NT>
-struct MtcRP { static constexpr int v = NT == 2 ? 16 : MtcKP<NT>::v; };
-
-template <int NT, int kStages, int PASSES>
-__global__ void __launch_bounds__(kThreads, NT <= 2 ? 2 : 1)
-k_band_solve_mtc(const float* __restrict__ base, const BandDesc* __restrict__ descs,
-                 double* __restrict__ xbase, const int64_t* __restrict__ xoff, int col0, int kcap,
-                 const int32_t* __restrict__ nrhs_dev, const int32_t* __restrict__ skip, int ring,
-                 DevStatus* st) {
-  constexpr int SNB = 16;
-  constexpr int KP = MtcKP<NT>::v;   // row stride of zb and of the partial sums
-  constexpr int RP = MtcRP<NT>::v;   // row stride of the ring
-  constexpr bool SWZ = NT == 2;
-  constexpr int NW = kThreads / 32;
-  const BandDesc d = descs[blockIdx.x];
-  // vectors, counts and skip flags are indexed by the subdomain id (a
-  // batch may hold a subset of the subdomains)
-  const int mi = d.id >= 0 ? d.id : (int)blockIdx.x;
-  if (skip && skip[mi]) return;
-  // column split: block y takes the columns [8 NT y, 8 NT (y + 1)) of the kcap
-  col0 += (int)blockIdx.y * 8 * NT;
-  kcap -= (int)blockIdx.y * 8 * NT;
-  int k = min(kcap, 8 * NT);
-  if (nrhs_dev) k = min(k, nrhs_dev[mi] - col0);
-  if (k <= 0) return;
-  const int n = d.n, w = d.w;
-  if (n <= 0) return;
-  const int ld = d.ld;
-  const float* L = base + d.off;
-  const float* Dg = base + d.dinv;
-  double* X = xbase + xoff[mi] + (int64_t)col0 * n;
-  const int rmask = ring - 1;
-  auto slot = [&](int r) { return r & rmask; };
-
-  extern __shared__ __align__(128) unsigned char smem_raw[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem_raw);      // kStages
-  float* stage = reinterpret_cast<float*>(smem_raw + 128);     // kStages * SNB * ld
-  float* dstage = stage + (size_t)kStages * SNB * ld;          // kStages * 256
-  float* win = dstage + (size_t)kStages * 256;                 // ring * RP
-  float* red = win + (size_t)ring * RP;                        // NW * SNB * KP
-  float* zb = red + (size_t)NW * SNB * KP;                     // SNB * KP
-  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int g = lane >> 2, tg = lane & 3;
-  const int nb = (n + SNB - 1) / SNB;
-  const int nvis = 2 * nb;
-
-  // columns >= k stay zero in the ring and in zb
-  for (int idx = tid; idx < ring * RP; idx += kThreads) win[idx] = 0.f;
-  auto rptr = [&](int r, int c) -> float* {
-    const int sl = slot(r);
-    return win + (size_t)sl * RP + (SWZ ? (c ^ ((sl << 2) & 8)) : c);
-  };
-  for (int idx = tid; idx < SNB * KP; idx += kThreads) zb[idx] = 0.f;
-  if (tid == 0) {
-    for (int s = 0; s < kStages; ++s) mbar_init(&bars[s], 1);
-    fence_barrier_init();
-  }
-  __syncthreads();
-  auto issue = [&](int v) {
-    const int blk = visit_block(v, nb), kb = blk * SNB;
-    const int b = min(SNB, n - kb);
-    const int s = v % kStages;
-    const uint32_t bytes = (uint32_t)((size_t)b * ld * sizeof(float));
-    fence_proxy_async();
-    mbar_arrive_expect_tx(&bars[s], bytes + 256 * (uint32_t)sizeof(float));
-    bulk_load(stage + (size_t)s * SNB * ld, L + (int64_t)kb * ld, bytes, &bars[s]);
-    bulk_load(dstage + (size_t)s * 256, Dg + (int64_t)blk * 256, 256 * sizeof(float), &bars[s]);
-  };
-  int issued = 0;
-  if (tid == 0)
-    for (; issued < min(kStages - 1, nvis); ++issued) issue(issued);
-  const float* Sg = d.scl >= 0 ? base + d.scl : nullptr;  // equilibrated band: solve with S A S
-  // rows of the (16 x k) block of this thread; `scaled` multiplies by s
-  // (right-hand sides), the forward results re-entering the ring are not
-  auto load_rows = [&](int r0, int cnt, float* out, bool scaled) {
-#pragma unroll
-    for (int e = 0; e < 2; ++e) {
-      const int idx = tid + e * kThreads, c = idx >> 4, t = idx & 15;
-      float v = 0.f;
-      if (c < k && t < cnt) {
-        v = (float)X[(int64_t)c * n + r0 + t];
-        if (scaled && Sg) v *= Sg[r0 + t];
-      }
-      out[e] = v;
-    }
-  };
-  float xr[2];
-  load_rows(0, min(SNB, n), xr, true);
-  bool ok = true;
-  int waited = 0;
-  int lo = n;
-  const int nsteps = (w + 7) >> 3;  // k-steps of eight band positions
-  const int s0 = (nsteps * wid) / NW, s1 = (nsteps * (wid + 1)) / NW;
-
-  for (int v = 0; v < nvis; ++v) {
-    const int s = v % kStages;
-    const uint32_t parity = (uint32_t)((v / kStages) & 1);
-    if (tid == 0 && ok && issued < nvis) issue(issued++);
-    const int kb = visit_block(v, nb) * SNB;
-    const int b = min(SNB, n - kb);
-    const float* S = stage + (size_t)s * SNB * ld;
-    const float* D = dstage + (size_t)s * 256;   // M(i, t) at D[16 t + i]
-    if (v < nb) {
-      // ---------------- forward
-      // right-hand sides of this block (element e of this thread), kept in
-      // registers while the next block's are fetched
-      float bcur[2];
-#pragma unroll
-      for (int e = 0; e < 2; ++e) bcur[e] = xr[e];
-      if (v + 1 < nb) load_rows(kb + SNB, min(SNB, n - kb - SNB), xr, true);
-      if (ok) {
-        ok = mbar_wait_bounded(&bars[s], parity, st, d.id, v);
-        waited += ok ? 1 : 0;
-      }
-      {
-        // A(i, u) = L(kb + i, kb - w + u) = S[i ld + u - i] for u >= i and
-        // u >= w - kb (rows i = g, g + 8); B(u, c) = ring row kb - w + u
-        float acc[NT][3][4];
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-          for (int p = 0; p < 3; ++p)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) acc[nt][p][q] = 0.f;
-        const bool va = g < b, vb = g + 8 < b;
-        const int ia = g * (ld - 1), ib = (g + 8) * (ld - 1);
-        const int kfull = max(15, w - kb);   // from here every row's element is in band
-        for (int st8 = s0; st8 < s1; ++st8) {
-          const int u0 = 8 * st8;
-          const int k1 = u0 + tg, k2 = u0 + tg + 4;
-          const bool masked = u0 < kfull || u0 + 8 > w;
-          float x[4];
-          if (!masked) {
-            x[0] = va ? S[ia + k1] : 0.f;
-            x[1] = vb ? S[ib + k1] : 0.f;
-            x[2] = va ? S[ia + k2] : 0.f;
-            x[3] = vb ? S[ib + k2] : 0.f;
-          } else {
-            const int lo0 = max(0, w - kb);
-            x[0] = (va && k1 < w && k1 >= g && k1 >= lo0) ? S[ia + k1] : 0.f;
-            x[1] = (vb && k1 < w && k1 >= g + 8 && k1 >= lo0) ? S[ib + k1] : 0.f;
-            x[2] = (va && k2 < w && k2 >= g && k2 >= lo0) ? S[ia + k2] : 0.f;
-            x[3] = (vb && k2 < w && k2 >= g + 8 && k2 >= lo0) ? S[ib + k2] : 0.f;
-          }
-          uint32_t ah[4], al[4];
-#pragma unroll
-          for (int q = 0; q < 4; ++q) split_tf32(x[q], ah[q], al[q]);
-          const int sl1 = slot(kb - w + k1), sl2 = slot(kb - w + k2);
-          const float* r1 = win + (size_t)sl1 * RP + g;
-          const float* r2 = win + (size_t)sl2 * RP + g;
-          const int x1 = SWZ ? ((sl1 >> 1) & 1) : 0, x2 = SWZ ? ((sl2 >> 1) & 1) : 0;
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            uint32_t bh[2], bl[2];
-            split_tf32(r1[8 * (nt ^ x1)], bh[0], bl[0]);
-            split_tf32(r2[8 * (nt ^ x2)], bh[1], bl[1]);
-            if (PASSES == 3) {
-              mma_tf32(acc[nt][0], al, bh);
-              mma_tf32(acc[nt][1], ah, bl);
-            }
-            mma_tf32(acc[nt][2], ah, bh);
-          }
-        }
-        // partial sums: rows g, g + 8, columns 8 nt + 2 tg (+1)
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            const int row = g + ((q & 2) ? 8 : 0), col = 8 * nt + 2 * tg + (q & 1);
-            red[(size_t)(wid * SNB + row) * KP + col] = (acc[nt][0][q] + acc[nt][1][q]) + acc[nt][2][q];
-          }
-      }
-      __syncthreads();
-      // z = b - (the warps' partial sums) and y = M z for element (row t,
-      // column c) of this thread: the 16 rows of a column are the 16 lanes
-      // of one half-warp, which pass z to each other by shuffles (rows past
-      // the block end hold z = 0)
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int idx = tid + e * kThreads;
-        if (idx < SNB * k) {
-          const int c = idx >> 4, t = idx & 15;
-          float sum = 0.f;
-#pragma unroll
-          for (int ww = 0; ww < NW; ++ww) sum += red[(size_t)(ww * SNB + t) * KP + c];
-          const float z = bcur[e] - sum;
-          const unsigned hm = 0xffffu << (lane & 16);
-          float y = 0.f;
-#pragma unroll
-          for (int u = 0; u < SNB; ++u) {
-            const float zu = __shfl_sync(hm, z, u, 16);
-            if (u <= t) y += D[u * SNB + t] * zu;
-          }
-          if (t < b) {
-            *rptr(kb + t, c) = y;
-            X[(int64_t)c * n + kb + t] = (double)y;
-          }
-        }
-      }
-      if (v == nb - 1) lo = max(0, kb - w);
-    } else {
-      // ---------------- backward
-      const int nlo = max(0, kb - SNB - w);
-      float er[2];
-      load_rows(nlo, lo - nlo, er, false);  // rows entering the ring (forward results)
-      if (ok) {
-        ok = mbar_wait_bounded(&bars[s], parity, st, d.id, v);
-        waited += ok ? 1 : 0;
-      }
-      // x = M^T y into zb (the ring rows of the block are not needed again)
-      for (int idx = tid; idx < SNB * k; idx += kThreads) {
-        const int c = idx >> 4, t = idx & 15;
-        float x = 0.f;
-        if (t < b) {
-#pragma unroll
-          for (int j = 0; j < SNB; ++j) {
-            const int i = (t + j) & (SNB - 1);  // rotated: conflict-free reads of M
-            if (i >= t && i < b) x += D[t * SNB + i] * *rptr(kb + i, c);
-          }
-          X[(int64_t)c * n + kb + t] = Sg ? (double)(x * Sg[kb + t]) : (double)x;
-        }
-        zb[t * KP + c] = x;
-      }
-      __syncthreads();
-      // rows [lo, kb): y_rr -= sum_t L(kb + t, rr) x_t, 16-row tiles
-      {
-        uint32_t bh[2][NT][2], bl[2][NT][2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            split_tf32(zb[(8 * h + tg) * KP + 8 * nt + g], bh[h][nt][0], bl[h][nt][0]);
-            split_tf32(zb[(8 * h + tg + 4) * KP + 8 * nt + g], bh[h][nt][1], bl[h][nt][1]);
-          }
-        const int cnt = kb - lo;
-        const int ntile = (cnt + 15) >> 4;
-        for (int tile = wid; tile < ntile; tile += NW) {
-          const int ra = lo + 16 * tile + g, rb = ra + 8;
-          float cacc[NT][4];
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            const int col = 8 * nt + 2 * tg;
-            const float2 ya = ra < kb ? *reinterpret_cast<const float2*>(rptr(ra, col)) : make_float2(0.f, 0.f);
-            const float2 yb = rb < kb ? *reinterpret_cast<const float2*>(rptr(rb, col)) : make_float2(0.f, 0.f);
-            cacc[nt][0] = ya.x; cacc[nt][1] = ya.y; cacc[nt][2] = yb.x; cacc[nt][3] = yb.y;
-          }
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            // A(rr, t) = -L(kb + t, rr) = -S[t ld + rr - kb - t + w], t <= min(b - 1, rr - kb + w)
-            float x[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int rr = (q & 1) ? rb : ra;
-              const int t = 8 * h + tg + ((q & 2) ? 4 : 0);
-              const int off = rr - kb - t + w;
-              x[q] = (rr < kb && t < b && off >= 0) ? -S[t * ld + off] : 0.f;
-            }
-            uint32_t ah[4], al[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) split_tf32(x[q], ah[q], al[q]);
-#pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-              if (PASSES == 3) {
-                mma_tf32(cacc[nt], al, bh[h][nt]);
-                mma_tf32(cacc[nt], ah, bl[h][nt]);
-              }
-              mma_tf32(cacc[nt], ah, bh[h][nt]);
-            }
-          }
-#pragma unroll
-          for (int nt = 0; nt < NT; ++nt) {
-            const int col = 8 * nt + 2 * tg;
-            if (ra < kb) *reinterpret_cast<float2*>(rptr(ra, col)) = make_float2(cacc[nt][0], cacc[nt][1]);
-            if (rb < kb) *reinterpret_cast<float2*>(rptr(rb, col)) = make_float2(cacc[nt][2], cacc[nt][3]);
-          }
-        }
-      }
-#pragma unroll
-      for (int e = 0; e < 2; ++e) {
-        const int idx = tid + e * kThreads, c = idx >> 4, t = idx & 15;
-        if (c < k && t < lo - nlo) *rptr(nlo + t, c) = er[e];
-      }
-      lo = nlo;
-    }
-    __syncthreads();
-  }
-  if (tid == 0 && !ok)
-    for (int v = waited; v < issued; ++v)
-      mbar_wait_bounded(&bars[v % kStages], (uint32_t)((v / kStages) & 1), st, d.id, v);
-}
-
 constexpr int kNB = 32;
 constexpr size_t kSmemCap = 200 * 1024;
 
@@ -1841,7 +950,7 @@ inline int next_pow2(int v) {
 }  // namespace
 
 template <typename T>
-geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w, int max_n,
+geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w, int max_n, int blk_mask,
                           DevStatus* st, cudaStream_t s, bool equil, int32_t* weak, float weak_tol,
                           const Tc5Plan* tc5) {
   if (count <= 0) return GENEO_OK;
@@ -1854,12 +963,7 @@ geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w,
         GENEO_CUDA(cudaGetLastError());
       }
       GENEO_TRY(tc5_factor(*tc5, base, d_desc, st, s, weak, weak_tol * kTf32PivotScale));
-      if (max_n > 0) {
-        const int nb = (max_n + 15) / 16;
-        k_band_dinv<T><<<dim3((nb + 15) / 16, count), 256, 0, s>>>(base, d_desc); note_launch();
-        GENEO_CUDA(cudaGetLastError());
-      }
-      return GENEO_OK;
+      return band_blkinv(base, d_desc, count, max_n, blk_mask, s);
     }
   }
   if (equil && max_n > 0) {
@@ -1876,12 +980,7 @@ geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w,
       k_band_potrf_tc<<<count, kThreads, tc_smem, s>>>(base, d_desc, st, weak, weak_tol * kTf32PivotScale);
       note_launch();
       GENEO_CUDA(cudaGetLastError());
-      if (max_n > 0) {
-        const int nb = (max_n + 15) / 16;
-        k_band_dinv<T><<<dim3((nb + 15) / 16, count), 256, 0, s>>>(base, d_desc); note_launch();
-        GENEO_CUDA(cudaGetLastError());
-      }
-      return GENEO_OK;
+      return band_blkinv(base, d_desc, count, max_n, blk_mask, s);
     }
   }
   // one large matrix (the coarse matrix): spread each panel's update over SMs
@@ -1898,10 +997,7 @@ geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w,
       }
     }
     GENEO_CUDA(cudaGetLastError());
-    const int nb = (max_n + 15) / 16;
-    k_band_dinv<T><<<dim3((nb + 15) / 16, 1), 256, 0, s>>>(base, d_desc); note_launch();
-    GENEO_CUDA(cudaGetLastError());
-    return GENEO_OK;
+    return band_blkinv(base, d_desc, count, max_n, blk_mask, s);
   }
   // the panel starts at a 16-byte boundary (diag block: 32 x 33 values) and
   // its row stride phmax is a multiple of 4
@@ -1917,12 +1013,7 @@ geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w,
     kern<<<count, kThreads, diag, s>>>(base, d_desc, 0, st, weak, weak_tol); note_launch();
   }
   GENEO_CUDA(cudaGetLastError());
-  if (max_n > 0) {
-    const int nb = (max_n + 15) / 16;
-    k_band_dinv<T><<<dim3((nb + 15) / 16, count), 256, 0, s>>>(base, d_desc); note_launch();
-    GENEO_CUDA(cudaGetLastError());
-  }
-  return GENEO_OK;
+  return band_blkinv(base, d_desc, count, max_n, blk_mask, s);
 }
 
 // Shared memory of one solve launch with k right-hand sides.
@@ -1930,15 +1021,6 @@ template <typename T>
 size_t solve_smem(int max_w, int k, int ring, int snb, int stages) {
   const int ld = band_ld(max_w);
   return 128 + sizeof(T) * ((size_t)stages * snb * ld + (size_t)ring * k + (size_t)snb * k + 4 * kThreads);
-}
-
-// Shared memory of the register-tiled multi-right-hand-side solve.
-template <typename T>
-size_t multi_smem(int max_w, int ring, int CT, int stages) {
-  const int ld = band_ld(max_w);
-  const int KP = 2 * CT + 4;
-  return 128 + sizeof(T) * ((size_t)stages * (16 * ld + 256) + (size_t)ring * KP +
-                            (size_t)(kThreads / 32 + 1) * 16 * KP);
 }
 
 // Column split of a multi-right-hand-side launch: when a batch holds at most
@@ -1962,89 +1044,6 @@ inline int split_parts(int count, int units) {
   return std::max(1, std::min(units, sms / count));
 }
 
-template <typename T, typename A, int CT, int kStages>
-geneo_status_t launch_multi_t(dim3 grid, size_t smem, cudaStream_t s, const T* base, const BandDesc* d_desc,
-                              double* xbase, const int64_t* xoff, int c0, int kc,
-                              const int32_t* nrhs_dev, const int32_t* skip_dev, int ring, DevStatus* st) {
-  auto kern = k_band_solve_multi<T, A, CT, kStages>;
-  GENEO_CUDA(allow_smem(kern));
-  kern<<<grid, kThreads, smem, s>>>(base, d_desc, xbase, xoff, c0, kc, nrhs_dev, skip_dev, ring, st);
-  note_launch();
-  GENEO_CUDA(cudaGetLastError());
-  return GENEO_OK;
-}
-
-template <typename T, typename A = T>
-geneo_status_t launch_multi(int CT, int stages, dim3 grid, size_t smem, cudaStream_t s, const T* base,
-                            const BandDesc* d_desc, double* xbase, const int64_t* xoff, int c0, int kc,
-                            const int32_t* nrhs_dev, const int32_t* skip_dev, int ring, DevStatus* st) {
-#define GENEO_MULTI(ct, sg)                                                                       \
-  if (CT == ct && stages == sg)                                                                  \
-    return launch_multi_t<T, A, ct, sg>(grid, smem, s, base, d_desc, xbase, xoff, c0, kc, nrhs_dev, \
-                                     skip_dev, ring, st);
-  GENEO_MULTI(4, 2) GENEO_MULTI(4, 4) GENEO_MULTI(8, 2) GENEO_MULTI(8, 4)
-  if constexpr (sizeof(T) == 4) {
-    GENEO_MULTI(12, 2) GENEO_MULTI(12, 4) GENEO_MULTI(16, 2) GENEO_MULTI(16, 4)
-  }
-#undef GENEO_MULTI
-  return GENEO_ERR_ARG;
-}
-
-// Shared memory of the tensor-core multi-right-hand-side solve (ring and
-// partial-sum strides as in MtcRP / MtcKP).
-inline size_t mtc_smem(int max_w, int ring, int NT, int stages) {
-  const int ld = band_ld(max_w);
-  const int KP = NT == 1 ? 8 : (NT == 4 ? 40 : 24);
-  const int RP = NT == 2 ? 16 : KP;
-  return 128 + sizeof(float) * ((size_t)stages * (16 * ld + 256) + (size_t)ring * RP +
-                                (size_t)(kThreads / 32 + 1) * 16 * KP);
-}
-// Shared memory per block that still lets two blocks share an SM.
-constexpr size_t kTwoPerSm = 112 * 1024;
-
-template <int NT, int kStages, int PASSES>
-geneo_status_t launch_mtc_t(dim3 grid, size_t smem, cudaStream_t s, const float* base, const BandDesc* d_desc,
-                            double* xbase, const int64_t* xoff, int c0, int kc,
-                            const int32_t* nrhs_dev, const int32_t* skip_dev, int ring, DevStatus* st) {
-  auto kern = k_band_solve_mtc<NT, kStages, PASSES>;
-  GENEO_CUDA(allow_smem(kern));
-  kern<<<grid, kThreads, smem, s>>>(base, d_desc, xbase, xoff, c0, kc, nrhs_dev, skip_dev, ring, st);
-  note_launch();
-  GENEO_CUDA(cudaGetLastError());
-  return GENEO_OK;
-}
-
-geneo_status_t launch_mtc(int NT, int stages, int passes, dim3 grid, size_t smem, cudaStream_t s,
-                          const float* base, const BandDesc* d_desc, double* xbase, const int64_t* xoff,
-                          int c0, int kc, const int32_t* nrhs_dev, const int32_t* skip_dev, int ring,
-                          DevStatus* st) {
-#define GENEO_MTC(nt, sg)                                                                              \
-  if (NT == nt && stages == sg)                                                                        \
-    return passes == 1 ? launch_mtc_t<nt, sg, 1>(grid, smem, s, base, d_desc, xbase, xoff, c0, kc,    \
-                                                 nrhs_dev, skip_dev, ring, st)                         \
-                       : launch_mtc_t<nt, sg, 3>(grid, smem, s, base, d_desc, xbase, xoff, c0, kc,    \
-                                                 nrhs_dev, skip_dev, ring, st);
-  GENEO_MTC(1, 2) GENEO_MTC(1, 3) GENEO_MTC(1, 4) GENEO_MTC(2, 2) GENEO_MTC(2, 3) GENEO_MTC(2, 4)
-  GENEO_MTC(3, 2) GENEO_MTC(3, 3) GENEO_MTC(3, 4) GENEO_MTC(4, 2) GENEO_MTC(4, 3) GENEO_MTC(4, 4)
-#undef GENEO_MTC
-  return GENEO_ERR_ARG;
-}
-
-// Shared memory of the resident-vector one-right-hand-side solve.
-template <typename T>
-size_t res_smem(int max_w, int max_n, int snb, int stages) {
-  const int ld = band_ld(max_w);
-  return 128 + sizeof(T) * ((size_t)stages * (snb * ld + 256) + (size_t)((max_n + 3) & ~3) + snb);
-}
-
-// Shared memory of the ring one-right-hand-side solve: barriers, hs half
-// blocks of 8 rows with a diagonal block each, the ring, three 16-vectors.
-template <typename T>
-size_t ring_smem(int max_w, int ring, int hs) {
-  const int ld = band_ld(max_w);
-  return 256 + sizeof(T) * ((size_t)hs * (8 * (size_t)ld + 256) + (size_t)ring + 48);
-}
-
 // Solves with the kernels that do not apply a band's row scaling (the
 // caller scales the vectors around them).
 template <typename T, typename A = T>
@@ -2063,31 +1062,6 @@ geneo_status_t band_solve_plain(const T* base, const BandDesc* d_desc, int count
     kern<<<count, kThreads, smem, s>>>(base, d_desc, xbase, xoff, 0, 1, nrhs_dev, skip_dev, ring, st); note_launch();
     GENEO_CUDA(cudaGetLastError());
     return GENEO_OK;
-  }
-  // register-tiled kernel: up to 32 (FP32) or 16 (FP64) columns per launch
-  {
-    const int ring = next_pow2(max_w + 32);
-    const int kmax = std::min(nrhs, sizeof(T) == 4 ? 32 : 16);
-    const int CT0 = (((kmax + 1) / 2) + 3) & ~3;
-    if (multi_smem<T>(max_w, ring, CT0, 2) <= 227 * 1024) {
-      for (int c0 = 0; c0 < nrhs; c0 += kmax) {
-        const int kc = std::min(kmax, nrhs - c0);
-        int CT = (((kc + 1) / 2) + 3) & ~3;
-        // parts of 8 k columns (CT a multiple of 4)
-        const int units = (kc + 7) / 8, parts = split_parts(live, units);
-        int nsplit = 1;
-        if (parts > 1) {
-          CT = 4 * ((units + parts - 1) / parts);
-          nsplit = (kc + 2 * CT - 1) / (2 * CT);
-        }
-        const int stages = multi_smem<T>(max_w, ring, CT, 4) <= 227 * 1024 ? 4 : 2;
-        const geneo_status_t rc = launch_multi<T, A>(CT, stages, dim3(count, nsplit),
-                                                      multi_smem<T>(max_w, ring, CT, stages), s, base, d_desc,
-                                                      xbase, xoff, c0, kc, nrhs_dev, skip_dev, ring, st);
-        if (rc != GENEO_OK) return rc;
-      }
-      return GENEO_OK;
-    }
   }
   constexpr int stg = Stages<T>::v;
   int snb = 16;
@@ -2113,98 +1087,20 @@ geneo_status_t band_solve_plain(const T* base, const BandDesc* d_desc, int count
   return GENEO_OK;
 }
 
-template <typename T, typename A>
-geneo_status_t band_solve_impl(const T* base, const BandDesc* d_desc, int count, int max_w,
+template <typename T, bool DS>
+geneo_status_t band_solve_impl(const T* base, const BandDesc* d_desc, int count, int blk, int max_w,
                                double* xbase, const int64_t* xoff, int nrhs, const int32_t* nrhs_dev,
                                const int32_t* skip_dev, DevStatus* st, cudaStream_t s, int max_n, int tc_passes,
-                               int res_stages, int active) {
+                               int slots, int active) {
   if (count <= 0 || nrhs <= 0) return GENEO_OK;
-  // double-single arithmetic covers the multi-column solves; one right-hand
-  // side keeps the FP64 kernels
-  if constexpr (!std::is_same_v<A, T>) {
-    if (nrhs == 1)
-      return band_solve_impl<T, T>(base, d_desc, count, max_w, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, s, max_n,
-                                   tc_passes, res_stages, active);
-  }
-  // matrices to solve (the others are skipped by their blocks at once): the
-  // column split and the pipeline depth follow this number
-  const int live = active > 0 ? std::min(active, count) : count;
-  // One right-hand side (the preconditioner's local solves): two stages and
-  // one register slot per warp keep the block small enough for several
-  // blocks per SM, which hides the latency of the sequential sweep.
-  if (nrhs == 1) {
-    // whole vector resident in shared memory when it fits; the deepest
-    // pipeline (at most four stages) that keeps two blocks per SM for FP32
-    // batches (one for FP64 or a small batch) hides the latency of the
-    // factor stream
-    if (max_n > 0) {
-      const size_t budget = (sizeof(T) == 4 && count > 152) ? 112 * 1024 : 226 * 1024;
-      int stages = 4;
-      while (stages > 2 && res_smem<T>(max_w, max_n, 16, stages) > budget) --stages;
-      // a depth chosen by the autotuner (solve.cu) when it fits
-      if (res_stages >= 2 && res_stages <= 4 && res_smem<T>(max_w, max_n, 16, res_stages) <= 227 * 1024)
-        stages = res_stages;
-      const size_t smem = res_smem<T>(max_w, max_n, 16, stages);
-      if (smem <= 227 * 1024) {
-        auto kern = stages == 4 ? k_band_solve_res<T, 4>
-                  : stages == 3 ? k_band_solve_res<T, 3> : k_band_solve_res<T, 2>;
-        GENEO_CUDA(allow_smem(kern));
-        kern<<<count, kThreads, smem, s>>>(base, d_desc, xbase, xoff, nrhs_dev, skip_dev, st); note_launch();
-        GENEO_CUDA(cudaGetLastError());
-        return GENEO_OK;
-      }
-    }
-    // the vector does not fit: a window of it in a ring, the band in
-    // half-block stages, as many as fit
-    const int ring = next_pow2(max_w + 32);
-    int hs = 6;
-    while (hs > 2 && ring_smem<T>(max_w, ring, hs) > 227 * 1024) hs = hs == 6 ? 4 : hs - 1;
-    const size_t smem = ring_smem<T>(max_w, ring, hs);
-    if (smem <= 227 * 1024) {
-      auto kern = hs == 6 ? k_band_solve_ring<T, 6>
-                : hs == 4 ? k_band_solve_ring<T, 4>
-                : hs == 3 ? k_band_solve_ring<T, 3> : k_band_solve_ring<T, 2>;
-      GENEO_CUDA(allow_smem(kern));
-      kern<<<count, kThreads + 32, smem, s>>>(base, d_desc, xbase, xoff, nrhs_dev, skip_dev, ring, st);
-      note_launch();
-      GENEO_CUDA(cudaGetLastError());
-      return GENEO_OK;
-    }
-  }
-  // FP32 factors: tensor-core kernel, up to 32 columns per launch
-  if constexpr (sizeof(T) == 4) {
-    const int ring = next_pow2(max_w + 32);
-    if (mtc_smem(max_w, ring, 1, 2) <= 227 * 1024) {
-      for (int c0 = 0; c0 < nrhs; c0 += 32) {
-        const int kc = std::min(32, nrhs - c0);
-        int NT = (kc + 7) / 8;
-        while (NT > 1 && mtc_smem(max_w, ring, NT, 2) > 227 * 1024) --NT;
-        const int kk = std::min(kc, 8 * NT);
-        // column parts of 8 NT columns for small batches
-        int nsplit = 1;
-        {
-          const int parts = split_parts(live, NT);
-          if (parts > 1) {
-            NT = (NT + parts - 1) / parts;
-            nsplit = (kk + 8 * NT - 1) / (8 * NT);
-          }
-        }
-        // the deepest pipeline that keeps two blocks per SM when the batch
-        // fills more than one wave of single blocks (NT <= 2), else the
-        // deepest that fits
-        int stages = 4;
-        const size_t cap = (NT <= 2 && live > 152 && mtc_smem(max_w, ring, NT, 2) <= kTwoPerSm) ? kTwoPerSm
-                                                                                                : 227 * 1024;
-        while (stages > 2 && mtc_smem(max_w, ring, NT, stages) > cap) --stages;
-        GENEO_TRY(launch_mtc(NT, stages, tc_passes, dim3(count, nsplit), mtc_smem(max_w, ring, NT, stages), s,
-                             base, d_desc, xbase, xoff, c0, kk, nrhs_dev, skip_dev, ring, st));
-        if (kk < kc) c0 -= kc - kk;  // the rest of this chunk goes in the next launch
-      }
-      return GENEO_OK;
-    }
-  }
-  // other kernels: the vectors are scaled around the solve where the bands
-  // are equilibrated (FP32 factors)
+  // matrices to solve side by side (this batch's, or those of all classes)
+  const int live = active > 0 ? active : count;
+  if (blk > 0)
+    return sweep_solve<T, DS>(base, d_desc, count, blk, max_w, max_n, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, s,
+                              tc_passes, slots, live);
+  // bands too wide for the sweeps: the streamed kernel on the factor itself,
+  // the vectors scaled around the solve where the bands are equilibrated
+  // (FP32 factors); double-single covers several right-hand sides
   if constexpr (sizeof(T) == 4) {
     const int gx = std::max(1, std::min(64, (max_n > 0 ? max_n : 4096) * nrhs / 256));
     k_band_scale_x<T><<<dim3(gx, count), 256, 0, s>>>(base, d_desc, xbase, xoff, 0, nrhs, nrhs_dev, skip_dev);
@@ -2214,35 +1110,37 @@ geneo_status_t band_solve_impl(const T* base, const BandDesc* d_desc, int count,
     note_launch();
     GENEO_CUDA(cudaGetLastError());
     return GENEO_OK;
+  } else if (DS && nrhs > 1) {
+    return band_solve_plain<T, dsv>(base, d_desc, count, max_w, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, s, live);
   } else {
-    return band_solve_plain<T, A>(base, d_desc, count, max_w, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, s, live);
+    return band_solve_plain<T>(base, d_desc, count, max_w, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, s, live);
   }
 }
 
 template <typename T>
-geneo_status_t band_solve(const T* base, const BandDesc* d_desc, int count, int max_w,
+geneo_status_t band_solve(const T* base, const BandDesc* d_desc, int count, int blk, int max_w,
                           double* xbase, const int64_t* xoff, int nrhs, const int32_t* nrhs_dev,
                           const int32_t* skip_dev, DevStatus* st, cudaStream_t s, int max_n, int tc_passes,
-                          int res_stages, int active) {
-  return band_solve_impl<T, T>(base, d_desc, count, max_w, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, s, max_n,
-                               tc_passes, res_stages, active);
+                          int slots, int active) {
+  return band_solve_impl<T, false>(base, d_desc, count, blk, max_w, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, s,
+                                   max_n, tc_passes, slots, active);
 }
 
-geneo_status_t band_solve_ds(const double* base, const BandDesc* d_desc, int count, int max_w, double* xbase,
-                             const int64_t* xoff, int nrhs, const int32_t* nrhs_dev, const int32_t* skip_dev,
-                             DevStatus* st, cudaStream_t s, int max_n, int active) {
-  return band_solve_impl<double, dsv>(base, d_desc, count, max_w, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, s,
-                                      max_n, 3, 0, active);
+geneo_status_t band_solve_ds(const double* base, const BandDesc* d_desc, int count, int blk, int max_w,
+                             double* xbase, const int64_t* xoff, int nrhs, const int32_t* nrhs_dev,
+                             const int32_t* skip_dev, DevStatus* st, cudaStream_t s, int max_n, int active) {
+  return band_solve_impl<double, true>(base, d_desc, count, blk, max_w, xbase, xoff, nrhs, nrhs_dev, skip_dev, st,
+                                       s, max_n, 3, 0, active);
 }
 
-template geneo_status_t band_potrf<double>(double*, const BandDesc*, int, int, int, DevStatus*,
+template geneo_status_t band_potrf<double>(double*, const BandDesc*, int, int, int, int, DevStatus*,
                                            cudaStream_t, bool, int32_t*, float, const Tc5Plan*);
-template geneo_status_t band_potrf<float>(float*, const BandDesc*, int, int, int, DevStatus*,
+template geneo_status_t band_potrf<float>(float*, const BandDesc*, int, int, int, int, DevStatus*,
                                           cudaStream_t, bool, int32_t*, float, const Tc5Plan*);
-template geneo_status_t band_solve<double>(const double*, const BandDesc*, int, int, double*,
+template geneo_status_t band_solve<double>(const double*, const BandDesc*, int, int, int, double*,
                                            const int64_t*, int, const int32_t*, const int32_t*,
                                            DevStatus*, cudaStream_t, int, int, int, int);
-template geneo_status_t band_solve<float>(const float*, const BandDesc*, int, int, double*,
+template geneo_status_t band_solve<float>(const float*, const BandDesc*, int, int, int, double*,
                                           const int64_t*, int, const int32_t*, const int32_t*,
                                           DevStatus*, cudaStream_t, int, int, int, int);
 

@@ -252,7 +252,9 @@ geneo_status_t build_coarse(geneo_handle_s* h, const AssemblyOut& asmb, const do
     }
   }
   h->wH = wH;
-  GENEO_TRY(h->mem.get(&h->bandH, (size_t)h->dimH * band_ld(wH) + dinv_elems(h->dimH)));
+  wH = band_w(wH);  // as stored
+  const int blkH = sweep_block(wH, true);
+  GENEO_TRY(h->mem.get(&h->bandH, (size_t)h->dimH * band_ld(wH)));
   GENEO_CUDA(cudaMemsetAsync(h->bandH, 0, sizeof(double) * h->dimH * band_ld(wH), s));
   int2* dpairs = nullptr;
   GENEO_TRY(tmp.get(&dpairs, pairs.size()));
@@ -264,12 +266,12 @@ geneo_status_t build_coarse(geneo_handle_s* h, const AssemblyOut& asmb, const do
   *ms_matrix = ms_since(t1);
 
   auto t2 = std::chrono::steady_clock::now();
-  BandDesc bh{0, h->dimH, wH, -2, band_ld(wH), (int64_t)h->dimH * band_ld(wH), -1};
+  BandDesc bh{0, h->dimH, wH, -2, band_ld(wH), blkH, -1};
   GENEO_TRY(h->mem.get(&h->dbandH, 1));
   GENEO_CUDA(cudaMemcpyAsync(h->dbandH, &bh, sizeof(BandDesc), cudaMemcpyHostToDevice, s));
   const int pf = h->prof.begin(GENEO_PROF_FACTOR, band_factor_flops(h->dimH, wH),
                                2.0 * 8.0 * band_entries(h->dimH, wH), s);
-  GENEO_TRY(band_potrf<double>(h->bandH, h->dbandH, 1, wH, h->dimH, h->dstat, s));
+  GENEO_TRY(band_potrf<double>(h->bandH, h->dbandH, 1, wH, h->dimH, blkH, h->dstat, s));
   h->prof.end(pf, s);
   GENEO_TRY(check_status(h, s));
   // The preconditioner's coarse solve A_H y = c runs on one small band, a
@@ -305,9 +307,9 @@ geneo_status_t build_coarse(geneo_handle_s* h, const AssemblyOut& asmb, const do
     // FP32 pipe (about 46 bits; GB300 issues FP64 at 1/64 of the FP32 rate),
     // an error far below the FP32 local solves' beside it in M^{-1}
     if (h->fp32)
-      GENEO_TRY(band_solve_ds(h->bandH, drep, nc, wH, h->Hinv, dxo, 16, dcnt, nullptr, h->dstat, s, 0));
+      GENEO_TRY(band_solve_ds(h->bandH, drep, nc, blkH, wH, h->Hinv, dxo, 16, dcnt, nullptr, h->dstat, s, dim));
     else
-      GENEO_TRY(band_solve<double>(h->bandH, drep, nc, wH, h->Hinv, dxo, 16, dcnt, nullptr, h->dstat, s, 0));
+      GENEO_TRY(band_solve<double>(h->bandH, drep, nc, blkH, wH, h->Hinv, dxo, 16, dcnt, nullptr, h->dstat, s, dim));
     GENEO_TRY(check_status(h, s));
   }
   *ms_factor = ms_since(t2);

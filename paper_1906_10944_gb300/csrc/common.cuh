@@ -143,10 +143,10 @@ struct SubDesc {
 // base[r * ld + (c - r + w)]; ld = w + 1 rounded up to a multiple of 4, so
 // every row (and every block of rows) starts on a 16-byte boundary (32 for
 // FP64) and can be moved by one bulk copy.  Slots with c < 0 are zero.
-// Beside the band, the factorisation stores the inverses of the 16 x 16
-// diagonal blocks of L (block b: rows and columns 16 b .. 16 b + 15; entry
-// (i, t) at dinv + 256 b + 16 i + t, zero outside the lower triangle and
-// beyond n), which the solves apply instead of substituting.
+// After the factorisation the blk x blk diagonal blocks of L (blk rows and
+// columns from every multiple of blk) hold their inverses, in place, which the
+// sweeps apply instead of substituting; blk = 0: L everywhere (a band too wide
+// for the sweeps of sweep.cu).
 struct BandDesc {
   int64_t off;     // element offset of the band (a multiple of 4)
   int32_t n, w;
@@ -154,14 +154,15 @@ struct BandDesc {
                    // skip flags by id when it is >= 0 (subdomain index), by
                    // the position in the batch otherwise
   int32_t ld;      // row stride
-  int64_t dinv;    // element offset of the inverted diagonal blocks
+  int32_t blk;     // rows per sweep block (sweep_block), 0: none
   int64_t scl;     // element offset of the row scaling s = diag^{-1/2} of an
                    // equilibrated band (the factor is that of S A S), or -1
 };
 
 __host__ __device__ __forceinline__ int band_ld(int w) { return (w + 4) & ~3; }
-// elements of the inverted diagonal blocks of an order-n band
-__host__ __device__ __forceinline__ int64_t dinv_elems(int n) { return (int64_t)((n + 15) / 16) * 256; }
+// half width a band is stored with: at least 15, so that the smallest sweep
+// block's triangle lies in it (entries beyond the matrix's own width are 0)
+__host__ __device__ __forceinline__ int band_w(int w) { return w < 15 ? 15 : w; }
 // elements of the row scaling of an order-n band (a multiple of 4)
 __host__ __device__ __forceinline__ int64_t scl_elems(int n) { return (int64_t)((n + 3) & ~3); }
 
@@ -330,8 +331,26 @@ bool tc5_fits(int w);
 geneo_status_t tc5_factor(const Tc5Plan& p, float* band, const BandDesc* d_desc, DevStatus* st, cudaStream_t s,
                           int32_t* weak, float weak_tol);
 
+// sweep.cu
+// Rows per block of the sweeps for a band of half width w >= 15 (stored as
+// FP64 or FP32); 0: too wide for them.
+int sweep_block(int w, bool f64);
+// the inverses of the diagonal blocks, in place, of every matrix whose blk is
+// in blk_mask (an OR of block sizes, which are powers of two)
+template <typename T>
+geneo_status_t band_blkinv(T* base, const BandDesc* d_desc, int count, int max_n, int blk_mask, cudaStream_t s);
+// band_solve (below) for a batch whose matrices all have the block size blk
+// > 0; DS: FP64 factors in double-single arithmetic; live: matrices that
+// skip_dev leaves.
+template <typename T, bool DS>
+geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int blk, int max_w, int max_n,
+                           double* xbase, const int64_t* xoff, int nrhs, const int32_t* nrhs_dev,
+                           const int32_t* skip_dev, DevStatus* st, cudaStream_t s, int tc_passes, int slots,
+                           int live);
+
 // band.cu
-// Batched Cholesky.  equil: factor S A S (s = diag^{-1/2}) and keep s.
+// Batched Cholesky.  blk_mask: the block sizes of the batch, whose diagonal
+// blocks are inverted in place at the end.  equil: factor S A S (s = diag^{-1/2}) and keep s.
 // weak (may be NULL): instead of reporting GENEO_ERR_NOT_SPD, matrix d sets
 // weak[d.id] = 1 when one of its pivots is not above weak_tol (relative to
 // the unit diagonal of an equilibrated band); the caller factors those
@@ -339,7 +358,7 @@ geneo_status_t tc5_factor(const Tc5Plan& p, float* band, const BandDesc* d_desc,
 // tc5 (FP32, may be NULL): a prepared plan sends the factorisation to the
 // fifth-generation tensor-core kernel.
 template <typename T>
-geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w, int max_n,
+geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w, int max_n, int blk_mask,
                           DevStatus* st, cudaStream_t s, bool equil = false,
                           int32_t* weak = nullptr, float weak_tol = 0.f, const Tc5Plan* tc5 = nullptr);
 // Solve L L^T X = X in place for `nrhs` columns per matrix (column-major,
@@ -348,25 +367,25 @@ geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w,
 // xbase + xoff[i]; nrhs_dev (may be NULL) gives per-matrix column counts
 // capped by nrhs; skip_dev (may be NULL) skips matrices with a non-zero flag;
 // a descriptor with n = 0 is skipped.
-// max_n (largest matrix order, 0 if unknown) enables the one-right-hand-side
-// solve with the vector resident in shared memory.  tc_passes (FP32 factors,
+// blk: the block size of every matrix of the batch (0: the streamed kernels).
+// max_n: largest matrix order (0 if unknown).  tc_passes (FP32 factors,
 // several right-hand sides): 3 = each tensor-core product as three TF32
-// passes (about FP32 accuracy), 1 = one TF32 pass.  res_stages (one
-// right-hand side with the vector resident, 2-4; 0 = by shared memory): the
-// pipeline depth of that kernel, as an autotuner picked it.  active (0 =
-// count): how many of the matrices skip_dev leaves to solve, which sizes the
-// column split of the multi-column kernels.
+// passes (about FP32 accuracy), 1 = one TF32 pass.  slots (one right-hand
+// side, 2-4; 0 = as many as fit): row slots of the factor stream, as an
+// autotuner picked them.  active (0 = count): how many matrices are solved at
+// the same time (those skip_dev leaves, of this batch and of others running
+// beside it), which sizes the clusters and the column split.
 template <typename T>
-geneo_status_t band_solve(const T* base, const BandDesc* d_desc, int count, int max_w,
+geneo_status_t band_solve(const T* base, const BandDesc* d_desc, int count, int blk, int max_w,
                           double* xbase, const int64_t* xoff, int nrhs, const int32_t* nrhs_dev,
                           const int32_t* skip_dev, DevStatus* st, cudaStream_t s, int max_n = 0,
-                          int tc_passes = 3, int res_stages = 0, int active = 0);
+                          int tc_passes = 3, int slots = 0, int active = 0);
 
 // FP64 factors solved in double-single arithmetic on the FP32 pipe (about
 // 46 significant bits) for several right-hand sides: the FP64 fallback
 // factors of the FP32 mode, where FP64's 1/64 rate on GB300 bounds the
 // sweeps; one right-hand side is solved in FP64.
-geneo_status_t band_solve_ds(const double* base, const BandDesc* d_desc, int count, int max_w, double* xbase,
+geneo_status_t band_solve_ds(const double* base, const BandDesc* d_desc, int count, int blk, int max_w, double* xbase,
                              const int64_t* xoff, int nrhs, const int32_t* nrhs_dev, const int32_t* skip_dev,
                              DevStatus* st, cudaStream_t s, int max_n, int active = 0);
 
@@ -380,7 +399,7 @@ struct SolveClass {
   bool f64 = false;
   bool ds = false;             // FP64 factors, several right-hand sides in double-single
   BandDesc* d = nullptr;       // the class's descriptors (device), largest sweep first
-  int count = 0, max_w = 0, max_n = 0;
+  int count = 0, blk = 0, max_w = 0, max_n = 0;
   double cost = 0.0;           // bytes of one forward and backward sweep over the class
   int lane = 0;
 };
@@ -408,6 +427,6 @@ geneo_status_t make_solve_set(const void* base, bool f64, const BandDesc* d_desc
 // to solve.
 geneo_status_t solve_set_run(const SolveSet& ss, const SolveStreams& pool, double* xbase, const int64_t* xoff,
                              int nrhs, const int32_t* nrhs_dev, const int32_t* skip_dev, DevStatus* st,
-                             cudaStream_t s, int tc_passes = 3, int res_stages = 0, int active = 0);
+                             cudaStream_t s, int tc_passes = 3, int slots = 0, int active = 0);
 
 }  // namespace geneo

@@ -43,11 +43,13 @@ geneo_status_t add_part(const void* base, bool f64, bool ds, const BandDesc* d_d
   });
   const double esz = f64 ? 8.0 : 4.0;
   std::vector<std::vector<BandDesc>> groups;
-  int top = -1;
+  int top = -1, blk = -1;
   for (const BandDesc& b : live) {
-    if (groups.empty() || ((double)b.w < kClassRatio * top && (int)groups.size() < kMaxClassesPerPart)) {
+    if (groups.empty() || b.blk != blk ||
+        ((double)b.w < kClassRatio * top && (int)groups.size() < kMaxClassesPerPart)) {
       groups.emplace_back();
       top = b.w;
+      blk = b.blk;
     }
     groups.back().push_back(b);
   }
@@ -60,6 +62,7 @@ geneo_status_t add_part(const void* base, bool f64, bool ds, const BandDesc* d_d
     c.f64 = f64;
     c.ds = ds;
     c.count = (int)g.size();
+    c.blk = g.front().blk;
     for (const BandDesc& b : g) {
       c.max_w = std::max(c.max_w, b.w);
       c.max_n = std::max(c.max_n, b.n);
@@ -74,16 +77,15 @@ geneo_status_t add_part(const void* base, bool f64, bool ds, const BandDesc* d_d
 
 geneo_status_t run_class(const SolveClass& c, double* xbase, const int64_t* xoff, int nrhs,
                          const int32_t* nrhs_dev, const int32_t* skip_dev, DevStatus* st, cudaStream_t s,
-                         int tc_passes, int res_stages, int active) {
-  const int act = active > 0 ? std::min(active, c.count) : 0;
+                         int tc_passes, int slots, int active) {
   if (c.ds && nrhs > 1)
-    return band_solve_ds(static_cast<const double*>(c.base), c.d, c.count, c.max_w, xbase, xoff, nrhs, nrhs_dev,
-                         skip_dev, st, s, c.max_n, act);
+    return band_solve_ds(static_cast<const double*>(c.base), c.d, c.count, c.blk, c.max_w, xbase, xoff, nrhs, nrhs_dev,
+                         skip_dev, st, s, c.max_n, active);
   if (c.f64)
-    return band_solve<double>(static_cast<const double*>(c.base), c.d, c.count, c.max_w, xbase, xoff, nrhs,
-                              nrhs_dev, skip_dev, st, s, c.max_n, tc_passes, res_stages, act);
-  return band_solve<float>(static_cast<const float*>(c.base), c.d, c.count, c.max_w, xbase, xoff, nrhs,
-                           nrhs_dev, skip_dev, st, s, c.max_n, tc_passes, res_stages, act);
+    return band_solve<double>(static_cast<const double*>(c.base), c.d, c.count, c.blk, c.max_w, xbase, xoff, nrhs,
+                              nrhs_dev, skip_dev, st, s, c.max_n, tc_passes, slots, active);
+  return band_solve<float>(static_cast<const float*>(c.base), c.d, c.count, c.blk, c.max_w, xbase, xoff, nrhs,
+                           nrhs_dev, skip_dev, st, s, c.max_n, tc_passes, slots, active);
 }
 
 }  // namespace
@@ -116,16 +118,20 @@ geneo_status_t make_solve_set(const void* base, bool f64, const BandDesc* d_desc
 
 geneo_status_t solve_set_run(const SolveSet& ss, const SolveStreams& pool, double* xbase, const int64_t* xoff,
                              int nrhs, const int32_t* nrhs_dev, const int32_t* skip_dev, DevStatus* st,
-                             cudaStream_t s, int tc_passes, int res_stages, int active) {
+                             cudaStream_t s, int tc_passes, int slots, int active) {
   if (ss.cls.empty() || nrhs <= 0) return GENEO_OK;
   if (ss.lanes > 1) {
     GENEO_CUDA(cudaEventRecord(pool.fork, s));
     for (int l = 1; l < ss.lanes; ++l) GENEO_CUDA(cudaStreamWaitEvent(pool.s[l - 1], pool.fork, 0));
   }
+  // the classes run side by side: each sizes its clusters for all of them
+  int live = 0;
+  for (const SolveClass& c : ss.cls) live += c.count;
+  if (active > 0) live = std::min(live, active);
   geneo_status_t rc = GENEO_OK;
   for (const SolveClass& c : ss.cls) {
     const cudaStream_t cs = c.lane == 0 ? s : pool.s[c.lane - 1];
-    rc = run_class(c, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, cs, tc_passes, res_stages, active);
+    rc = run_class(c, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, cs, tc_passes, slots, live);
     if (rc != GENEO_OK) break;
   }
   // join every lane, also after a failed launch, so that no work is left
