@@ -12,6 +12,7 @@
 // All inner products are fixed-order two-stage reductions.
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "handle.cuh"
@@ -20,110 +21,129 @@ namespace geneo {
 namespace {
 
 constexpr int kT = 256;
-constexpr int kNb = 512;   // blocks of the vector kernels (partials per column)
+constexpr int kNb = 608;   // blocks of the vector kernels (partials per column): four per SM
 constexpr int kSl = 16;    // scalar slots per column
 // slots: 0 rz, 1 alpha, 2 beta, 3 rr, 4 pq, 5 bb, 6 flag, 7 true rr,
 //        8 active (1.0 / 0.0), 9 restart (1.0: beta = 0 at the next update)
 
-// Q = A P for k columns (SELL-32, thread per row, a slice per warp):
+// Kernels take the number of columns K as a template argument where they keep
+// one accumulator per column: a runtime count kept every loop over columns
+// (and the gathers in it) rolled and the loads one at a time.
+
+// y(0 .. K - 1) = row l of slice sl of A times the K columns of X; U entries of
+// the row in flight at once
+template <int K>
+__device__ __forceinline__ void sell_row_cols(const int64_t* __restrict__ off, const int32_t* __restrict__ scol,
+                                              const double* __restrict__ sval, const double* __restrict__ X, int64_t n,
+                                              int64_t sl, int l, double* acc) {
+  constexpr int U = K <= 2 ? 4 : K <= 4 ? 3 : 2;
+  const int64_t o = off[sl] + l;
+  const int w = (int)((off[sl + 1] - off[sl]) >> 5);
+#pragma unroll
+  for (int c = 0; c < K; ++c) acc[c] = 0.0;
+  int t = 0;
+  for (; t + U <= w; t += U) {
+    double v[U], x[U][K];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t e = o + 32 * (int64_t)(t + u);
+      v[u] = sval[e];
+      const double* xc = X + scol[e];
+#pragma unroll
+      for (int c = 0; c < K; ++c) x[u][c] = xc[c * n];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int c = 0; c < K; ++c) acc[c] += v[u] * x[u][c];
+  }
+  for (; t < w; ++t) {
+    const int64_t e = o + 32 * (int64_t)t;
+    const double v = sval[e];
+    const double* xc = X + scol[e];
+#pragma unroll
+    for (int c = 0; c < K; ++c) acc[c] += v * xc[c * n];
+  }
+}
+
+// Q = A P for K columns (SELL-32, thread per row, a slice per warp):
 // partial p_c.q_c per block
+template <int K>
 __global__ void __launch_bounds__(kT)
 k_spmm_sell_cols(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ scol,
-                 const double* __restrict__ sval, const double* __restrict__ P, double* __restrict__ Q, int k,
+                 const double* __restrict__ sval, const double* __restrict__ P, double* __restrict__ Q,
                  double* __restrict__ part) {
   __shared__ double red[kT / 32];
   const int l = threadIdx.x & 31;
   const int64_t nsl = (n + 31) / 32;
-  double dsum[kBlk];
+  double dsum[K];
 #pragma unroll
-  for (int c = 0; c < kBlk; ++c) dsum[c] = 0.0;
+  for (int c = 0; c < K; ++c) dsum[c] = 0.0;
   for (int64_t sl = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; sl < nsl;
        sl += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int64_t o = off[sl] + l;
-    const int w = (int)((off[sl + 1] - off[sl]) >> 5);
-    double acc[kBlk];
-#pragma unroll
-    for (int c = 0; c < kBlk; ++c) acc[c] = 0.0;
-    for (int t = 0; t < w; ++t) {
-      const int64_t e = o + 32 * (int64_t)t;
-      const double v = sval[e];
-      const int64_t cc = scol[e];
-#pragma unroll
-      for (int c = 0; c < kBlk; ++c)
-        if (c < k) acc[c] += v * P[c * n + cc];
-    }
+    double acc[K];
+    sell_row_cols<K>(off, scol, sval, P, n, sl, l, acc);
     const int64_t r = sl * 32 + l;
     if (r < n) {
 #pragma unroll
-      for (int c = 0; c < kBlk; ++c)
-        if (c < k) {
-          Q[c * n + r] = acc[c];
-          dsum[c] += acc[c] * P[c * n + r];
-        }
+      for (int c = 0; c < K; ++c) {
+        Q[c * n + r] = acc[c];
+        dsum[c] += acc[c] * P[c * n + r];
+      }
     }
   }
-  for (int c = 0; c < k; ++c) {
+#pragma unroll
+  for (int c = 0; c < K; ++c) {
     const double sc = block_sum(dsum[c], red);
     if (threadIdx.x == 0) part[(int64_t)c * kNb + blockIdx.x] = sc;
   }
 }
 
-// R_c = B_c - A X_c for k columns; partial r_c.r_c per block
+// R_c = B_c - A X_c for K columns; partial r_c.r_c per block
+template <int K>
 __global__ void __launch_bounds__(kT)
 k_resid_sell_cols(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ scol,
                   const double* __restrict__ sval, const double* __restrict__ X, const double* __restrict__ B,
-                  double* __restrict__ Rt, int k, double* __restrict__ part) {
+                  double* __restrict__ Rt, double* __restrict__ part) {
   __shared__ double red[kT / 32];
   const int l = threadIdx.x & 31;
   const int64_t nsl = (n + 31) / 32;
-  double rs[kBlk];
+  double rs[K];
 #pragma unroll
-  for (int c = 0; c < kBlk; ++c) rs[c] = 0.0;
+  for (int c = 0; c < K; ++c) rs[c] = 0.0;
   for (int64_t sl = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; sl < nsl;
        sl += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int64_t o = off[sl] + l;
-    const int w = (int)((off[sl + 1] - off[sl]) >> 5);
-    double acc[kBlk];
-#pragma unroll
-    for (int c = 0; c < kBlk; ++c) acc[c] = 0.0;
-    for (int t = 0; t < w; ++t) {
-      const int64_t e = o + 32 * (int64_t)t;
-      const double v = sval[e];
-      const int64_t cc = scol[e];
-#pragma unroll
-      for (int c = 0; c < kBlk; ++c)
-        if (c < k) acc[c] += v * X[c * n + cc];
-    }
+    double acc[K];
+    sell_row_cols<K>(off, scol, sval, X, n, sl, l, acc);
     const int64_t r = sl * 32 + l;
     if (r < n) {
 #pragma unroll
-      for (int c = 0; c < kBlk; ++c)
-        if (c < k) {
-          const double ri = B[c * n + r] - acc[c];
-          Rt[c * n + r] = ri;
-          rs[c] += ri * ri;
-        }
+      for (int c = 0; c < K; ++c) {
+        const double ri = B[c * n + r] - acc[c];
+        Rt[c * n + r] = ri;
+        rs[c] += ri * ri;
+      }
     }
   }
-  for (int c = 0; c < k; ++c) {
+#pragma unroll
+  for (int c = 0; c < K; ++c) {
     const double sc = block_sum(rs[c], red);
     if (threadIdx.x == 0) part[(int64_t)c * kNb + blockIdx.x] = sc;
   }
 }
 
-// partial a_c.b_c per block for k columns
+// partial a_c.b_c per block, column c = blockIdx.y
 __global__ void __launch_bounds__(kT)
-k_dot_cols(int64_t n, const double* __restrict__ A, const double* __restrict__ B, int k, double* __restrict__ part) {
+k_dot_cols(int64_t n, const double* __restrict__ A, const double* __restrict__ B, double* __restrict__ part) {
   __shared__ double red[kT / 32];
-  for (int c = 0; c < k; ++c) {
-    double s = 0.0;
-    const double* a = A + (int64_t)c * n;
-    const double* b = B + (int64_t)c * n;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-      s += a[i] * b[i];
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) part[(int64_t)c * kNb + blockIdx.x] = s;
-  }
+  const int c = blockIdx.y;
+  double s = 0.0;
+  const double* a = A + (int64_t)c * n;
+  const double* b = B + (int64_t)c * n;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    s += a[i] * b[i];
+  s = block_sum(s, red);
+  if (threadIdx.x == 0) part[(int64_t)c * kNb + blockIdx.x] = s;
 }
 
 // per column (block c): the sum of its partials, then the scalar step `what`
@@ -168,37 +188,35 @@ __global__ void k_finish_cols(const double* __restrict__ part, double* __restric
   }
 }
 
-// X_c += alpha_c P_c, R_c -= alpha_c Q_c; partial r_c.r_c per block
+// X_c += alpha_c P_c, R_c -= alpha_c Q_c; partial r_c.r_c per block (c = blockIdx.y)
 __global__ void __launch_bounds__(kT)
 k_update_xr_cols(int64_t n, const double* __restrict__ scal, const double* __restrict__ P,
-                 const double* __restrict__ Q, double* __restrict__ X, double* __restrict__ R, int k,
+                 const double* __restrict__ Q, double* __restrict__ X, double* __restrict__ R,
                  double* __restrict__ part) {
   __shared__ double red[kT / 32];
-  for (int c = 0; c < k; ++c) {
-    const double alpha = scal[c * kSl + 1];
-    double s = 0.0;
-    const int64_t o = (int64_t)c * n;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-      X[o + i] += alpha * P[o + i];
-      const double ri = R[o + i] - alpha * Q[o + i];
-      R[o + i] = ri;
-      s += ri * ri;
-    }
-    s = block_sum(s, red);
-    if (threadIdx.x == 0) part[(int64_t)c * kNb + blockIdx.x] = s;
+  const int c = blockIdx.y;
+  const double alpha = scal[c * kSl + 1];
+  double s = 0.0;
+  const int64_t o = (int64_t)c * n;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+    X[o + i] += alpha * P[o + i];
+    const double ri = R[o + i] - alpha * Q[o + i];
+    R[o + i] = ri;
+    s += ri * ri;
   }
+  s = block_sum(s, red);
+  if (threadIdx.x == 0) part[(int64_t)c * kNb + blockIdx.x] = s;
 }
 
-// P_c = Z_c + beta_c P_c (active columns)
+// P_c = Z_c + beta_c P_c (active columns, c = blockIdx.y)
 __global__ void k_update_p_cols(int64_t n, const double* __restrict__ scal, const double* __restrict__ Z,
-                                double* __restrict__ P, int k) {
-  for (int c = 0; c < k; ++c) {
-    if (scal[c * kSl + 8] == 0.0) continue;
-    const double beta = scal[c * kSl + 2];
-    const int64_t o = (int64_t)c * n;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-      P[o + i] = Z[o + i] + beta * P[o + i];
-  }
+                                double* __restrict__ P) {
+  const int c = blockIdx.y;
+  if (scal[c * kSl + 8] == 0.0) return;
+  const double beta = scal[c * kSl + 2];
+  const int64_t o = (int64_t)c * n;
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    P[o + i] = Z[o + i] + beta * P[o + i];
 }
 
 // column c of Dst = column c of Src where mask[c] != 0 (replacement)
@@ -212,26 +230,53 @@ __global__ void k_copy_masked(int64_t n, const double* __restrict__ Src, double*
   }
 }
 
-// restriction of k columns: U_j (nD_j x k at k offN_j) and C (dimH x k)
+// restriction of K columns: U_j (nD_j x K at K offN_j), gathered by the blocks
+// y < gy of subdomain x, and C (dimH x K), coarse vector m by block y = gy + m:
+// one block per subdomain did all m K products one after another, 535 of 1690 us
+// of an apply at 64^3 with 8 columns, most SMs idle
+template <int K>
 __global__ void __launch_bounds__(kT)
 k_restrict_cols(const SubDesc* __restrict__ sub, const int32_t* __restrict__ Dlist, const double* __restrict__ R,
                 int64_t n, const double* __restrict__ Z, double* __restrict__ U, double* __restrict__ C, int dimH,
-                int k) {
-  const int j = blockIdx.x;
+                int gy) {
+  const int j = blockIdx.x, y = blockIdx.y;
   const SubDesc d = sub[j];
-  __shared__ double red[kT / 32];
   const int32_t* Dj = Dlist + d.offN;
-  double* uj = U + (int64_t)k * d.offN;
-  for (int c = 0; c < k; ++c)
-    for (int i = threadIdx.x; i < d.nD; i += blockDim.x) uj[(int64_t)c * d.nD + i] = R[c * n + Dj[i]];
-  const double* zj = Z + d.offZ;
-  for (int c = 0; c < k; ++c)
-    for (int m = 0; m < d.m; ++m) {
-      double s = 0.0;
-      for (int i = threadIdx.x; i < d.nD; i += blockDim.x) s += zj[(int64_t)m * d.nD + i] * R[c * n + Dj[i]];
-      s = block_sum(s, red);
-      if (threadIdx.x == 0) C[(int64_t)c * dimH + d.offH + m] = s;
+  if (y < gy) {
+    double* uj = U + (int64_t)K * d.offN;
+    for (int i = y * kT + threadIdx.x; i < d.nD; i += gy * kT) {
+      const double* r = R + Dj[i];
+#pragma unroll
+      for (int c = 0; c < K; ++c) uj[(int64_t)c * d.nD + i] = r[c * n];
     }
+    return;
+  }
+  const int m = y - gy;
+  if (m >= d.m) return;
+  __shared__ double red[kT / 32][K];
+  const double* zm = Z + d.offZ + (int64_t)m * d.nD;
+  double s[K];
+#pragma unroll
+  for (int c = 0; c < K; ++c) s[c] = 0.0;
+  for (int i = threadIdx.x; i < d.nD; i += kT) {
+    const double z = zm[i];
+    const double* r = R + Dj[i];
+#pragma unroll
+    for (int c = 0; c < K; ++c) s[c] += z * r[c * n];
+  }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int c = 0; c < K; ++c) {
+    const double v = warp_sum(s[c]);
+    if (lane == 0) red[wid][c] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < K) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kT / 32; ++w) t += red[w][threadIdx.x];
+    C[(int64_t)threadIdx.x * dimH + d.offH + m] = t;
+  }
 }
 
 // Y = X C with X = A_H^{-1} (row i read as column i): one warp per row
@@ -258,40 +303,65 @@ k_coarse_gemm(const double* __restrict__ X, int dim, const double* __restrict__ 
   }
 }
 
-// prolongation of k columns (gather form, as k_prolong in solve.cu)
+// prolongation of K columns (gather form, as k_prolong in solve.cu); each entry
+// of Z is read once for all columns
+template <int K>
 __global__ void __launch_bounds__(kT)
 k_prolong_cols(int64_t n, const uint8_t* __restrict__ dir, const double* __restrict__ R,
                const int64_t* __restrict__ invD_ptr, const int32_t* __restrict__ invD_sub,
                const int32_t* __restrict__ invD_loc, const SubDesc* __restrict__ sub, const double* __restrict__ U,
-               const double* __restrict__ Z, const double* __restrict__ Y, int dimH, double* __restrict__ Zout,
-               int k) {
+               const double* __restrict__ Z, const double* __restrict__ Y, int dimH, double* __restrict__ Zout) {
   for (int64_t kk = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; kk < n; kk += (int64_t)gridDim.x * blockDim.x) {
     if (dir[kk]) {
-      for (int c = 0; c < k; ++c) Zout[c * n + kk] = R[c * n + kk];
+#pragma unroll
+      for (int c = 0; c < K; ++c) Zout[c * n + kk] = R[c * n + kk];
       continue;
     }
-    double acc[kBlk];
+    double acc[K];
 #pragma unroll
-    for (int c = 0; c < kBlk; ++c) acc[c] = 0.0;
+    for (int c = 0; c < K; ++c) acc[c] = 0.0;
     for (int64_t t = invD_ptr[kk]; t < invD_ptr[kk + 1]; ++t) {
       const int j = invD_sub[t], i = invD_loc[t];
       const SubDesc& d = sub[j];
-      const double* uj = U + (int64_t)k * d.offN + i;
-      const double* zr = Z + d.offZ + i;
+      const double* uj = U + (int64_t)K * d.offN + i;
+      const int nD = d.nD;
+      double v[K];
 #pragma unroll
-      for (int c = 0; c < kBlk; ++c) {
-        if (c >= k) break;
-        double v = uj[(int64_t)c * d.nD];
-        if (Y)
-          for (int m = 0; m < d.m; ++m) v += zr[(int64_t)m * d.nD] * Y[(int64_t)c * dimH + d.offH + m];
-        acc[c] += v;
+      for (int c = 0; c < K; ++c) v[c] = uj[(int64_t)c * nD];
+      if (Y) {
+        const double* zr = Z + d.offZ + i;
+        const double* yr = Y + d.offH;
+        const int dm = d.m;
+#pragma unroll 2
+        for (int m = 0; m < dm; ++m) {
+          const double z = zr[(int64_t)m * nD];
+#pragma unroll
+          for (int c = 0; c < K; ++c) v[c] += z * yr[(int64_t)c * dimH + m];
+        }
       }
+#pragma unroll
+      for (int c = 0; c < K; ++c) acc[c] += v[c];
     }
 #pragma unroll
-    for (int c = 0; c < kBlk; ++c)
-      if (c < k) Zout[c * n + kk] = acc[c];
+    for (int c = 0; c < K; ++c) Zout[c * n + kk] = acc[c];
   }
 }
+
+// the call f(std::integral_constant<int, K>) for K = k (1 .. kBlk)
+template <typename F>
+void with_cols(int k, F f) {
+  switch (k) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 3: return f(std::integral_constant<int, 3>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    case 5: return f(std::integral_constant<int, 5>{});
+    case 6: return f(std::integral_constant<int, 6>{});
+    case 7: return f(std::integral_constant<int, 7>{});
+    default: return f(std::integral_constant<int, 8>{});
+  }
+}
+static_assert(kBlk == 8, "with_cols covers 1 .. 8 columns");
 
 double cond_est(const double* a, const double* b, int m, std::vector<double>& d, std::vector<double>& e) {
   if (m <= 0) return 1.0;
@@ -306,7 +376,11 @@ double cond_est(const double* a, const double* b, int m, std::vector<double>& d,
 // handle hold the subdomain vectors.
 geneo_status_t apply_prec_cols(geneo_handle_s* h, const double* R, double* Zo, int k, cudaStream_t s) {
   const int N = h->N;
-  k_restrict_cols<<<N, kT, 0, s>>>(h->dsub, h->Dlist, R, h->n, h->Z, h->blk_u, h->blk_c, std::max(h->dimH, 1), k);
+  const int gy = std::max(1, std::min(ceil_div(h->maxnD, kT), 4));
+  with_cols(k, [&](auto K) {
+    k_restrict_cols<K.value><<<dim3(N, gy + h->maxm), kT, 0, s>>>(h->dsub, h->Dlist, R, h->n, h->Z, h->blk_u,
+                                                                   h->blk_c, std::max(h->dimH, 1), gy);
+  });
   note_launch();
   GENEO_CUDA(cudaGetLastError());
   const double* Y = nullptr;
@@ -321,8 +395,10 @@ geneo_status_t apply_prec_cols(geneo_handle_s* h, const double* R, double* Zo, i
   GENEO_TRY(solve_set_run(h->setA, h->solve_streams, h->blk_u, h->blk_uoff, k, nullptr, nullptr, h->dstat, s));
   h->prof.end(pl, s);
   const int grid = (int)std::min<int64_t>((h->n + kT - 1) / kT, 152 * 8);
-  k_prolong_cols<<<grid, kT, 0, s>>>(h->n, h->dir, R, h->invD_ptr, h->invD_sub, h->invD_loc, h->dsub, h->blk_u,
-                                     h->Z, Y, std::max(h->dimH, 1), Zo, k);
+  with_cols(k, [&](auto K) {
+    k_prolong_cols<K.value><<<grid, kT, 0, s>>>(h->n, h->dir, R, h->invD_ptr, h->invD_sub, h->invD_loc, h->dsub,
+                                                h->blk_u, h->Z, Y, std::max(h->dimH, 1), Zo);
+  });
   note_launch();
   GENEO_CUDA(cudaGetLastError());
   return GENEO_OK;
@@ -384,7 +460,7 @@ geneo_status_t pcg_block(geneo_handle_s* h, const double* b, double* x, int k, d
   std::fill(hs.begin(), hs.end(), 0.0);
   for (int c = 0; c < k; ++c) hs[c * kSl + 8] = 1.0;
   GENEO_TRY(set_scal());
-  k_dot_cols<<<kNb, kT, 0, s>>>(n, b, b, k, part); note_launch();
+  k_dot_cols<<<dim3(kNb, k), kT, 0, s>>>(n, b, b, part); note_launch();
   k_finish_cols<<<k, kT, 0, s>>>(part, scal, 4, ha_d, hb_d, cap, 0); note_launch();
   GENEO_CUDA(cudaGetLastError());
   GENEO_TRY(read_scal());
@@ -402,10 +478,16 @@ geneo_status_t pcg_block(geneo_handle_s* h, const double* b, double* x, int k, d
     }
   }
   GENEO_TRY(set_scal());
+  auto true_residuals = [&]() {
+    with_cols(k, [&](auto K) {
+      k_resid_sell_cols<K.value><<<kNb, kT, 0, s>>>(n, h->sell_off, h->sell_col, h->sell_val, x, b, T, part);
+    });
+    note_launch();
+  };
   auto restart_all = [&]() -> geneo_status_t {  // Z = M^{-1} R, P = Z, rz (all columns)
     GENEO_TRY(apply_prec_cols(h, R, Zv, k, s));
     GENEO_CUDA(cudaMemcpyAsync(P, Zv, sizeof(double) * n * k, cudaMemcpyDeviceToDevice, s));
-    k_dot_cols<<<kNb, kT, 0, s>>>(n, R, Zv, k, part); note_launch();
+    k_dot_cols<<<dim3(kNb, k), kT, 0, s>>>(n, R, Zv, part); note_launch();
     k_finish_cols<<<k, kT, 0, s>>>(part, scal, 0, ha_d, hb_d, cap, 0); note_launch();
     GENEO_CUDA(cudaGetLastError());
     return GENEO_OK;
@@ -420,11 +502,14 @@ geneo_status_t pcg_block(geneo_handle_s* h, const double* b, double* x, int k, d
   while (it < maxit && it < cap - 1 && running()) {
     {
       const int pv = h->prof.begin(GENEO_PROF_SPMV, h->spmv_flops * k, h->spmv_bytes, s);
-      k_spmm_sell_cols<<<kNb, kT, 0, s>>>(n, h->sell_off, h->sell_col, h->sell_val, P, Q, k, part); note_launch();
+      with_cols(k, [&](auto K) {
+        k_spmm_sell_cols<K.value><<<kNb, kT, 0, s>>>(n, h->sell_off, h->sell_col, h->sell_val, P, Q, part);
+      });
+      note_launch();
       h->prof.end(pv, s);
     }
     k_finish_cols<<<k, kT, 0, s>>>(part, scal, 1, ha_d, hb_d, cap, it); note_launch();
-    k_update_xr_cols<<<kNb, kT, 0, s>>>(n, scal, P, Q, x, R, k, part); note_launch();
+    k_update_xr_cols<<<dim3(kNb, k), kT, 0, s>>>(n, scal, P, Q, x, R, part); note_launch();
     k_finish_cols<<<k, kT, 0, s>>>(part, scal, 2, ha_d, hb_d, cap, it); note_launch();
     GENEO_CUDA(cudaGetLastError());
     GENEO_TRY(read_scal());
@@ -449,7 +534,7 @@ geneo_status_t pcg_block(geneo_handle_s* h, const double* b, double* x, int k, d
     }
     std::fill(mask.begin(), mask.end(), 0);
     if (check) {
-      k_resid_sell_cols<<<kNb, kT, 0, s>>>(n, h->sell_off, h->sell_col, h->sell_val, x, b, T, k, part); note_launch();
+      true_residuals();
       k_finish_cols<<<k, kT, 0, s>>>(part, scal, 5, ha_d, hb_d, cap, it); note_launch();
       GENEO_CUDA(cudaGetLastError());
       GENEO_TRY(read_scal());
@@ -479,16 +564,16 @@ geneo_status_t pcg_block(geneo_handle_s* h, const double* b, double* x, int k, d
       k_copy_masked<<<kNb, kT, 0, s>>>(n, T, R, k, h->blk_mask); note_launch();
     }
     GENEO_TRY(apply_prec_cols(h, R, Zv, k, s));
-    k_dot_cols<<<kNb, kT, 0, s>>>(n, R, Zv, k, part); note_launch();
+    k_dot_cols<<<dim3(kNb, k), kT, 0, s>>>(n, R, Zv, part); note_launch();
     k_finish_cols<<<k, kT, 0, s>>>(part, scal, 3, ha_d, hb_d, cap, it - 1); note_launch();
-    k_update_p_cols<<<kNb, kT, 0, s>>>(n, scal, Zv, P, k); note_launch();
+    k_update_p_cols<<<dim3(kNb, k), kT, 0, s>>>(n, scal, Zv, P); note_launch();
     GENEO_CUDA(cudaGetLastError());
   }
   // columns still running at the cap: their true residual
   bool left = false;
   for (int c = 0; c < k; ++c) left |= state[c] == 0 || !std::isfinite(rel_true[c]);
   if (left) {
-    k_resid_sell_cols<<<kNb, kT, 0, s>>>(n, h->sell_off, h->sell_col, h->sell_val, x, b, T, k, part); note_launch();
+    true_residuals();
     k_finish_cols<<<k, kT, 0, s>>>(part, scal, 5, ha_d, hb_d, cap, it); note_launch();
     GENEO_CUDA(cudaGetLastError());
     GENEO_TRY(read_scal());
