@@ -209,88 +209,100 @@ k_band_potrf(T* __restrict__ base, const BandDesc* __restrict__ descs, int phmax
   }
 }
 
-// Right-looking factorisation of one large band over many SMs (the coarse
-// matrix A_H, whose FP64 work is too much for one SM).  Per panel of NB
-// columns: one warp factors the diagonal block (k_band_panel_diag), a grid
-// of one-warp blocks solves the panel rows below it, one row per thread
-// (k_band_panel_rows), then a grid of 64 x 64 tiles applies the rank-NB
-// update to the trailing window (k_band_trail).  Three launches per panel;
-// the stream orders them.  GB300 issues FP64 at 2 fused multiply-adds per
-// clock per SM, so the rows' solves (h NB^2 / 2 of them) are spread over
-// h / 32 SMs instead of one.
-template <typename T, int NB>
-__global__ void __launch_bounds__(32)
+// Right-looking factorisation of FP64 bands over many SMs: the coarse matrix
+// A_H, and batches of fewer subdomain bands than the GPU has SMs.  GB300 issues
+// FP64 at 2 fused multiply-adds per clock per SM, so one thread block per
+// matrix (k_band_potrf) leaves a batch of 27 bands of order 9261 and half width
+// 463 to 27 SMs: 202 ms, against 33 ms of FP64 work for all 152.  Per panel of
+// 32 columns, every matrix at once (grid y): the diagonal block
+// (k_band_panel_diag), the panel rows below it, one row per thread
+// (k_band_panel_rows), and the rank-32 update of the trailing window in 32 x 32
+// tiles (k_band_trail).  Three launches per panel; the stream orders them.
+constexpr int kPN = 32;   // panel width
+
+// Four warps, lane r holds row r of the columns c with c % 4 = warp: the warp of
+// column t takes pivot and column, the block passes the column on through
+// shared memory, and every warp updates its own columns.  The four warps run on
+// the SM's four FP64 units.
+template <typename T>
+__global__ void __launch_bounds__(128)
 k_band_panel_diag(T* __restrict__ base, const BandDesc* __restrict__ descs, int kb, DevStatus* st) {
-  const BandDesc d = descs[0];
+  const BandDesc d = descs[blockIdx.x];
   const int n = d.n, w = d.w;
+  if (kb >= n) return;
   const int64_t ld = d.ld;
   T* L = base + d.off;
-  __shared__ T Dk[NB * (NB + 1)];
-  constexpr int DS = NB + 1;
-  const int lane = threadIdx.x;
-  const int b = min(NB, n - kb);
-  for (int idx = lane; idx < NB * NB; idx += 32) {
-    const int r = idx / NB, c = idx % NB;
-    T v = T(0);
-    if (r < b && c < b && r >= c && r - c <= w) v = L[bidx(kb + r, kb + c, w, ld)];
-    Dk[r * DS + c] = v;
+  __shared__ T col[2][kPN];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int b = min(kPN, n - kb);
+  T a[kPN / 4];
+#pragma unroll
+  for (int i = 0; i < kPN / 4; ++i) {
+    const int c = 4 * i + wid;
+    a[i] = (lane < b && c <= lane && lane - c <= w) ? L[bidx(kb + lane, kb + c, w, ld)] : T(0);
   }
-  __syncwarp();
-  for (int t = 0; t < b; ++t) {
-    if (lane == t) {
-      T dv = Dk[t * DS + t];
-      if (!finite_pos(dv)) {
-        record_error(st, isfinite(dv) ? GENEO_ERR_NOT_SPD : GENEO_ERR_NONFINITE, d.id, (int64_t)kb + t);
-        dv = T(1);
+#pragma unroll
+  for (int t = 0; t < kPN; ++t) {
+    if (t < b) {   // the same for the whole block
+      if (wid == (t & 3)) {
+        T p = __shfl_sync(0xffffffffu, a[t >> 2], t);
+        if (!finite_pos(p)) {
+          if (lane == 0)
+            record_error(st, isfinite(p) ? GENEO_ERR_NOT_SPD : GENEO_ERR_NONFINITE, d.id, (int64_t)kb + t);
+          p = T(1);
+        }
+        const T s = sqrt(p);
+        a[t >> 2] = lane == t ? s : lane > t ? a[t >> 2] / s : T(0);
+        col[t & 1][lane] = a[t >> 2];
       }
-      Dk[t * DS + t] = sqrt(dv);
+      __syncthreads();
+      const T lrt = col[t & 1][lane];
+#pragma unroll
+      for (int i = 0; i < kPN / 4; ++i) {
+        const int c = 4 * i + wid;
+        if (4 * i + 3 > t && c > t && lane >= c) a[i] -= lrt * col[t & 1][c];
+      }
     }
-    __syncwarp();
-    const T piv = Dk[t * DS + t];
-    if (lane > t && lane < b) Dk[lane * DS + t] /= piv;
-    __syncwarp();
-    if (lane > t && lane < b) {
-      const T lrt = Dk[lane * DS + t];
-      for (int u = t + 1; u <= lane; ++u) Dk[lane * DS + u] -= lrt * Dk[u * DS + t];
-    }
-    __syncwarp();
   }
-  for (int idx = lane; idx < NB * NB; idx += 32) {
-    const int r = idx / NB, c = idx % NB;
-    if (r < b && c < b && r >= c && r - c <= w) L[bidx(kb + r, kb + c, w, ld)] = Dk[r * DS + c];
+#pragma unroll
+  for (int i = 0; i < kPN / 4; ++i) {
+    const int c = 4 * i + wid;
+    if (lane < b && c <= lane && lane - c <= w) L[bidx(kb + lane, kb + c, w, ld)] = a[i];
   }
 }
 
-// Rows kb + b + 32 blockIdx.x + lane of the panel: x L_kk^T = a (the
-// diagonal block already factored), multiplying by the pivots' reciprocals.
-template <typename T, int NB>
+// Rows kb + b + 32 blockIdx.x + lane of the panel of matrix blockIdx.y:
+// x L_kk^T = a (the diagonal block already factored), multiplying by the
+// pivots' reciprocals.
+template <typename T>
 __global__ void __launch_bounds__(32)
 k_band_panel_rows(T* __restrict__ base, const BandDesc* __restrict__ descs, int kb) {
-  const BandDesc d = descs[0];
+  const BandDesc d = descs[blockIdx.y];
   const int n = d.n, w = d.w;
+  const int b = min(kPN, n - kb);
+  const int h = min(w, n - kb - b);
+  if (kb >= n || 32 * (int)blockIdx.x >= h) return;
   const int64_t ld = d.ld;
   T* L = base + d.off;
-  __shared__ T Dk[NB * (NB + 1)];
-  __shared__ T rp[NB];
-  constexpr int DS = NB + 1;
+  __shared__ T Dk[kPN * (kPN + 1)];
+  __shared__ T rp[kPN];
+  constexpr int DS = kPN + 1;
   const int lane = threadIdx.x;
-  const int b = min(NB, n - kb);
-  const int h = min(w, n - kb - b);
-  for (int idx = lane; idx < NB * NB; idx += 32) {
-    const int r = idx / NB, c = idx % NB;
+  for (int idx = lane; idx < kPN * kPN; idx += 32) {
+    const int r = idx / kPN, c = idx % kPN;
     Dk[r * DS + c] = (r < b && c < b && r >= c && r - c <= w) ? L[bidx(kb + r, kb + c, w, ld)] : T(0);
   }
   __syncwarp();
-  for (int t = lane; t < NB; t += 32) rp[t] = t < b ? T(1) / Dk[t * DS + t] : T(0);
+  rp[lane] = lane < b ? T(1) / Dk[lane * DS + lane] : T(0);
   __syncwarp();
   const int i = 32 * blockIdx.x + lane;
   if (i >= h) return;
   const int rr = kb + b + i;
-  T x[NB];
+  T x[kPN];
 #pragma unroll
-  for (int t = 0; t < NB; ++t) x[t] = (t < b && rr - (kb + t) <= w) ? L[bidx(rr, kb + t, w, ld)] : T(0);
+  for (int t = 0; t < kPN; ++t) x[t] = (t < b && rr - (kb + t) <= w) ? L[bidx(rr, kb + t, w, ld)] : T(0);
 #pragma unroll
-  for (int t = 0; t < NB; ++t) {
+  for (int t = 0; t < kPN; ++t) {
     if (t < b) {
       T v = x[t];
 #pragma unroll
@@ -299,64 +311,68 @@ k_band_panel_rows(T* __restrict__ base, const BandDesc* __restrict__ descs, int 
     }
   }
 #pragma unroll
-  for (int t = 0; t < NB; ++t)
+  for (int t = 0; t < kPN; ++t)
     if (t < b && rr - (kb + t) <= w) L[bidx(rr, kb + t, w, ld)] = x[t];
 }
 
-// Trailing update of panel kb: C(i, i') -= sum_t P(i, t) P(i', t) over the
-// h x h window below the panel, block (ti, tj) of 64 x 64 (ti >= tj), 4 x 4
-// register tiles, panel rows staged in shared memory.
-template <typename T, int NB>
-__global__ void __launch_bounds__(kThreads)
+// Trailing update of panel kb of matrix blockIdx.y: C(i, i') -= sum_t P(i, t)
+// P(i', t) over the h x h window below the panel, tile (ti, tj) of 32 x 32
+// (ti >= tj), one 4 x 4 register tile per thread, panel rows staged in shared
+// memory.  Tiles of 32 rather than 64 keep the share of the work outside the
+// window's lower triangle small (14 % at h = 463, not 37 %) and give a batch
+// enough blocks to even out.
+constexpr int kTT = 32;
+template <typename T>
+__global__ void __launch_bounds__(64)
 k_band_trail(T* __restrict__ base, const BandDesc* __restrict__ descs, int kb) {
-  const BandDesc d = descs[0];
+  const BandDesc d = descs[blockIdx.y];
   const int n = d.n, w = d.w;
-  const int64_t ld = d.ld;
-  T* L = base + d.off;
-  const int b = min(NB, n - kb);
+  const int b = min(kPN, n - kb);
   const int h = min(w, n - kb - b);
   // block index -> (ti, tj) in the lower triangle, row-major
   const int t = blockIdx.x;
-  int ti = (int)((sqrt(8.0 * t + 1.0) - 1.0) * 0.5);
+  int ti = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
   while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
   while (ti * (ti + 1) / 2 > t) --ti;
   const int tj = t - ti * (ti + 1) / 2;
-  const int i0 = 64 * ti, j0 = 64 * tj;
-  if (i0 >= h) return;
-  __shared__ T Pi[NB][64 + 1], Pj[NB][64 + 1];
-  for (int idx = threadIdx.x; idx < NB * 64; idx += blockDim.x) {
-    const int tt = idx / 64, r = idx % 64;
+  const int i0 = kTT * ti, j0 = kTT * tj;
+  if (kb >= n || i0 >= h) return;
+  const int64_t ld = d.ld;
+  T* L = base + d.off;
+  // row-major in t: a thread's four rows (columns) are one 32-byte read
+  __shared__ __align__(16) T Pi[kPN][kTT + 2], Pj[kPN][kTT + 2];
+  for (int idx = threadIdx.x; idx < kPN * kTT; idx += 64) {
+    const int tt = idx % kPN, r = idx / kPN;   // consecutive threads along a band row
     const int ii = i0 + r, jj = j0 + r;
     Pi[tt][r] = (tt < b && ii < h && b + ii - tt <= w) ? L[bidx(kb + b + ii, kb + tt, w, ld)] : T(0);
     Pj[tt][r] = (tt < b && jj < h && b + jj - tt <= w) ? L[bidx(kb + b + jj, kb + tt, w, ld)] : T(0);
   }
   __syncthreads();
-  const int ty = threadIdx.x / 16, tx = threadIdx.x % 16;  // 16 x 16 threads, 4 x 4 each
+  const int tr = threadIdx.x >> 3, tc = threadIdx.x & 7;
+  if (ti == tj && 4 * tc > 4 * tr + 3) return;   // above the diagonal
   T acc[4][4];
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
+  for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[a][c] = T(0);
-  for (int tt = 0; tt < b; ++tt) {
+    for (int p = 0; p < 4; ++p) acc[q][p] = T(0);
+#pragma unroll 4
+  for (int tt = 0; tt < kPN; ++tt) {
     T pr[4], pc[4];
+    load4(&Pi[tt][4 * tr], pr);
+    load4(&Pj[tt][4 * tc], pc);
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      pr[a] = Pi[tt][4 * ty + a];
-      pc[a] = Pj[tt][4 * tx + a];
-    }
+    for (int q = 0; q < 4; ++q)
 #pragma unroll
-    for (int a = 0; a < 4; ++a)
-#pragma unroll
-      for (int c = 0; c < 4; ++c) acc[a][c] += pr[a] * pc[c];
+      for (int p = 0; p < 4; ++p) acc[q][p] += pr[q] * pc[p];
   }
 #pragma unroll
-  for (int a = 0; a < 4; ++a) {
-    const int i = i0 + 4 * ty + a;
+  for (int q = 0; q < 4; ++q) {
+    const int i = i0 + 4 * tr + q;
     if (i >= h) continue;
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int jj = j0 + 4 * tx + c;
-      if (jj < h && jj <= i) L[bidx(kb + b + i, kb + b + jj, w, ld)] -= acc[a][c];
+    for (int p = 0; p < 4; ++p) {
+      const int c = j0 + 4 * tc + p;
+      if (c < h && i >= c) L[bidx(kb + b + i, kb + b + c, w, ld)] -= acc[q][p];
     }
   }
 }
@@ -938,6 +954,16 @@ k_band_solve(const T* __restrict__ base, const BandDesc* __restrict__ descs,
       mbar_wait_bounded(&bars[v % kStages], (uint32_t)((v / kStages) & 1), st, d.id, v);
 }
 
+inline int sm_count() {
+  static int sms[64] = {0};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+  if (!sms[dev] && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+    cudaGetLastError();
+    return 152;
+  }
+  return sms[dev];
+}
 constexpr int kNB = 32;
 constexpr size_t kSmemCap = 200 * 1024;
 
@@ -983,21 +1009,29 @@ geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w,
       return band_blkinv(base, d_desc, count, max_n, blk_mask, s);
     }
   }
-  // one large matrix (the coarse matrix): spread each panel's update over SMs
-  if (count == 1 && max_n > 256 && max_w >= 128 && !weak) {
-    constexpr int PB = 32;
-    for (int kb = 0; kb < max_n; kb += PB) {
-      k_band_panel_diag<T, PB><<<1, 32, 0, s>>>(base, d_desc, kb, st); note_launch();
-      const int b = std::min(PB, max_n - kb);
-      const int h = std::min(max_w, max_n - kb - b);
-      if (h > 0) {
-        k_band_panel_rows<T, PB><<<(h + 31) / 32, 32, 0, s>>>(base, d_desc, kb); note_launch();
-        const int T64 = (h + 63) / 64;
-        k_band_trail<T, PB><<<T64 * (T64 + 1) / 2, kThreads, 0, s>>>(base, d_desc, kb); note_launch();
+  // FP64 bands too few for one SM each: every panel's work spread over the GPU.
+  // Both sides in units of 32^3 / 2 multiply-adds: one block per matrix runs the
+  // widest alone on its SM; spread, a panel's three launches cost about 75 us
+  // (measured: 20 + 24 + 3 x 4 beside the update) whatever the batch
+  if constexpr (sizeof(T) == 8) {
+    if (!weak && max_n > 256 && max_w >= 96) {
+      const double panel = 0.5 * (double)max_w * max_w * kPN;          // multiply-adds of one panel's update
+      const double alone = panel / 2.0 * ceil_div(count, sm_count());  // clocks, 2 per clock and SM
+      const double spread = 1.2 * panel * count / (2.0 * sm_count()) + 150e3;
+      if (spread < alone) {
+        for (int kb = 0; kb < max_n; kb += kPN) {
+          k_band_panel_diag<T><<<count, 128, 0, s>>>(base, d_desc, kb, st); note_launch();
+          const int h = std::min(max_w, max_n - kb - std::min(kPN, max_n - kb));
+          if (h > 0) {
+            const int nt = (h + kTT - 1) / kTT;
+            k_band_panel_rows<T><<<dim3((h + 31) / 32, count), 32, 0, s>>>(base, d_desc, kb); note_launch();
+            k_band_trail<T><<<dim3(nt * (nt + 1) / 2, count), 64, 0, s>>>(base, d_desc, kb); note_launch();
+          }
+        }
+        GENEO_CUDA(cudaGetLastError());
+        return band_blkinv(base, d_desc, count, max_n, blk_mask, s);
       }
     }
-    GENEO_CUDA(cudaGetLastError());
-    return band_blkinv(base, d_desc, count, max_n, blk_mask, s);
   }
   // the panel starts at a 16-byte boundary (diag block: 32 x 33 values) and
   // its row stride phmax is a multiple of 4
@@ -1028,16 +1062,6 @@ size_t solve_smem(int max_w, int k, int ring, int snb, int stages) {
 // into parts (grid y) that run on otherwise idle SMs, each part a shorter
 // dependent sweep with less work per step; at most `units` parts and no more
 // blocks than SMs.
-inline int sm_count() {
-  static int sms[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
-  if (!sms[dev] && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 152;
-  }
-  return sms[dev];
-}
 inline int split_parts(int count, int units) {
   const int sms = sm_count();
   if (count <= 0 || 2 * count > sms || units <= 1) return 1;
