@@ -40,7 +40,8 @@ namespace {
 
 constexpr int kT = 256;
 constexpr int kMaxW = 104;      // largest [X, Q] width handled by the dense kernels
-constexpr int kRS = 4;          // row splits of the Gram kernel
+constexpr int kMinRS = 4, kMaxRS = 16;  // row splits of the Gram kernels (grid x)
+constexpr int kTD = 512;        // most threads of the dense kernels
 constexpr int kRB = 32;         // rows per shared-memory chunk in the Gram kernel
 constexpr int kMaxSweeps = 40;  // bound of the Jacobi sweep loop
 constexpr int kFirstPassNev = 8; // wanted pairs of the narrow first pass
@@ -336,7 +337,8 @@ k_gram_part(const SubDesc* __restrict__ sub, ColRefT<S> A, ColRefT<S> B, int sym
   for (int u = 0; u < 3; ++u)
 #pragma unroll
     for (int z = 0; z < 16; ++z) acc[u][z] = 0;
-  const int r0 = (int)((int64_t)rs * d.nN / kRS), r1 = (int)((int64_t)(rs + 1) * d.nN / kRS);
+  const int nrs = (int)gridDim.x;
+  const int r0 = (int)((int64_t)rs * d.nN / nrs), r1 = (int)((int64_t)(rs + 1) * d.nN / nrs);
   for (int rb = r0; rb < r1; rb += kRB) {
     const int nr = min(kRB, r1 - rb);
     __syncthreads();
@@ -455,7 +457,8 @@ k_gram_one(const SubDesc* __restrict__ sub, ColRefT<S> A, ColRefT<S> B, int sym,
   Acc acc[16];
 #pragma unroll
   for (int z = 0; z < 16; ++z) acc[z] = Acc{};
-  const int r0 = (int)((int64_t)rs * d.nN / kRS), r1 = (int)((int64_t)(rs + 1) * d.nN / kRS);
+  const int nrs = (int)gridDim.x;
+  const int r0 = (int)((int64_t)rs * d.nN / nrs), r1 = (int)((int64_t)(rs + 1) * d.nN / nrs);
   // thread (lane, warp) handles row `lane` of a chunk and the combined
   // [A | B] columns warp + 8 u (kRB = 32 rows, 8 warps, up to 128 columns);
   // rows beyond the range and padded columns are zero
@@ -563,7 +566,7 @@ k_gram_one(const SubDesc* __restrict__ sub, ColRefT<S> A, ColRefT<S> B, int sym,
 template <typename S>
 __global__ void k_gram_reduce(const SubDesc* __restrict__ sub, ColRefT<S> A, ColRefT<S> B, int sym,
                               const double* __restrict__ Gp, double* __restrict__ G, int ldg,
-                              int nsub, const int32_t* __restrict__ skip) {
+                              int nsub, const int32_t* __restrict__ skip, int nrs) {
   const int j = blockIdx.x;
   if (skip && skip[j]) return;
   const int p = cr_w(A, j), q = cr_w(B, j);
@@ -572,7 +575,7 @@ __global__ void k_gram_reduce(const SubDesc* __restrict__ sub, ColRefT<S> A, Col
     int rr = r, cc = c;
     if (sym && c > r) { rr = c; cc = r; }
     double s = 0.0;
-    for (int rs = 0; rs < kRS; ++rs) s += Gp[((int64_t)rs * nsub + j) * ldg * ldg + (int64_t)cc * ldg + rr];
+    for (int rs = 0; rs < nrs; ++rs) s += Gp[((int64_t)rs * nsub + j) * ldg * ldg + (int64_t)cc * ldg + rr];
     G[(int64_t)j * ldg * ldg + (int64_t)c * ldg + r] = s;
   }
 }
@@ -829,6 +832,36 @@ __device__ __forceinline__ bool jacobi_rot(T app, T aqq, T apq, T& c, T& s) {
   s = t * c;
   return s != T(0);
 }
+// FP64: the divisions and square roots of the formula above are dependent
+// chains on a pipe of 1/64 of the FP32 rate, a third of k_rr<double> (2.25 ms
+// a launch at 27 subdomains, m = 39).  The tangent is formed in FP32 and
+// improved by one Newton step on a_pq t^2 + (a_qq - a_pp) t - a_pq = 0 whose
+// residual is FP64 (error of the order of the FP32 error squared); c = (1 +
+// t^2)^(-1/2) is FP64, so c^2 + s^2 = 1 holds to FP64 rounding.
+template <>
+__device__ __forceinline__ bool jacobi_rot<double>(double app, double aqq, double apq, double& c, double& s) {
+  using J = JacobiOps<double>;
+  const double a = fabs(apq);
+  if (!(a > J::tiny && a * a > J::eps_rot * J::eps_rot * fabs(app * aqq))) return false;
+  const double dd = aqq - app;
+  const float af = (float)apq, df = (float)dd;
+  double t;
+  if (fabsf(af) > 1e-30f && fabsf(af) < 1e30f && fabsf(df) < 1e30f) {
+    const float theta = df / (2.f * af);
+    float t0 = copysignf(1.f, theta) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f)));
+    if (fabsf(theta) > 1e15f) t0 = 0.5f / theta;
+    const double td = (double)t0;
+    const double f = fma(fma(apq, td, dd), td, -apq);
+    const float fp = fmaf(2.f * af, t0, df);
+    t = fp != 0.f ? td - (double)((float)f / fp) : td;
+  } else {
+    const double theta = dd / (2.0 * apq);
+    t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+  }
+  c = rsqrt(fma(t, t, 1.0));
+  s = t * c;
+  return s != 0.0;
+}
 // Double-single: the angle in FP32 from the double-single difference of the
 // pivots.  An angle good to FP32 leaves a_pq about 1e-7 of its size instead of
 // zero (the next sweep removes the rest, Jacobi converges just as well with
@@ -965,7 +998,7 @@ __device__ void jacobi_eig(T* A, int lda, T* V, int ldv, int m, T* cs, T* sn,
 // stride wmax + 1), arithmetic T.
 template <typename T>
 size_t dense_smem_bytes(int wmax) {
-  return sizeof(T) * ((size_t)2 * wmax * (wmax + 1) + 6 * (size_t)wmax + kT / 32 + 8);
+  return sizeof(T) * ((size_t)2 * wmax * (wmax + 1) + 6 * (size_t)wmax + kTD / 32);
 }
 
 // SVQB: columns whose Gram matrix is G (q x q) -> T (q x r) with
@@ -973,7 +1006,7 @@ size_t dense_smem_bytes(int wmax) {
 // removed.  Writes T into Tout (ldg) and r into r_out[j].  The Jacobi step
 // runs in arithmetic T (FP32 for a Gram formed in FP32 arithmetic).
 template <typename T>
-__global__ void __launch_bounds__(kT)
+__global__ void __launch_bounds__(kTD)
 k_svqb(const double* __restrict__ Gall, double* __restrict__ Tout, int ldg,
        const int32_t* __restrict__ wq, const int32_t* __restrict__ wq2, int32_t* __restrict__ r_out,
        double drop, const int32_t* __restrict__ skip, int wmax) {
@@ -1124,7 +1157,7 @@ __global__ void k_fill_i32(int32_t* __restrict__ dst, int32_t v, int n) {
 // the FP32 rate, and the sweeps are most of this kernel).  The double-single
 // sweeps run on G scaled by a power of two to |g_ij| < 1 (exact).
 template <typename T>
-__global__ void __launch_bounds__(kT)
+__global__ void __launch_bounds__(kTD)
 k_rr(const double* __restrict__ Gall, double* __restrict__ Tout, int ldg,
      const int32_t* __restrict__ sj, const int32_t* __restrict__ qj, double* __restrict__ nu_out,
      int ldnu, const int32_t* __restrict__ skip, int wmax) {
@@ -1142,7 +1175,7 @@ k_rr(const double* __restrict__ Gall, double* __restrict__ Tout, int ldg,
   T* sn = cs + wmax;
   auto* red = reinterpret_cast<typename JacobiOps<T>::R*>(sn + wmax);
   __shared__ int order[kMaxW];
-  __shared__ double wmx[kT / 32];
+  __shared__ double wmx[kTD / 32];
   if (m <= 0) return;
   const double* G = Gall + (int64_t)j * ldg * ldg;
   int ex = 0;
@@ -1184,129 +1217,147 @@ k_rr(const double* __restrict__ Gall, double* __restrict__ Tout, int ldg,
   for (int k = threadIdx.x; k < s; k += blockDim.x) nu_out[(int64_t)j * ldnu + k] = ev[order[k]];
 }
 
-// Residuals, convergence and the next search block.  One block per
-// subdomain.  R = BX - KX diag(nu) is written (active columns only,
-// compacted) to S after X, then the s_p columns of P follow.
+// Residuals, convergence and the next search block, in three kernels (one
+// block per subdomain took 517 us at 64 subdomains of 9261 dofs, 11 columns:
+// eight warps on 64 SMs).
+// 1. relative residual norms: column blockIdx.x of subdomain blockIdx.y
 __global__ void __launch_bounds__(kT)
-k_resid(const SubDesc* __restrict__ sub, ColRef S, ColRef BX, ColRef KX, ColRef P,
-        const double* __restrict__ nu_all, int ldnu, const int32_t* __restrict__ sj,
-        const int32_t* __restrict__ spj, int32_t* __restrict__ aj, int32_t* __restrict__ qj,
-        int32_t* __restrict__ done, int32_t* __restrict__ iters, int32_t* __restrict__ notdone,
-        double* __restrict__ rn_out, double tol, double tau, double sigma, const int32_t* __restrict__ nevj, int fixed,
-        int it, double* __restrict__ best, int32_t* __restrict__ stall, int32_t* __restrict__ o64,
-        int32_t* __restrict__ ok32, int stall_lim) {
-  const int j = blockIdx.x;
-  if (done[j]) return;
+k_resid_norm(const SubDesc* __restrict__ sub, ColRef BX, ColRef KX, const double* __restrict__ nu_all, int ldnu,
+             const int32_t* __restrict__ sj, const int32_t* __restrict__ done, double* __restrict__ rn_out) {
+  const int j = blockIdx.y, c = blockIdx.x;
+  if (done[j] || c >= sj[j]) return;
   const SubDesc d = sub[j];
-  const int s = sj[j];
-  const int nev = nevj[j];
-  const double* nu = nu_all + (int64_t)j * ldnu;
-  const double* bx = cr_ptr(BX, d, j);
-  const double* kx = cr_ptr(KX, d, j);
-  __shared__ double rn[kMaxW];
-  __shared__ int act[kMaxW];
-  __shared__ int na, fin;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  for (int c = wid; c < s; c += nw) {
-    double r2 = 0.0, b2 = 0.0, k2 = 0.0;
-    const double* bc = bx + (int64_t)c * d.nN;
-    const double* kc = kx + (int64_t)c * d.nN;
-    const double nc = nu[c];
-    for (int a = lane; a < d.nN; a += 32) {
-      const double bv = bc[a], kv = kc[a];
-      const double rv = bv - nc * kv;
-      r2 += rv * rv;
-      b2 += bv * bv;
-      k2 += kv * kv;
-    }
-    r2 = warp_sum(r2);
-    b2 = warp_sum(b2);
-    k2 = warp_sum(k2);
-    if (lane == 0) {
-      const double den = sqrt(b2) + fabs(nc) * sqrt(k2);
-      rn[c] = den > 0.0 ? sqrt(r2) / den : 0.0;
-    }
+  const double* __restrict__ bc = cr_ptr(BX, d, j) + (int64_t)c * d.nN;
+  const double* __restrict__ kc = cr_ptr(KX, d, j) + (int64_t)c * d.nN;
+  const double nc = nu_all[(int64_t)j * ldnu + c];
+  __shared__ double red[3][kT / 32];
+  double r2 = 0.0, b2 = 0.0, k2 = 0.0;
+#pragma unroll 4
+  for (int a = threadIdx.x; a < d.nN; a += kT) {
+    const double bv = bc[a], kv = kc[a];
+    const double rv = bv - nc * kv;
+    r2 += rv * rv;
+    b2 += bv * bv;
+    k2 += kv * kv;
+  }
+  r2 = warp_sum(r2);
+  b2 = warp_sum(b2);
+  k2 = warp_sum(k2);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (lane == 0) {
+    red[0][wid] = r2;
+    red[1][wid] = b2;
+    red[2][wid] = k2;
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    bool ok = true;
-    if (fixed) {
-      for (int i = 0; i < min(nev, s); ++i) ok = ok && rn[i] <= tol;
-    } else {
-      for (int i = 0; i < min(nev, s); ++i) {
-        if (rn[i] > tol) { ok = false; break; }
-        const double lam = nu[i] > 0.0 ? sigma + 1.0 / nu[i] : INFINITY;
-        if (lam >= tau) break;
-      }
+    r2 = b2 = k2 = 0.0;
+    for (int w = 0; w < kT / 32; ++w) {
+      r2 += red[0][w];
+      b2 += red[1][w];
+      k2 += red[2][w];
     }
-    int k = 0;
-    for (int i = 0; i < s; ++i)
-      if (rn[i] > tol) act[k++] = i;
-    na = k;
-    fin = ok || k == 0;
-    if (fin) {
-      done[j] = 1;
-    } else {
-      atomicAdd(notdone, 1);
-    }
-    // FP32 first passes: a subdomain whose largest wanted residual has not
-    // halved in stall_lim iterations (counted after iteration kStallFrom of
-    // the pass), or that is still iterating at iteration kForce64From,
-    // switches to FP64 products and orthogonalisation (notdone[1] counts the
-    // switches)
-    if (best && !fin && !o64[j]) {
-      double r = 0.0;
-      for (int i = 0; i < min(nev, s); ++i) {
-        r = fmax(r, rn[i]);
-        const double lam = nu[i] > 0.0 ? sigma + 1.0 / nu[i] : INFINITY;
-        if (!fixed && lam >= tau) break;
-      }
-      bool sw = false;
-      if (it >= kForce64From) {  // a straggler: FP64 from here on
-        sw = true;
-      } else if (it <= kStallFrom || r < 0.5 * best[j]) {
-        best[j] = r;
-        stall[j] = 0;
-      } else if (++stall[j] >= stall_lim) {
-        sw = true;
-      }
-      if (sw) {
-        o64[j] = 1;
-        ok32[j] = 0;
-        atomicAdd(notdone + 1, 1);
-      }
-    }
-    iters[j] = it;
-    aj[j] = fin ? 0 : k;
-    qj[j] = fin ? 0 : k + spj[j];
-    for (int i = 0; i < s; ++i) rn_out[(int64_t)j * ldnu + i] = rn[i];
-  }
-  __syncthreads();
-  if (fin) return;
-  double* sbase = cr_ptr(S, d, j);
-  double* w0 = sbase + (int64_t)s * d.nN;
-  const int k = na;
-  // S, BX, KX and P are distinct buffers: the loads of later rows may be
-  // issued before the stores of earlier ones
-  for (int t = 0; t < k; ++t) {
-    const int c = act[t];
-    const double nc = nu[c];
-    const double* __restrict__ bc = bx + (int64_t)c * d.nN;
-    const double* __restrict__ kc = kx + (int64_t)c * d.nN;
-    double* __restrict__ o = w0 + (int64_t)t * d.nN;
-#pragma unroll 4
-    for (int a = threadIdx.x; a < d.nN; a += blockDim.x) o[a] = bc[a] - nc * kc[a];
-  }
-  const int sp = spj[j];
-  const double* pc = cr_ptr(P, d, j);
-  for (int t = 0; t < sp; ++t) {
-    double* __restrict__ o = w0 + (int64_t)(k + t) * d.nN;
-    const double* __restrict__ src = pc + (int64_t)t * d.nN;
-#pragma unroll 4
-    for (int a = threadIdx.x; a < d.nN; a += blockDim.x) o[a] = src[a];
+    const double den = sqrt(b2) + fabs(nc) * sqrt(k2);
+    rn_out[(int64_t)j * ldnu + c] = den > 0.0 ? sqrt(r2) / den : 0.0;
   }
 }
 
+// 2. convergence and the active columns (act, aj of them), one warp per subdomain
+__global__ void __launch_bounds__(32)
+k_resid_decide(const double* __restrict__ nu_all, int ldnu, const int32_t* __restrict__ sj,
+               const int32_t* __restrict__ spj, int32_t* __restrict__ aj, int32_t* __restrict__ qj,
+               int32_t* __restrict__ act_all, int32_t* __restrict__ done, int32_t* __restrict__ iters,
+               int32_t* __restrict__ notdone, const double* __restrict__ rn_all, double tol, double tau, double sigma,
+               const int32_t* __restrict__ nevj, int fixed, int it, double* __restrict__ best,
+               int32_t* __restrict__ stall, int32_t* __restrict__ o64, int32_t* __restrict__ ok32, int stall_lim) {
+  const int j = blockIdx.x;
+  if (done[j]) return;
+  const int s = sj[j];
+  const int nev = nevj[j];
+  __shared__ double rn[kMaxW], nu[kMaxW];
+  for (int i = threadIdx.x; i < s; i += 32) {
+    rn[i] = rn_all[(int64_t)j * ldnu + i];
+    nu[i] = nu_all[(int64_t)j * ldnu + i];
+  }
+  __syncwarp();
+  if (threadIdx.x != 0) return;
+  bool ok = true;
+  if (fixed) {
+    for (int i = 0; i < min(nev, s); ++i) ok = ok && rn[i] <= tol;
+  } else {
+    for (int i = 0; i < min(nev, s); ++i) {
+      if (rn[i] > tol) { ok = false; break; }
+      const double lam = nu[i] > 0.0 ? sigma + 1.0 / nu[i] : INFINITY;
+      if (lam >= tau) break;
+    }
+  }
+  int k = 0;
+  for (int i = 0; i < s; ++i)
+    if (rn[i] > tol) act_all[(int64_t)j * ldnu + k++] = i;
+  const bool fin = ok || k == 0;
+  if (fin) {
+    done[j] = 1;
+  } else {
+    atomicAdd(notdone, 1);
+  }
+  // FP32 first passes: a subdomain whose largest wanted residual has not
+  // halved in stall_lim iterations (counted after iteration kStallFrom of
+  // the pass), or that is still iterating at iteration kForce64From,
+  // switches to FP64 products and orthogonalisation (notdone[1] counts the
+  // switches)
+  if (best && !fin && !o64[j]) {
+    double r = 0.0;
+    for (int i = 0; i < min(nev, s); ++i) {
+      r = fmax(r, rn[i]);
+      const double lam = nu[i] > 0.0 ? sigma + 1.0 / nu[i] : INFINITY;
+      if (!fixed && lam >= tau) break;
+    }
+    bool sw = false;
+    if (it >= kForce64From) {  // a straggler: FP64 from here on
+      sw = true;
+    } else if (it <= kStallFrom || r < 0.5 * best[j]) {
+      best[j] = r;
+      stall[j] = 0;
+    } else if (++stall[j] >= stall_lim) {
+      sw = true;
+    }
+    if (sw) {
+      o64[j] = 1;
+      ok32[j] = 0;
+      atomicAdd(notdone + 1, 1);
+    }
+  }
+  iters[j] = it;
+  aj[j] = fin ? 0 : k;
+  qj[j] = fin ? 0 : k + spj[j];
+}
+
+// 3. R = BX - KX diag(nu) (active columns only, compacted) to S after X, then
+// the s_p columns of P; one row per thread
+__global__ void __launch_bounds__(kT)
+k_resid_write(const SubDesc* __restrict__ sub, ColRef S, ColRef BX, ColRef KX, ColRef P,
+              const double* __restrict__ nu_all, int ldnu, const int32_t* __restrict__ sj,
+              const int32_t* __restrict__ spj, const int32_t* __restrict__ aj, const int32_t* __restrict__ act_all,
+              const int32_t* __restrict__ done) {
+  const int j = blockIdx.y;
+  if (done[j]) return;
+  const SubDesc d = sub[j];
+  const int a = blockIdx.x * kT + threadIdx.x;
+  if (a >= d.nN) return;
+  const int64_t nn = d.nN;
+  const double* __restrict__ bx = cr_ptr(BX, d, j) + a;
+  const double* __restrict__ kx = cr_ptr(KX, d, j) + a;
+  const double* __restrict__ pc = cr_ptr(P, d, j) + a;
+  double* __restrict__ w0 = cr_ptr(S, d, j) + (int64_t)sj[j] * nn + a;
+  const int k = aj[j], sp = spj[j];
+#pragma unroll 4
+  for (int t = 0; t < k; ++t) {
+    const int c = act_all[(int64_t)j * ldnu + t];
+    w0[t * nn] = bx[c * nn] - nu_all[(int64_t)j * ldnu + c] * kx[c * nn];
+  }
+#pragma unroll 4
+  for (int t = 0; t < sp; ++t) w0[(k + t) * nn] = pc[t * nn];
+}
 
 __global__ void k_sub_nnz(const SubDesc* __restrict__ sub, const int64_t* __restrict__ lrow,
                           int64_t* __restrict__ out, int n) {
@@ -1362,17 +1413,22 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
   if (W3 > kMaxW) return GENEO_ERR_ARG;
   const int64_t rows = h->sumN;
   double *S, *KS, *BS, *P, *Tmp, *G, *Gp, *Tm, *nu, *rn;
+  // row splits of the Gram matrices: about two blocks per SM (18 subdomains of
+  // 38x31x24 elasticity in four splits used 72 of 152 SMs: 812 us per FP64
+  // Gram matrix against 268 us in 16)
+  const int nrs = std::max(kMinRS, std::min(kMaxRS, ceil_div(2 * 152, N)));
   GENEO_TRY(tmp.get(&S, (size_t)rows * W3));
   GENEO_TRY(tmp.get(&KS, (size_t)rows * W3));
   GENEO_TRY(tmp.get(&BS, (size_t)rows * W3));
   GENEO_TRY(tmp.get(&Tmp, (size_t)rows * W3));
   GENEO_TRY(tmp.get(&P, (size_t)rows * s));
   GENEO_TRY(tmp.get(&G, (size_t)N * ldg * ldg));
-  GENEO_TRY(tmp.get(&Gp, (size_t)kRS * N * ldg * ldg));
+  GENEO_TRY(tmp.get(&Gp, (size_t)nrs * N * ldg * ldg));
   GENEO_TRY(tmp.get(&Tm, (size_t)N * ldg * ldg));
   GENEO_TRY(tmp.get(&nu, (size_t)N * s));
   GENEO_TRY(tmp.get(&rn, (size_t)N * s));
-  int32_t *sj, *aj, *qj, *rj, *spj, *done, *iters, *notdone, *nevj;
+  int32_t *sj, *aj, *qj, *rj, *spj, *done, *iters, *notdone, *nevj, *act;
+  GENEO_TRY(tmp.get(&act, (size_t)N * s));
   GENEO_TRY(tmp.get(&nevj, (size_t)N));
   GENEO_TRY(tmp.get(&sj, (size_t)N));
   GENEO_TRY(tmp.get(&aj, (size_t)N));
@@ -1428,12 +1484,15 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
   GENEO_CUDA(allow_smem(k_gemm32<float, double>));
   GENEO_CUDA(allow_smem(k_gemm32<double, double>));
 
+  // threads of the Jacobi kernels: one block per SM at most, so more warps hide
+  // its latencies; with several blocks per SM, 256
+  const int td = N <= 152 ? kTD : kT;
   const bool f32 = h->fp32;
   // Rayleigh-Ritz sweeps in double-single arithmetic in the FP32 mode
   auto rr_launch = [&](const double* Gm, double* Tt, int ld, const int32_t* s_, const int32_t* q_,
                        double* nu_, int ldnu, const int32_t* skip, int wm) {
-    if (f32) k_rr<dsv><<<N, kT, dsm, st>>>(Gm, Tt, ld, s_, q_, nu_, ldnu, skip, wm);
-    else k_rr<double><<<N, kT, dsm, st>>>(Gm, Tt, ld, s_, q_, nu_, ldnu, skip, wm);
+    if (f32) k_rr<dsv><<<N, td, dsm, st>>>(Gm, Tt, ld, s_, q_, nu_, ldnu, skip, wm);
+    else k_rr<double><<<N, td, dsm, st>>>(Gm, Tt, ld, s_, q_, nu_, ldnu, skip, wm);
   };
   // Subdomains whose K_j was factored in FP64 (a weak FP32 pivot: coefficient
   // contrast beyond FP32) also orthogonalise in FP64: their K-norms span
@@ -1595,23 +1654,23 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
           sds = dsk1;
           s64 = dsk2;
         }
-        k_gram_one<double, true><<<dim3(kRS, N), kT, gram1_smem, st>>>(h->dsub, A, B, sym, Gp, ldg, N, sds);
+        k_gram_one<double, true><<<dim3(nrs, N), kT, gram1_smem, st>>>(h->dsub, A, B, sym, Gp, ldg, N, sds);
         note_launch();
         if (s64) {
-          k_gram_one<double, false><<<dim3(kRS, N), kT, gram1_smem, st>>>(h->dsub, A, B, sym, Gp, ldg, N, s64);
+          k_gram_one<double, false><<<dim3(nrs, N), kT, gram1_smem, st>>>(h->dsub, A, B, sym, Gp, ldg, N, s64);
           note_launch();
         }
         one_done = true;
       }
     }
     if (!one_done) {
-      k_gram_one<S><<<dim3(kRS, N), kT, gram1_smem, st>>>(h->dsub, A, B, sym, Gp, ldg, N, skip); note_launch();
+      k_gram_one<S><<<dim3(nrs, N), kT, gram1_smem, st>>>(h->dsub, A, B, sym, Gp, ldg, N, skip); note_launch();
     }
     if (W3 > 64) {
-      k_gram_part<S><<<dim3(kRS, N), kT, gram_smem, st>>>(h->dsub, A, B, sym, Gp, ldg, N, skip, 1);
+      k_gram_part<S><<<dim3(nrs, N), kT, gram_smem, st>>>(h->dsub, A, B, sym, Gp, ldg, N, skip, 1);
       note_launch();
     }
-    k_gram_reduce<S><<<N, kT, 0, st>>>(h->dsub, A, B, sym, Gp, G, ldg, N, skip); note_launch();
+    k_gram_reduce<S><<<N, kT, 0, st>>>(h->dsub, A, B, sym, Gp, G, ldg, N, skip, nrs); note_launch();
     h->prof.end(pr, st);
     GENEO_CUDA(cudaGetLastError());
     return GENEO_OK;
@@ -1759,7 +1818,7 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
     GENEO_TRY(solveK(xoffX, sj, skip));
     spmm(true, false, Xr, KXr, KXr, skip);
     GENEO_TRY(gram(Xr, KXr, 1, skip));
-    { const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st); k_svqb<double><<<N, kT, dsm, st>>>(G, Tm, ldg, sj, nullptr, rj, 1e-14, skip, wcur); note_launch(); h->prof.end(prs, st); }
+    { const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st); k_svqb<double><<<N, td, dsm, st>>>(G, Tm, ldg, sj, nullptr, rj, 1e-14, skip, wcur); note_launch(); h->prof.end(prs, st); }
     GENEO_TRY(gemm(Xr, Tm, 0, nullptr, cref(Tmp, W3, 0, nullptr, 0, rj), 1.0, 0.0, skip));
     k_set_i32<<<ceil_div(N, 128), 128, 0, st>>>(sj, rj, N, skip); note_launch();
     k_copy_cols<double, double><<<gridR, kT, 0, st>>>(h->dsub, cref(Tmp, W3, 0, nullptr, 0, sj), Xr, skip); note_launch();
@@ -1778,9 +1837,14 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
     for (int it = 0; it < o.eig_maxit; ++it, ++total_it) {
       spmm(true, true, Xr, KXr, BXr, done);
       GENEO_CUDA(cudaMemsetAsync(notdone, 0, 2 * sizeof(int32_t), st));
-      k_resid<<<N, kT, 0, st>>>(h->dsub, cref(S, W3, 0, nullptr, 0, nullptr), BXr, KXr, Pr, nu, s, sj,
-                                spj, aj, qj, done, iters, notdone, rn, o.eig_tol, o.tau, o.sigma, nevj,
-                                o.fixed_nev, it, f32 ? best : nullptr, stall, o64, ok32, kStallIts); note_launch();
+      k_resid_norm<<<dim3(s, N), kT, 0, st>>>(h->dsub, BXr, KXr, nu, s, sj, done, rn); note_launch();
+      k_resid_decide<<<N, 32, 0, st>>>(nu, s, sj, spj, aj, qj, act, done, iters, notdone, rn, o.eig_tol, o.tau,
+                                       o.sigma, nevj, o.fixed_nev, it, f32 ? best : nullptr, stall, o64, ok32,
+                                       kStallIts);
+      note_launch();
+      k_resid_write<<<gridR, kT, 0, st>>>(h->dsub, cref(S, W3, 0, nullptr, 0, nullptr), BXr, KXr, Pr, nu, s, sj, spj,
+                                          aj, act, done);
+      note_launch();
       GENEO_CUDA(cudaGetLastError());
       int32_t cnt[2] = {0, 0};
       GENEO_CUDA(cudaMemcpyAsync(cnt, notdone, 2 * sizeof(int32_t), cudaMemcpyDeviceToHost, st));
@@ -1823,7 +1887,7 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
             GENEO_TRY(gram(Qr32, KQr32, 1, s32));
             {
               const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st);
-              k_svqb<float><<<N, kT, dsm32, st>>>(G, Tm, ldg, qj, nullptr, rj, 1e-12, s32, wcur); note_launch();
+              k_svqb<float><<<N, td, dsm32, st>>>(G, Tm, ldg, qj, nullptr, rj, 1e-12, s32, wcur); note_launch();
               h->prof.end(prs, st);
             }
             // Q = Q32 T straight into the FP64 block (no aliasing: T acts on the copy)
@@ -1849,7 +1913,7 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
         {
           const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st);
           if (pass == 0) {
-            k_svqb<double><<<N, kT, dsm, st>>>(G, Tm, ldg, qj, nullptr, rj, 1e-12, sp, wcur);
+            k_svqb<double><<<N, td, dsm, st>>>(G, Tm, ldg, qj, nullptr, rj, 1e-12, sp, wcur);
             note_launch();
           } else {
             // the block is nearly K-orthonormal: Cholesky QR, SVQB where a
@@ -1857,7 +1921,7 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
             k_fill_i32<<<ceil_div(N, 128), 128, 0, st>>>(rj, -1, N); note_launch();
             k_cholqr<<<N, kT, dsm, st>>>(G, Tm, ldg, qj, rj, 1e-12, done, wcur); note_launch();
             k_mark_fallback<<<ceil_div(N, 128), 128, 0, st>>>(rj, done, redo, N); note_launch();
-            k_svqb<double><<<N, kT, dsm, st>>>(G, Tm, ldg, qj, nullptr, rj, 1e-12, redo, wcur); note_launch();
+            k_svqb<double><<<N, td, dsm, st>>>(G, Tm, ldg, qj, nullptr, rj, 1e-12, redo, wcur); note_launch();
             if (f32 && n64 > 0) { k_and_not<<<ceil_div(N, 128), 128, 0, st>>>(redo, o64, N); note_launch(); }
           }
           h->prof.end(prs, st);
