@@ -420,9 +420,14 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
   A* xb = zb + (size_t)ZB * NC;                                     // ZB * NC
   A* mail = xb + (size_t)ZB * NC;                                   // C * B * NC (C > 1)
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  const int ph = lane & (PH - 1), row = wid * RPW + lane / PH;      // this lane's row and its element's column
+  const int ph = lane & (PH - 1), row = wid * RPW + lane / PH;      // this lane's row
   const int p0 = ph * RPW;                                          // first column (row) of 32 of this lane
-  const bool mine = ph < k;                                         // element (row, ph) exists
+  // the column whose sum this lane ends up with, and whether it is the one
+  // lane of its row that stores it
+  constexpr int LC = PH / NC;
+  static_assert(LC >= 1, "a row's lanes must cover the columns");
+  const int col = ph / LC;
+  const bool mine = ph % LC == 0 && col < k;
 
   RS rs;
   rs.full = bars->full;
@@ -466,7 +471,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
   auto fetch = [&](int kk) {
     const int r = kk * B + row;
     if (mine && r < n) {
-      xnext = X[(int64_t)ph * n + r];
+      xnext = X[(int64_t)col * n + r];
       if (Sg) snext = Sg[r];
     }
   };
@@ -495,16 +500,26 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
   uint32_t rstep[RPW];                 // bytes from this lane's first row to the others, down a column
 #pragma unroll
   for (int i = 0; i < RPW; ++i) rstep[i] = (uint32_t)(i * (ld - 1) * (int)sizeof(T));
-  // sums of the PH lanes of a row, element ph of them returned
+  // sums over the PH lanes of a row, of which this lane returns column `col`:
+  // halving exchanges while a lane still holds several columns
   auto reduce = [&](A* acc) -> A {
-    A v = A();
+    int m = NC;
 #pragma unroll
-    for (int c = 0; c < NC; ++c) {
+    for (int o = PH / 2; o > 0; o >>= 1) {
+      if (m > 1) {
+        m >>= 1;
+        const bool up = (ph & o) != 0;
 #pragma unroll
-      for (int o = 1; o < PH; o <<= 1) acc[c] += shfl_xor(acc[c], o);
-      if (NC == 1 || c == ph) v = acc[c];
+        for (int c = 0; c < NC / 2; ++c)
+          if (c < m) {
+            const A give = up ? acc[c] : acc[c + m], keep = up ? acc[c + m] : acc[c];
+            acc[c] = keep + shfl_xor(give, o);
+          }
+      } else {
+        acc[0] += shfl_xor(acc[0], o);
+      }
     }
-    return v;
+    return acc[0];
   };
   // the columns below `seen` that this lane multiplies by (NC > 1: all of them)
   // have arrived
@@ -522,7 +537,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
     if ((j & (C - 1)) != rank) {
       A v[1];
       if (mine && ok)
-        ok = wait_set<1>(v, [&](int) { return win + (size_t)(slot * B + row) * NC + ph; }, [](int) { return true; },
+        ok = wait_set<1>(v, [&](int) { return win + (size_t)(slot * B + row) * NC + col; }, [](int) { return true; },
                          st, d.id, j);
       csync<kThreads>();
     }
@@ -599,7 +614,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
     }
     {
       const A t = reduce(acc);
-      if (mine) zb[row * NC + ph] = in ? rhs - t : A();
+      if (mine) zb[row * NC + col] = in ? rhs - t : A();
     }
     csync<kThreads>();
     // y = M z, M the inverted diagonal block (its lower triangle)
@@ -623,8 +638,8 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
     {
       const A t = reduce(acc);
       const A y = in ? t : A();
-      A* dst = win + (size_t)(rb * B + row) * NC + (NC == 1 ? 0 : ph);
-      const uint32_t off = (uint32_t)((rb * B + row) * NC + (NC == 1 ? 0 : ph)) * (uint32_t)sizeof(A);
+      A* dst = win + (size_t)(rb * B + row) * NC + col;
+      const uint32_t off = (uint32_t)((rb * B + row) * NC + col) * (uint32_t)sizeof(A);
       if constexpr (NC == 1) {  // every lane of the row has y
         for (int q = 1 + ph; q < C; q += PH) st_cluster(map_rank(win_at, (uint32_t)((rank + q) & (C - 1))) + off, y);
       } else if (mine) {
@@ -635,7 +650,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
       rb += C;
       if (rb >= rwb) rb -= rwb;
       csync<kThreads>();
-      if (mine && in) X[(int64_t)ph * n + kb + row] = value(y);
+      if (mine && in) X[(int64_t)col * n + kb + row] = value(y);
     }
   }
   if (C > 1) {  // every solved block has arrived before the ring changes its use
@@ -644,7 +659,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
     {
       A v[1];
       if (mine && ok)
-        ok = wait_set<1>(v, [&](int) { return win + (size_t)((j % rwb) * B + row) * NC + ph; },
+        ok = wait_set<1>(v, [&](int) { return win + (size_t)((j % rwb) * B + row) * NC + col; },
                          [](int) { return true; }, st, d.id, j);
     }
   }
@@ -686,12 +701,12 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
     const T* S1 = R > 1 ? rows_of(1) - (ptrdiff_t)32 * (ld - 1) : S0;
     // z = y - the partial sums of this block
     if (mine) {
-      A* a = ring(0) + row * NC + ph;
+      A* a = ring(0) + row * NC + col;
       A z = yk - *a;
       *a = A();
       if (nsrc > 0) {
         A v[kMaxC - 1];
-        auto at = [&](int q) { return mail + ((size_t)((rank + 1 + q) & (C - 1)) * B + row) * NC + ph; };
+        auto at = [&](int q) { return mail + ((size_t)((rank + 1 + q) & (C - 1)) * B + row) * NC + col; };
         if (ok) ok = wait_set<kMaxC - 1>(v, at, [&](int q) { return q < nsrc; }, st, d.id, -1 - kk);
 #pragma unroll
         for (int q = kMaxC - 2; q >= 0; --q)
@@ -700,7 +715,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
             unset(at(q));
           }
       }
-      zb[row * NC + ph] = row < b ? z : A();
+      zb[row * NC + col] = row < b ? z : A();
     }
     csync<kThreads>();
     const uint32_t sa0 = smem_u32(S0), sa1 = smem_u32(S1) + (uint32_t)(32 * (ld - 1) * (int)sizeof(T));
@@ -748,17 +763,17 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
       column_sum(acc, zb, 0, row, b - 1, false);
     }
     const A x = reduce(acc);
-    if (mine) xb[row * NC + ph] = row < b ? x : A();
+    if (mine) xb[row * NC + col] = row < b ? x : A();
     csync<kThreads>();
     if (kk > 0) {
       // the link of the chain: contribution to block kk - 1
       {
-        A* a = ring(1) + row * NC + ph;
+        A* a = ring(1) + row * NC + col;
         const A old = mine ? *a : A();
         column_sum(acc, xb, -B, 0, min(b - 1, row - B + w), B >= 32 && b == B && w >= 2 * B - 1);
         const A s = reduce(acc) + old;
         if (mine) {
-          if (C > 1) send(1, row, ph, s);
+          if (C > 1) send(1, row, col, s);
           *a = C > 1 ? A() : s;
         }
       }
@@ -822,8 +837,8 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
     }
     csync<kThreads>();
     if (mine && row < b) {
-      if constexpr (std::is_same_v<A, float>) X[(int64_t)ph * n + kb + row] = f2d_bits(x * sc);
-      else X[(int64_t)ph * n + kb + row] = value(x);
+      if constexpr (std::is_same_v<A, float>) X[(int64_t)col * n + kb + row] = f2d_bits(x * sc);
+      else X[(int64_t)col * n + kb + row] = value(x);
     }
   }
   if (C > 1) cluster_sync();  // no block leaves while another may still store into it
