@@ -286,7 +286,8 @@ __device__ __forceinline__ A factor_value(T x) {
 // acc[c] += sum L(e) X(e, c) over I entries of each of R groups of 32 (entry i
 // of group q at index 32 q + i): L(e) = at(e), rows X(e, .) of NC values one
 // after another at x, entries skipped where !in(e)
-template <int I, int R, int NC, typename T, typename A, typename At, typename In>
+// (of the NC columns the first KC are formed)
+template <int I, int R, int NC, int KC, typename T, typename A, typename At, typename In>
 __device__ __forceinline__ void madd(A* acc, const A* x, At at, In in) {
   if constexpr (NC == 1) {
     constexpr int N = I * R, W = N >= 8 && sizeof(T) == 4 ? 4 : N >= 4 ? 2 : 1;   // chains
@@ -318,7 +319,7 @@ __device__ __forceinline__ void madd(A* acc, const A* x, At at, In in) {
         A xv[NC];
         load_n<NC>(x + i * NC, xv);
 #pragma unroll
-        for (int c = 0; c < NC; ++c) acc[c] += a * xv[c];
+        for (int c = 0; c < KC; ++c) acc[c] += a * xv[c];
       }
     }
   }
@@ -382,11 +383,11 @@ __device__ __forceinline__ T chains(const T (&a)[W]) {
 // warp's 32 band addresses fall in distinct banks (ld - 1 is odd), and the
 // row's sum ends in two to five shuffles instead of a block barrier.
 // ---------------------------------------------------------------------------
-template <typename T, typename A, int NC, int B>
+template <typename T, typename A, int NC, int B, int KC>
 __global__ void __launch_bounds__(32 * sweep_warps<NC, B>() + 32, NC == 1 && sizeof(T) == 4 && B < 64 ? 2 : 1)
 k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* __restrict__ xbase,
         const int64_t* __restrict__ xoff, int col0, int kcap, const int32_t* __restrict__ nrhs_dev,
-        const int32_t* __restrict__ skip, int C, int nslot, int rwb, DevStatus* st) {
+        const int32_t* __restrict__ skip, int cpp, int C, int nslot, int rwb, DevStatus* st) {
   using RS = RowStream<T, B>;
   constexpr int SR = RS::SR, HB = RS::HB;
   constexpr int NW = sweep_warps<NC, B>(), kThreads = 32 * NW;
@@ -402,8 +403,8 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
   const BandDesc d = descs[mat];
   const int mi = d.id >= 0 ? d.id : mat;
   if (skip && skip[mi]) return;
-  col0 += (int)blockIdx.y * NC;
-  int k = min(kcap - (int)blockIdx.y * NC, NC);
+  col0 += (int)blockIdx.y * cpp;       // cpp <= KC <= NC columns per block
+  int k = min(kcap - (int)blockIdx.y * cpp, cpp);
   if (nrhs_dev) k = min(k, nrhs_dev[mi] - col0);
   if (k <= 0 || d.n <= 0) return;  // the same decision in every block of the cluster
   const int n = d.n, w = d.w, ld = d.ld;
@@ -599,10 +600,10 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
                             [&](int e) { return la + (uint32_t)((c0 + 32 * (e / RPW) + e % RPW) * (int)sizeof(T)); },
                             [](T l, int) { return l; });
           else
-            madd<RPW, R, NC, T>(acc, yw, [&](int i) { return Lc[i]; }, [](int) { return true; });
+            madd<RPW, R, NC, KC, T>(acc, yw, [&](int i) { return Lc[i]; }, [](int) { return true; });
         } else
         {
-          madd<RPW, R, NC, T>(acc, yw, [&](int i) { return Lc[i]; },
+          madd<RPW, R, NC, KC, T>(acc, yw, [&](int i) { return Lc[i]; },
                               [&](int i) { return c0 + i >= cmin && c0 + i < cmax; });
         }
       }
@@ -632,7 +633,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
                       [&](T l, int e) { return masked(l, mf[e]); });
       acc[0] = chains(a2);
     } else if (in) {
-      madd<RPW, R, NC, T>(acc, zb + (size_t)p0 * NC, [&](int i) { return Lr[kb + i]; },
+      madd<RPW, R, NC, KC, T>(acc, zb + (size_t)p0 * NC, [&](int i) { return Lr[kb + i]; },
                           [&](int i) { return p0 + i <= row; });
     }
     {
@@ -738,9 +739,9 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
           dot_lds<RPW, R>(a2, smem_u32(x + p0), [&](int e) { return row_at(e, shift); }, [](T l, int) { return l; });
           acc[0] = chains(a2);
         } else
-          madd<RPW, R, NC, T>(acc, x + (size_t)p0 * NC, at, [](int) { return true; });
+          madd<RPW, R, NC, KC, T>(acc, x + (size_t)p0 * NC, at, [](int) { return true; });
       } else
-        madd<RPW, R, NC, T>(acc, x + (size_t)p0 * NC, at,
+        madd<RPW, R, NC, KC, T>(acc, x + (size_t)p0 * NC, at,
                             [&](int i) { return p0 + i >= first && p0 + i <= last; });
     };
     // x = M^T z: column `row` of the inverted block
@@ -808,16 +809,16 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
                 const int part = t0 / SR;
                 const T* S = rs.slot(part) - (ptrdiff_t)part * SR * ld + (cc - kb + w) + (ptrdiff_t)t0 * (ld - 1);
                 if (tmx >= t0 + TU - 1)
-                  madd<TU, 1, NC, T>(a2, xb + (size_t)t0 * NC, [&](int i) { return S[(ptrdiff_t)i * (ld - 1)]; },
+                  madd<TU, 1, NC, KC, T>(a2, xb + (size_t)t0 * NC, [&](int i) { return S[(ptrdiff_t)i * (ld - 1)]; },
                                      [](int) { return true; });
                 else
-                  madd<TU, 1, NC, T>(a2, xb + (size_t)t0 * NC, [&](int i) { return S[(ptrdiff_t)i * (ld - 1)]; },
+                  madd<TU, 1, NC, KC, T>(a2, xb + (size_t)t0 * NC, [&](int i) { return S[(ptrdiff_t)i * (ld - 1)]; },
                                      [&](int i) { return t0 + i <= tmx; });
               }
               const int jb = cc / B;
               A* a = ring(kk - jb) + (size_t)(cc - jb * B) * NC;
 #pragma unroll
-              for (int c = 0; c < NC; ++c) a[c] += a2[c];
+              for (int c = 0; c < KC; ++c) a[c] += a2[c];
             }
           }
         }
@@ -847,21 +848,30 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
 // ---------------------------------------------------------------------------
 // Tensor-core sweep for several right-hand sides (FP32 factors): the same
 // chain with every product an m16n8k8 TF32 MMA (three passes: hi*hi + hi*lo +
-// lo*hi; PASSES = 1: one pass off the diagonal blocks).  Eight warps: B / 16
-// row tiles x KP k-parts.  The k index of an MMA is permuted so that a
+// lo*hi; PASSES = 1: one pass off the diagonal blocks).  B / 16 row
+// tiles x KP k-parts of warps.  The k index of an MMA is permuted so that a
 // quad's four lanes read columns (backward: rows) CGS apart: with the band's
 // odd address stride ld - 1 that makes the 32 fragment addresses distinct
 // banks, and odd column strides of win and zb do the same for B.
 // ---------------------------------------------------------------------------
+// Sixteen warps: a link is a chain of short steps (shared loads, splits, a few
+// MMAs, a barrier), and twice the warps halve each warp's share of all but the
+// barrier (elasticity 38^3, half width about 500, 24 columns: the 56 sweeps of
+// the eigensolver 81 ms with eight warps, 54 ms with sixteen).
+template <int B>
+__host__ __device__ constexpr int mma_warps() {
+  return 16;
+}
 template <int B, int NT, int PASSES>
-__global__ void __launch_bounds__(kThreads + 32, 1)
+__global__ void __launch_bounds__(32 * mma_warps<B>() + 32, 1)
 k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, double* __restrict__ xbase,
             const int64_t* __restrict__ xoff, int col0, int kcap, const int32_t* __restrict__ nrhs_dev,
             const int32_t* __restrict__ skip, int C, int nslot, int rwb, DevStatus* st) {
   using RS = RowStream<float, B>;
   constexpr int SR = RS::SR;
   constexpr int NC = 8 * NT;
-  constexpr int MT = B / 16, KP = 8 / MT;       // row tiles, k-parts
+  constexpr int NW = mma_warps<B>(), kThreads = 32 * NW;
+  constexpr int MT = B / 16, KP = NW / MT;      // row tiles, k-parts
   constexpr int ST = B / 8;                     // k-steps per block
   constexpr int SPW = ST / KP > 0 ? ST / KP : 1;  // k-steps per warp and block
   constexpr int KPB = ST / SPW;                 // k-parts that share a block
@@ -915,7 +925,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
   if (tid == 0) {
     for (int s = 0; s < nslot; ++s) {
       mbar_init(&bars->full[s], 1);
-      mbar_init(&bars->empty[s], kThreads / 32);
+      mbar_init(&bars->empty[s], NW);
     }
     fence_barrier_init();
   }
@@ -1002,7 +1012,9 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
   // k positions of an MMA: a quad's lanes are 8 apart (4 in 16-row blocks), the
   // two halves of k next to each other: position kl + 2 i + half of k-step i
   const int gkp = kp / KPB;
-  const int kl = B == 64 ? 32 * kp + 8 * tg : B == 32 ? 8 * tg + 2 * kp : 4 * tg + 2 * (kp % KPB);
+  const int s0 = (kp % KPB) * SPW;               // this warp's first k-step in a block
+  const int kq = B < 32 ? 0 : s0 >> 2, km = 2 * (B < 32 ? s0 : s0 & 3);   // its 32-row group and place there
+  const int kl = 32 * kq + (B < 32 ? 4 : 8) * tg + km;
   const uint32_t win_at = smem_u32(win), zb_at = smem_u32(zb) + (uint32_t)((g * ZS + kl) * 4);
   const uint32_t ys8 = (uint32_t)(8 * YS * 4), zs8 = (uint32_t)(8 * ZS * 4);
   const uint32_t row8 = (uint32_t)(8 * (ld - 1) * 4);
@@ -1040,7 +1052,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
           if (ok)
             ok = wait_set<E>(v, [&](int e) { return win + (size_t)(ph + e * P) * YS + rb * B + row; },
                              [&](int e) { return ph + e * P < k; }, st, d.id, j);
-          csync();
+          csync<kThreads>();
         }
         ready = j + 1;
       }
@@ -1067,13 +1079,13 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
       rb = rb + 1 == rwb ? 0 : rb + 1;
     }
     put_red();
-    csync();
+    csync<kThreads>();
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int c = ph + e * P;
       if (c < k) zb[c * ZS + row] = row < b ? d2f_bits(xc[e]) * sc - red_sum(c) : 0.f;
     }
-    csync();
+    csync<kThreads>();
     // y = M z
     clear();
     if (gkp == 0) {
@@ -1093,7 +1105,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
       }
     }
     put_red();
-    csync();
+    csync<kThreads>();
     {
 #pragma unroll
       for (int e = 0; e < E; ++e) {
@@ -1111,7 +1123,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
     rs.release();
     rbk += C;
     if (rbk >= rwb) rbk -= rwb;
-    csync();
+    csync<kThreads>();
   }
   if (C > 1) {
     const int last = own > 0 ? rank + C * (own - 1) : -1;
@@ -1123,13 +1135,13 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
                          [&](int e) { return ph + e * P < k; }, st, d.id, j);
     }
   }
-  csync();
+  csync<kThreads>();
 
   // ------------------------------------------------------------ backward
   for (int i = tid; i < NC * YS; i += kThreads) win[i] = 0.f;
   const uint32_t mail_at = smem_u32(mail) + (uint32_t)(rank * NC * B) * 4u;
   if (own > 0) fetch(rank + C * (own - 1));
-  csync();
+  csync<kThreads>();
   for (int v = own; v < 2 * own; ++v) {
     const int kk = rank + C * (2 * own - 1 - v), kb = kk * B;
     const int b = min(B, n - kb);
@@ -1164,7 +1176,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
         zb[c * ZS + row] = row < b ? d2f_bits(xc[e]) - s : 0.f;
       }
     }
-    csync();
+    csync<kThreads>();
     // x = M^T z: A(m = column, k = row t) = M(t, m)
     clear();
     const int ca = 16 * mt + g, cb = ca + 8;
@@ -1176,8 +1188,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
     for (int q = 0; q < (B > 32 ? 2 : 1); ++q)
       sq[q] = rs.slot_at(q) + (uint32_t)((CL * tg * ld - 32 * q - CL * tg + w) * 4);
     // this warp's k-steps: rows kl + 2 i + half
-    const uint32_t sk = B == 64 ? (kp ? sq[B > 32 ? 1 : 0] : sq[0])
-                                : sq[0] + (uint32_t)(2 * (kp % KPB) * (ld - 1) * 4);
+    const uint32_t sk = sq[B > 32 ? kq : 0] + (uint32_t)(km * (ld - 1) * 4);
     if (gkp == 0) {
 #pragma unroll
       for (int i = 0; i < SPW; ++i) {
@@ -1196,7 +1207,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
       }
     }
     put_red();
-    csync();
+    csync<kThreads>();
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int c = ph + e * P;
@@ -1206,7 +1217,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
         if (row < b) X[(int64_t)c * n + kb + row] = f2d_bits(xx * sc);
       }
     }
-    csync();
+    csync<kThreads>();
     if (kk > 0) {
       // the link of the chain: contribution to block kk - 1
       clear();
@@ -1233,7 +1244,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
         }
       }
       put_red();
-      csync();
+      csync<kThreads>();
       {
         const uint32_t to = (uint32_t)((kk - 1) & (C - 1));
 #pragma unroll
@@ -1301,7 +1312,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
           }
       }
       rs.release();
-      csync();
+      csync<kThreads>();
       if (C > 2) {
         for (int i = tid; i < (C - 2) * B * k; i += kThreads) {
           const int r = i % B, c = (i / B) % k, jb = kk - 2 - i / (B * k);
@@ -1312,7 +1323,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
           const uint32_t to = (uint32_t)(jb & (C - 1));
           st_cluster(map_rank(mail_at, to) + (uint32_t)(c * B + r) * 4u, s);
         }
-        csync();
+        csync<kThreads>();
       }
     }
   }
@@ -1343,6 +1354,7 @@ k_band_blkinv(T* __restrict__ base, const BandDesc* __restrict__ descs) {
   A* Rs = Xs + B * B;                       // reciprocal pivots
   T* Ls = reinterpret_cast<T*>(Rs + B);     // B x B
   const int nt = blockDim.x, c = threadIdx.x;
+#pragma unroll 8
   for (int i = c; i < B * B; i += nt) {
     const int r = i / B, cc = i % B;
     Ls[i] = (r < b && cc <= r) ? L[(int64_t)r * ld + cc - r] : T(0);
@@ -1350,9 +1362,10 @@ k_band_blkinv(T* __restrict__ base, const BandDesc* __restrict__ descs) {
   if (c < b) Rs[c] = recip_arith<A>(L[(int64_t)c * ld]);
   __syncthreads();
   if (c < B) {
-    for (int r = 0; r < b; ++r) {
+    const int w0 = c & ~31;   // this warp's columns are zero above row w0
+    for (int r = w0; r < b; ++r) {
       A s0 = A(), s1 = A();
-      int t = 0;
+      int t = w0;
       for (; t + 1 < r; t += 2) {
         s0 += factor_value<A>(Ls[r * B + t]) * Xs[t * B + c];
         s1 += factor_value<A>(Ls[r * B + t + 1]) * Xs[(t + 1) * B + c];
@@ -1378,7 +1391,7 @@ size_t sweep_smem(int w, int C, int nslot) {
 }
 template <int B, int NT>
 size_t mma_smem(int w, int C, int nslot) {
-  const size_t SR = B < 32 ? B : 32, NC = 8 * NT, KP = 8 / (B / 16);
+  const size_t SR = B < 32 ? B : 32, NC = 8 * NT, KP = mma_warps<B>() / (B / 16);
   return sizeof(Bars) + sizeof(float) * (nslot * SR * band_ld(w) + NC * ((size_t)ring_blocks(w, B, C) * B + 1) +
                                          KP * NC * (B + 4) + NC * (B + 1) + (C > 1 ? (size_t)C * NC * B : 0));
 }
@@ -1433,8 +1446,8 @@ int fit_slots(F bytes, int need, int want) {
   return 0;
 }
 
-template <typename T, typename A, int NC, int B>
-geneo_status_t run_sweep(const T* base, const SweepArgs& a, int C, int parts) {
+template <typename T, typename A, int NC, int B, int KC = NC>
+geneo_status_t run_sweep(const T* base, const SweepArgs& a, int C, int parts, int cpp = KC) {
   constexpr int HB = RowStream<T, B>::HB;
   const int want = a.slots;
   int nslot = 0;
@@ -1445,8 +1458,8 @@ geneo_status_t run_sweep(const T* base, const SweepArgs& a, int C, int parts) {
     if (nslot > 0 || C == 1) break;
   }
   if (nslot == 0) return GENEO_ERR_ARG;
-  return launch_cluster(k_sweep<T, A, NC, B>, 32 * sweep_warps<NC, B>() + 32, dim3(a.count * C, parts), C, sweep_smem<T, A, NC, B>(a.w, C, nslot),
-                        a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev, a.skip, C, nslot,
+  return launch_cluster(k_sweep<T, A, NC, B, KC>, 32 * sweep_warps<NC, B>() + 32, dim3(a.count * C, parts), C, sweep_smem<T, A, NC, B>(a.w, C, nslot),
+                        a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev, a.skip, cpp, C, nslot,
                         ring_blocks(a.w, B, C), a.st);
 }
 
@@ -1463,28 +1476,31 @@ geneo_status_t run_mma(const float* base, const SweepArgs& a, int C, int parts, 
   const dim3 grid(a.count * C, parts);
   const int rwb = ring_blocks(a.w, B, C);
   if (passes == 1)
-    return launch_cluster(k_sweep_mma<B, NT, 1>, kThreads + 32, grid, C, smem, a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev,
+    return launch_cluster(k_sweep_mma<B, NT, 1>, 32 * mma_warps<B>() + 32, grid, C, smem, a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev,
                           a.skip, C, nslot, rwb, a.st);
-  return launch_cluster(k_sweep_mma<B, NT, 3>, kThreads + 32, grid, C, smem, a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev,
+  return launch_cluster(k_sweep_mma<B, NT, 3>, 32 * mma_warps<B>() + 32, grid, C, smem, a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev,
                         a.skip, C, nslot, rwb, a.st);
 }
 
 }  // namespace
 
-// Rows per block of the sweeps for a band of half width w (w >= 15), by what
-// fits in shared memory with room to stream ahead; 0: too wide, the factor
-// stays as it is for the streamed kernels of band.cu.
+// Rows per block of the sweeps for a band of half width w (w >= 15): the most
+// whose rows fit in shared memory at once beside the windows.  Room to stream
+// ahead counts for less than longer links (half width 660, 27 matrices, C = 4:
+// 466 us with 32 rows and a second block streaming in, 283 us with 64 and none;
+// the other blocks of the cluster work while the rows arrive).  0: too wide,
+// the factor stays as it is for the streamed kernels of band.cu.
 int sweep_block(int w, bool f64) {
   if (f64) {
-    if (w >= 31 && sweep_smem<double, double, 8, 32>(w, 1, 3) <= kSmemMax) return 32;
-    if (sweep_smem<double, double, 8, 16>(w, 1, 2) <= kSmemMax) return 16;
-    if (sweep_smem<double, double, 4, 8>(w, 1, 2) <= kSmemMax) return 8;
+    if (w >= 31 && sweep_smem<double, double, 8, 32>(w, 1, 2) <= kSmemMax) return 32;
+    if (sweep_smem<double, double, 8, 16>(w, 1, 1) <= kSmemMax) return 16;
+    if (sweep_smem<double, double, 4, 8>(w, 1, 1) <= kSmemMax) return 8;
     return 0;
   }
-  if (w >= 63 && mma_smem<64, 1>(w, 1, 3) <= kSmemMax) return 64;
-  if (w >= 31 && mma_smem<32, 1>(w, 1, 2) <= kSmemMax) return 32;
-  if (mma_smem<16, 1>(w, 1, 2) <= kSmemMax) return 16;
-  if (sweep_smem<float, float, 4, 8>(w, 1, 2) <= kSmemMax) return 8;
+  if (w >= 63 && mma_smem<64, 1>(w, 1, 2) <= kSmemMax) return 64;
+  if (w >= 31 && mma_smem<32, 1>(w, 1, 1) <= kSmemMax) return 32;
+  if (mma_smem<16, 1>(w, 1, 1) <= kSmemMax) return 16;
+  if (sweep_smem<float, float, 4, 8>(w, 1, 1) <= kSmemMax) return 8;
   return 0;
 }
 
@@ -1520,7 +1536,7 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
   // one column 1, 0.57, 0.35, 0.36; MMA 1, 0.54, 0.44; FP64 1, 0.54, 0.45); a
   // block is solved from the ceil(w / blk) before it, which bounds what C can
   // share, and each thread block has at least two
-  auto clusters = [&](int units) {
+  auto clusters = [&](int units, double* len = nullptr) {
     const double rel[4] = {1.0, 0.56, 0.40, 0.38};
     int best = 1;
     double least = 1e300;
@@ -1532,6 +1548,7 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
         best = C;
       }
     }
+    if (len) *len = least;
     return best;
   };
   if (nrhs == 1) {
@@ -1572,19 +1589,41 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
     return run_sweep<T, T, 4, 8>(base, a, clusters(parts), parts);
   } else {
     using A = std::conditional_t<DS, dsv, double>;
-    // eight columns per block, four when that leaves SMs idle or eight do not fit
-    const int p8 = (nrhs + 7) / 8, p4 = (nrhs + 3) / 4;
+    // the columns cut into parts of cpp per block (kernels for 3, 4 and 8); the
+    // FP64 and double-single pipes are full with one block per SM, so the time
+    // is the waves times the columns formed times the sweep's relative length
+    // (27 FP64 bands of order 9261, half width 463, 11 columns: 12.2 ms in three
+    // parts of 4, 11.3 in two of 6 on clusters of 2)
     const bool fit8 = blk != 8 || sweep_smem<double, A, 8, 8>(max_w, 1, 1) <= kSmemMax;
-    const bool four = nrhs <= 4 || !fit8 || (int64_t)live * p8 * 2 <= sms;
-    const int parts = four ? p4 : p8, C = clusters(parts);
-    if (four) {
-      if (blk == 32) return run_sweep<T, A, 4, 32>(base, a, C, parts);
-      if (blk == 16) return run_sweep<T, A, 4, 16>(base, a, C, parts);
-      return run_sweep<T, A, 4, 8>(base, a, C, parts);
+    const int most = fit8 ? 8 : 4;
+    int parts = (nrhs + most - 1) / most, C = 1;
+    double least = 1e300;
+    for (int p = parts; p <= nrhs; ++p) {
+      const int cpp = (nrhs + p - 1) / p;
+      if (p > parts && cpp == (nrhs + p - 2) / (p - 1)) continue;   // no narrower than with one part less
+      double len;
+      const int c = clusters(p, &len);
+      len *= cpp <= 3 ? 3.7 : cpp <= 4 ? 4.7 : 8.7;   // and the latency of a link
+      if (len < least - 1e-9) {
+        least = len;
+        parts = p;
+        C = c;
+      }
+      if (cpp <= 3) break;
     }
-    if (blk == 32) return run_sweep<T, A, 8, 32>(base, a, C, parts);
-    if (blk == 16) return run_sweep<T, A, 8, 16>(base, a, C, parts);
-    return run_sweep<T, A, 8, 8>(base, a, C, parts);
+    const int cpp = (nrhs + parts - 1) / parts;
+    if (cpp <= 3) {
+      if (blk == 32) return run_sweep<T, A, 4, 32, 3>(base, a, C, parts, cpp);
+      if (blk == 16) return run_sweep<T, A, 4, 16, 3>(base, a, C, parts, cpp);
+    }
+    if (cpp <= 4) {
+      if (blk == 32) return run_sweep<T, A, 4, 32>(base, a, C, parts, cpp);
+      if (blk == 16) return run_sweep<T, A, 4, 16>(base, a, C, parts, cpp);
+      return run_sweep<T, A, 4, 8>(base, a, C, parts, cpp);
+    }
+    if (blk == 32) return run_sweep<T, A, 8, 32>(base, a, C, parts, cpp);
+    if (blk == 16) return run_sweep<T, A, 8, 16>(base, a, C, parts, cpp);
+    return run_sweep<T, A, 8, 8>(base, a, C, parts, cpp);
   }
 }
 
