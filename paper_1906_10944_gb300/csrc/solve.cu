@@ -30,6 +30,67 @@ constexpr int kRedBlocks = 1024;
 constexpr int kNoAllocMaxIt = 4095;
 constexpr int kNoAllocScalars = 16;
 
+// scalars: 0 rz, 1 alpha, 2 beta, 3 rr, 4 pq, 5 bb, 6 flag; kTicket: blocks
+// done of the running reduction (an unsigned)
+constexpr int kTicket = 14;
+__device__ void finish_step(double s, double* __restrict__ scal, int what, double* __restrict__ hist_a,
+                            double* __restrict__ hist_b, int it) {
+  if (what == 0) {            // rz0
+    scal[0] = s;
+    if (!(s > 0.0)) scal[6] = 1.0;
+  } else if (what == 1) {     // alpha = rz / pq
+    scal[4] = s;
+    if (!(s > 0.0)) { scal[6] = 1.0; scal[1] = 0.0; }
+    else scal[1] = scal[0] / s;
+    hist_a[it] = scal[1];
+  } else if (what == 2) {     // rr
+    scal[3] = s;
+  } else if (what == 3) {     // beta = rz_new / rz
+    if (!(s > 0.0)) scal[6] = 1.0;
+    scal[2] = scal[0] > 0.0 ? s / scal[0] : 0.0;
+    scal[0] = s;
+    hist_b[it] = scal[2];
+  } else if (what == 4) {     // bb
+    scal[5] = s;
+  } else if (what == 5) {     // ||b - A x||^2
+    scal[7] = s;
+  }
+}
+
+// What a kernel's inner product is for (part = NULL: none).
+struct Dot {
+  double *part, *scal;
+  int what;
+  double *hist_a, *hist_b;
+  int it;
+};
+
+// The end of an inner product, called by every thread with its part: the block
+// sums go to dot.part, and the last block to finish adds them up in a fixed
+// order and takes the scalar step, so no kernel of its own waits for the
+// partials (3.5 us each, three per iteration).
+__device__ void dot_end(double v, const Dot& dot) {
+  __shared__ double red[kT / 32];
+  __shared__ bool last;
+  v = block_sum(v, red);
+  unsigned* ticket = reinterpret_cast<unsigned*>(dot.scal + kTicket);
+  if (threadIdx.x == 0) {
+    dot.part[blockIdx.x] = v;
+    __threadfence();
+    last = atomicAdd(ticket, 1u) == gridDim.x - 1;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double s = 0.0;
+  for (int i = threadIdx.x; i < (int)gridDim.x; i += blockDim.x) s += __ldcg(dot.part + i);
+  s = block_sum(s, red);
+  if (threadIdx.x == 0) {
+    *ticket = 0u;
+    finish_step(s, dot.scal, dot.what, dot.hist_a, dot.hist_b, dot.it);
+  }
+}
+
 // u_j = R_j r and c_j = Z_j^T r (the restriction to the coarse space) in one
 // pass over r: each gathered r value serves u and up to kRm coarse products,
 // and the kRm sums share one block reduction (fixed order).
@@ -75,16 +136,66 @@ k_restrict(const SubDesc* __restrict__ sub, const int32_t* __restrict__ Dlist, c
   }
 }
 
+// The same for batches that leave SMs idle with one block per subdomain: block
+// (j, y) gathers a share of u_j for y < gy and forms four coarse products
+// otherwise (elasticity 32^3, 27 subdomains with up to 30 vectors: 91 us in
+// one block each)
+constexpr int kRq = 4;
+__global__ void __launch_bounds__(kT)
+k_restrict_wide(const SubDesc* __restrict__ sub, const int32_t* __restrict__ Dlist, const double* __restrict__ r,
+                const double* __restrict__ Z, double* __restrict__ u, double* __restrict__ c, int gy) {
+  const int j = blockIdx.x, y = blockIdx.y;
+  const SubDesc d = sub[j];
+  const int32_t* Dj = Dlist + d.offN;
+  if (y < gy) {
+    double* uj = u + d.offN;
+    for (int i = y * kT + threadIdx.x; i < d.nD; i += gy * kT) uj[i] = r[Dj[i]];
+    return;
+  }
+  const int k0 = (y - gy) * kRq, km = min(kRq, d.m - k0);
+  if (km <= 0) return;
+  __shared__ double red[kT / 32][kRq];
+  const double* zj = Z + d.offZ + (int64_t)k0 * d.nD;
+  double acc[kRq];
+#pragma unroll
+  for (int k = 0; k < kRq; ++k) acc[k] = 0.0;
+#pragma unroll 2
+  for (int i = threadIdx.x; i < d.nD; i += kT) {
+    const double rv = r[Dj[i]];
+#pragma unroll
+    for (int k = 0; k < kRq; ++k)
+      if (k < km) acc[k] += zj[(int64_t)k * d.nD + i] * rv;
+  }
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+#pragma unroll
+  for (int k = 0; k < kRq; ++k) {
+    const double v = warp_sum(acc[k]);
+    if (lane == 0) red[wid][k] = v;
+  }
+  __syncthreads();
+  if (threadIdx.x < km) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kT / 32; ++w) t += red[w][threadIdx.x];
+    c[d.offH + k0 + threadIdx.x] = t;
+  }
+}
+
+// z = the sum over the subdomains of their local and coarse parts; with
+// dot.part also r.z
 __global__ void __launch_bounds__(kT)
 k_prolong(int64_t n, const uint8_t* __restrict__ dir, const double* __restrict__ r,
           const int64_t* __restrict__ invD_ptr, const int32_t* __restrict__ invD_sub,
           const int32_t* __restrict__ invD_loc, const SubDesc* __restrict__ sub,
           const double* __restrict__ u, const double* __restrict__ Z, const double* __restrict__ y,
-          double* __restrict__ z) {
+          double* __restrict__ z, Dot dot) {
+  double rz = 0.0;
   for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < n;
        k += (int64_t)gridDim.x * blockDim.x) {
+    const double rk = r[k];
     if (dir[k]) {
-      z[k] = r[k];
+      z[k] = rk;
+      rz += rk * rk;
       continue;
     }
     double acc = 0.0;
@@ -97,18 +208,18 @@ k_prolong(int64_t n, const uint8_t* __restrict__ dir, const double* __restrict__
       acc += v;
     }
     z[k] = acc;
+    rz += rk * acc;
   }
+  if (dot.part) dot_end(rz, dot);
 }
 
 __global__ void __launch_bounds__(kT)
-k_dot(int64_t n, const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ part) {
-  __shared__ double red[kT / 32];
+k_dot(int64_t n, const double* __restrict__ a, const double* __restrict__ b, Dot dot) {
   double s = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x)
     s += a[i] * b[i];
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  dot_end(s, dot);
 }
 
 // ---------------------------------------------------------------------------
@@ -203,9 +314,7 @@ __device__ __forceinline__ double sell_row(const int64_t* __restrict__ off, cons
 // q = A p; partial sums of p.q per block
 __global__ void __launch_bounds__(kT)
 k_spmv_sell_dot(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ scol,
-                const double* __restrict__ sval, const double* __restrict__ p, double* __restrict__ q,
-                double* __restrict__ part) {
-  __shared__ double red[kT / 32];
+                const double* __restrict__ sval, const double* __restrict__ p, double* __restrict__ q, Dot dot) {
   const int l = threadIdx.x & 31;
   const int64_t nsl = (n + 31) / 32;
   double dsum = 0.0;
@@ -224,16 +333,14 @@ k_spmv_sell_dot(int64_t n, const int64_t* __restrict__ off, const int32_t* __res
       dsum += v[1] * p[r2];
     }
   }
-  dsum = block_sum(dsum, red);
-  if (threadIdx.x == 0) part[blockIdx.x] = dsum;
+  dot_end(dsum, dot);
 }
 
 // r = b - A x; partial sums of r.r per block
 __global__ void __launch_bounds__(kT)
 k_true_resid_sell(int64_t n, const int64_t* __restrict__ off, const int32_t* __restrict__ scol,
                   const double* __restrict__ sval, const double* __restrict__ x, const double* __restrict__ b,
-                  double* __restrict__ r, double* __restrict__ part) {
-  __shared__ double red[kT / 32];
+                  double* __restrict__ r, Dot dot) {
   const int l = threadIdx.x & 31;
   const int64_t nsl = (n + 31) / 32;
   double rsum = 0.0;
@@ -247,8 +354,7 @@ k_true_resid_sell(int64_t n, const int64_t* __restrict__ off, const int32_t* __r
       rsum += ri * ri;
     }
   }
-  rsum = block_sum(rsum, red);
-  if (threadIdx.x == 0) part[blockIdx.x] = rsum;
+  dot_end(rsum, dot);
 }
 
 // y = X c with X = A_H^{-1} (symmetric; row i read as column i, contiguous):
@@ -265,42 +371,10 @@ k_coarse_gemv(const double* __restrict__ X, int dim, const double* __restrict__ 
   }
 }
 
-// scalars: 0 rz, 1 alpha, 2 beta, 3 rr, 4 pq, 5 bb, 6 flag
-__global__ void k_finish(const double* __restrict__ part, int nb, double* __restrict__ scal, int what,
-                         double* __restrict__ hist_a, double* __restrict__ hist_b, int it) {
-  __shared__ double red[kT / 32];
-  double s = 0.0;
-  for (int i = threadIdx.x; i < nb; i += blockDim.x) s += part[i];
-  s = block_sum(s, red);
-  if (threadIdx.x != 0) return;
-  if (what == 0) {            // rz0
-    scal[0] = s;
-    if (!(s > 0.0)) scal[6] = 1.0;
-  } else if (what == 1) {     // alpha = rz / pq
-    scal[4] = s;
-    if (!(s > 0.0)) { scal[6] = 1.0; scal[1] = 0.0; }
-    else scal[1] = scal[0] / s;
-    hist_a[it] = scal[1];
-  } else if (what == 2) {     // rr
-    scal[3] = s;
-  } else if (what == 3) {     // beta = rz_new / rz
-    if (!(s > 0.0)) scal[6] = 1.0;
-    scal[2] = scal[0] > 0.0 ? s / scal[0] : 0.0;
-    scal[0] = s;
-    hist_b[it] = scal[2];
-  } else if (what == 4) {     // bb
-    scal[5] = s;
-  } else if (what == 5) {     // ||b - A x||^2
-    scal[7] = s;
-  }
-}
-
 __global__ void __launch_bounds__(kT)
-k_update_xr(int64_t n, const double* __restrict__ scal, const double* __restrict__ p,
-            const double* __restrict__ q, double* __restrict__ x, double* __restrict__ r,
-            double* __restrict__ part) {
-  __shared__ double red[kT / 32];
-  const double alpha = scal[1];
+k_update_xr(int64_t n, const double* __restrict__ p, const double* __restrict__ q, double* __restrict__ x,
+            double* __restrict__ r, Dot dot) {
+  const double alpha = dot.scal[1];
   double s = 0.0;
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
        i += (int64_t)gridDim.x * blockDim.x) {
@@ -309,8 +383,7 @@ k_update_xr(int64_t n, const double* __restrict__ scal, const double* __restrict
     r[i] = ri;
     s += ri * ri;
   }
-  s = block_sum(s, red);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
+  dot_end(s, dot);
 }
 
 __global__ void k_update_p(int64_t n, const double* __restrict__ scal, const double* __restrict__ z,
@@ -608,9 +681,15 @@ geneo_status_t alloc_solver(geneo_handle_s* h) {
   return GENEO_OK;
 }
 
-geneo_status_t apply_prec(geneo_handle_s* h, const double* r, double* z, cudaStream_t s) {
+static geneo_status_t apply_dot(geneo_handle_s* h, const double* r, double* z, cudaStream_t s, const Dot& dot) {
   const int N = h->N;
-  k_restrict<<<N, kT, 0, s>>>(h->dsub, h->Dlist, r, h->Z, h->u, h->cH); note_launch();
+  if (N < 304) {   // fewer than two blocks per SM
+    const int gy = std::max(1, std::min(ceil_div(h->maxnD, kT), 4));
+    k_restrict_wide<<<dim3(N, gy + ceil_div(h->maxm, kRq)), kT, 0, s>>>(h->dsub, h->Dlist, r, h->Z, h->u, h->cH, gy);
+  } else {
+    k_restrict<<<N, kT, 0, s>>>(h->dsub, h->Dlist, r, h->Z, h->u, h->cH);
+  }
+  note_launch();
   GENEO_CUDA(cudaGetLastError());
   // the coarse solve: a dense product with A_H^{-1} on this stream (short),
   // or the band solve on one SM beside the batched local solves
@@ -640,11 +719,15 @@ geneo_status_t apply_prec(geneo_handle_s* h, const double* r, double* z, cudaStr
                           h->local_stages));
   h->prof.end(pl, s);
   if (h->dimH > 0 && !h->Hinv) GENEO_CUDA(cudaStreamWaitEvent(s, h->ev_join, 0));
-  const int grid = (int)std::min<int64_t>((h->n + kT - 1) / kT, 152 * 8);
+  const int grid = (int)std::min<int64_t>((h->n + kT - 1) / kT, kRedBlocks);
   k_prolong<<<grid, kT, 0, s>>>(h->n, h->dir, r, h->invD_ptr, h->invD_sub, h->invD_loc, h->dsub,
-                                h->u, h->Z, h->Hinv ? h->yH : h->cH, z); note_launch();
+                                h->u, h->Z, h->Hinv ? h->yH : h->cH, z, dot); note_launch();
   GENEO_CUDA(cudaGetLastError());
   return GENEO_OK;
+}
+
+geneo_status_t apply_prec(geneo_handle_s* h, const double* r, double* z, cudaStream_t s) {
+  return apply_dot(h, r, z, s, Dot{});
 }
 
 // Buffers of one PCG solve: device reduction partials, scalars and the
@@ -668,14 +751,14 @@ constexpr int kMaxReplace = 5;
 geneo_status_t pcg_core(geneo_handle_s* h, const double* b, double* x, double tol, int maxit,
                         geneo_solve_info_t* info, cudaStream_t s, const PcgBufs& B) {
   const int64_t n = h->n;
-  const int nb = kRedBlocks;
+  const int nb = (int)std::min<int64_t>(kRedBlocks, (n + kT - 1) / kT);  // blocks of the vector kernels
   double* scal = B.scal;
   double* red = B.red;
   GENEO_CUDA(cudaMemsetAsync(x, 0, sizeof(double) * n, s));
   GENEO_CUDA(cudaMemcpyAsync(h->r, b, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
   GENEO_CUDA(cudaMemsetAsync(scal, 0, sizeof(double) * 16, s));
-  k_dot<<<nb, kT, 0, s>>>(n, b, b, red); note_launch();
-  k_finish<<<1, kT, 0, s>>>(red, nb, scal, 4, B.da, B.db, 0); note_launch();
+  auto dot = [&](int what, int at) { return Dot{red, scal, what, B.da, B.db, at}; };
+  k_dot<<<nb, kT, 0, s>>>(n, b, b, dot(4, 0)); note_launch();
   GENEO_CUDA(cudaGetLastError());
   GENEO_CUDA(cudaMemcpyAsync(h->hpin, scal, sizeof(double) * 8, cudaMemcpyDeviceToHost, s));
   GENEO_CUDA(cudaStreamSynchronize(s));
@@ -708,12 +791,9 @@ geneo_status_t pcg_core(geneo_handle_s* h, const double* b, double* x, double to
   const bool det = h->opt.deterministic != 0;
   int it = 0;
   auto restart = [&]() -> geneo_status_t {  // p = z = M^{-1} r, rz = r.z
-    GENEO_TRY(apply_prec(h, h->r, h->zv, s));
+    GENEO_TRY(apply_dot(h, h->r, h->zv, s, det ? dot(0, 0) : Dot{}));
     GENEO_CUDA(cudaMemcpyAsync(h->p, h->zv, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
-    if (det) {
-      k_dot<<<nb, kT, 0, s>>>(n, h->r, h->zv, red); note_launch();
-      k_finish<<<1, kT, 0, s>>>(red, nb, scal, 0, B.da, B.db, 0); note_launch();
-    } else {
+    if (!det) {
       GENEO_CUDA(cudaMemsetAsync(scal + kRZ, 0, sizeof(double) * 6, s));
       k_dot_atomic<<<nb, kT, 0, s>>>(n, h->r, h->zv, scal, kRZ + (it & 1)); note_launch();
     }
@@ -722,9 +802,8 @@ geneo_status_t pcg_core(geneo_handle_s* h, const double* b, double* x, double to
   };
   // true residual into zv (free between the update and the next apply)
   auto true_residual = [&](double* out) -> geneo_status_t {
-    k_true_resid_sell<<<nb, kT, 0, s>>>(n, h->sell_off, h->sell_col, h->sell_val, x, b, h->zv, red);
+    k_true_resid_sell<<<nb, kT, 0, s>>>(n, h->sell_off, h->sell_col, h->sell_val, x, b, h->zv, dot(5, 0));
     note_launch();
-    k_finish<<<1, kT, 0, s>>>(red, nb, scal, 5, B.da, B.db, 0); note_launch();
     GENEO_CUDA(cudaGetLastError());
     GENEO_CUDA(cudaMemcpyAsync(h->hpin, scal, sizeof(double) * 8, cudaMemcpyDeviceToHost, s));
     GENEO_CUDA(cudaStreamSynchronize(s));
@@ -741,7 +820,7 @@ geneo_status_t pcg_core(geneo_handle_s* h, const double* b, double* x, double to
       const int pv = h->prof.begin(GENEO_PROF_SPMV, h->spmv_flops, h->spmv_bytes, s);
       if (det) {
         k_spmv_sell_dot<<<h->spmv_blocks, kT, 0, s>>>(n, h->sell_off, h->sell_col, h->sell_val, h->p, h->q,
-                                                      red);
+                                                      dot(1, it));
         note_launch();
       } else {
         k_spmv_atomic<<<nb, kT, 0, s>>>(n, h->sell_off, h->sell_col, h->sell_val, h->p, h->q, scal, par);
@@ -750,9 +829,7 @@ geneo_status_t pcg_core(geneo_handle_s* h, const double* b, double* x, double to
       h->prof.end(pv, s);
     }
     if (det) {
-      k_finish<<<1, kT, 0, s>>>(red, h->spmv_blocks, scal, 1, B.da, B.db, it); note_launch();
-      k_update_xr<<<nb, kT, 0, s>>>(n, scal, h->p, h->q, x, h->r, red); note_launch();
-      k_finish<<<1, kT, 0, s>>>(red, nb, scal, 2, B.da, B.db, it); note_launch();
+      k_update_xr<<<nb, kT, 0, s>>>(n, h->p, h->q, x, h->r, dot(2, it)); note_launch();
     } else {
       k_update_xr_atomic<<<nb, kT, 0, s>>>(n, scal, h->p, h->q, x, h->r, B.da, it, par); note_launch();
     }
@@ -787,10 +864,8 @@ geneo_status_t pcg_core(geneo_handle_s* h, const double* b, double* x, double to
       GENEO_TRY(restart());
       continue;
     }
-    GENEO_TRY(apply_prec(h, h->r, h->zv, s));
+    GENEO_TRY(apply_dot(h, h->r, h->zv, s, det ? dot(3, it - 1) : Dot{}));
     if (det) {
-      k_dot<<<nb, kT, 0, s>>>(n, h->r, h->zv, red); note_launch();
-      k_finish<<<1, kT, 0, s>>>(red, nb, scal, 3, B.da, B.db, it - 1); note_launch();
       k_update_p<<<nb, kT, 0, s>>>(n, scal, h->zv, h->p); note_launch();
     } else {
       k_dot_atomic<<<nb, kT, 0, s>>>(n, h->r, h->zv, scal, kRZ + (par ^ 1)); note_launch();
