@@ -496,6 +496,7 @@ k_tb_pack(const float* __restrict__ band, const BandDesc* __restrict__ descs, co
     const float* src = band + d.off + (int64_t)r * d.ld;
     const int64_t o = ((zoff[blockIdx.y] + I) * 32 + (r & 31)) * (int64_t)Wt;
     const float sr = (S && r < d.n) ? S[r] : 1.f;
+#pragma unroll 4
     for (int xx = lane; xx < Wt; xx += 32) {
       const int c = xx + 32 * I - W;
       float x = 0.f;
@@ -523,10 +524,21 @@ k_tb_unpack(float* __restrict__ band, const BandDesc* __restrict__ descs, const 
     const int I = r / 32;
     float* dst = band + d.off + (int64_t)r * d.ld;
     const int64_t o = ((zoff[blockIdx.y] + I) * 32 + (r & 31)) * (int64_t)Wt;
-    for (int c = max(0, r - d.w) + lane; c <= r; c += 32) {
-      const int xx = c - 32 * I + W;
-      dst[c - r + d.w] = phi[o + xx] + plo[o + xx];
+    // six groups of 32 in flight (one at a time left the copy at 3.0 TB/s)
+    constexpr int U = 6;
+    const int64_t oc = o - 32 * I + W;
+    int c = max(0, r - d.w) + lane;
+    for (; c + 32 * (U - 1) <= r; c += 32 * U) {
+      float v[U], l[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        v[u] = phi[oc + c + 32 * u];
+        l[u] = plo[oc + c + 32 * u];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) dst[c + 32 * u - r + d.w] = v[u] + l[u];
     }
+    for (; c <= r; c += 32) dst[c - r + d.w] = phi[oc + c] + plo[oc + c];
   }
 }
 
