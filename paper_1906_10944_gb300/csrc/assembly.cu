@@ -831,12 +831,28 @@ geneo_status_t assemble_local(geneo_handle_s* h, const geneo_problem_t* p, Assem
     // a weak pivot flags the matrix for an FP64 factorisation instead of
     // failing the setup
     const float wt = (float)h->opt.fp32_pivot_tol;
-    for (const FactorBatch& fb : batK)
-      GENEO_TRY(band_potrf<float>((float*)out.bandK, fb.d, (int)fb.h.size(), fb.maxw, fb.maxn, maskK, h->dstat, s, equil,
-                                  out.weak, wt, fb.plan.ok ? &fb.plan : nullptr));
-    for (const FactorBatch& fb : batA)
-      GENEO_TRY(band_potrf<float>((float*)h->bandA, fb.d, (int)fb.h.size(), fb.maxw, fb.maxn, maskA, h->dstat, h->aux,
-                                  equil, out.weak + N, wt, fb.plan.ok ? &fb.plan : nullptr));
+    auto factor = [&](const FactorBatch& fb, float* band, int32_t* weak, int mask, cudaStream_t on) {
+      return band_potrf<float>(band, fb.d, (int)fb.h.size(), fb.maxw, fb.maxn, mask, h->dstat, on, equil, weak, wt,
+                               fb.plan.ok ? &fb.plan : nullptr);
+    };
+    // the size classes of K_j side by side, the widest on the main stream and
+    // the others on the solve streams (one after another, each class's few
+    // matrices left most SMs idle); those of A_j one after another beside them
+    // and beside the eigensolver
+    const SolveStreams& ss = h->solve_streams;
+    const size_t lanes = std::min<size_t>(batK.size(), 1 + kSolveStreams);
+    for (size_t l = 1; l < lanes; ++l) GENEO_CUDA(cudaStreamWaitEvent(ss.s[l - 1], h->ev_fork, 0));
+    geneo_status_t rc = GENEO_OK;
+    for (size_t i = 0; i < batK.size() && rc == GENEO_OK; ++i) {
+      const size_t l = i % lanes;
+      rc = factor(batK[i], (float*)out.bandK, out.weak, maskK, l == 0 ? s : ss.s[l - 1]);
+    }
+    for (size_t l = 1; l < lanes; ++l) {   // joined also after a failed launch
+      GENEO_CUDA(cudaEventRecord(ss.ev[l - 1], ss.s[l - 1]));
+      GENEO_CUDA(cudaStreamWaitEvent(s, ss.ev[l - 1], 0));
+    }
+    GENEO_TRY(rc);
+    for (const FactorBatch& fb : batA) GENEO_TRY(factor(fb, (float*)h->bandA, out.weak + N, maskA, h->aux));
     h->factor_classes = (int)(batK.size() + batA.size());
   } else {
     GENEO_TRY(band_potrf<double>((double*)out.bandK, fdK, N, out.maxwK, maxnK, maskK, h->dstat, s));
