@@ -1413,10 +1413,20 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
   if (W3 > kMaxW) return GENEO_ERR_ARG;
   const int64_t rows = h->sumN;
   double *S, *KS, *BS, *P, *Tmp, *G, *Gp, *Tm, *nu, *rn;
-  // row splits of the Gram matrices: about two blocks per SM (18 subdomains of
-  // 38x31x24 elasticity in four splits used 72 of 152 SMs: 812 us per FP64
-  // Gram matrix against 268 us in 16)
-  const int nrs = std::max(kMinRS, std::min(kMaxRS, ceil_div(2 * 152, N)));
+  // row splits of the Gram matrices: the fewest waves of two blocks per SM per
+  // split, and few splits to sum (18 subdomains of 38x31x24 elasticity in four
+  // splits used 72 of 152 SMs: 812 us per FP64 Gram matrix, 328 us in 16; 64
+  // subdomains in 5 splits are 320 blocks, a second wave for the last 16 of
+  // them: 200 us per double-single Gram matrix, 164 us in 14)
+  int nrs = kMinRS;
+  double nrs_cost = 1e300;
+  for (int r = kMinRS; r <= kMaxRS; ++r) {
+    const double cost = (double)ceil_div(N * r, 2 * 152) / r + 0.002 * r;
+    if (cost < nrs_cost) {
+      nrs_cost = cost;
+      nrs = r;
+    }
+  }
   GENEO_TRY(tmp.get(&S, (size_t)rows * W3));
   GENEO_TRY(tmp.get(&KS, (size_t)rows * W3));
   GENEO_TRY(tmp.get(&BS, (size_t)rows * W3));
