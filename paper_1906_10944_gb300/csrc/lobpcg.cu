@@ -85,6 +85,34 @@ ColRefT<S> cref(S* base, int W, int c0, const int32_t* c0d, int w, const int32_t
 // ---------------------------------------------------------------------------
 // Multivector kernels (grid: x = row blocks, y = subdomain).
 // ---------------------------------------------------------------------------
+// The sparse products below form four columns per pass over a row's entries.
+// SHARED: a block's kT rows and w columns are cut into units of 32 rows x 4
+// columns, one warp each, the column groups of a row chunk on neighbouring
+// warps, so that all but the first take the entries from L1 (one thread per row
+// reads them again from L2 or HBM for every four columns: elasticity 38^3, 81
+// entries a row, 442 MB for each of six passes; k_spmm_ds 558 -> 546 us).
+// Otherwise one thread per row loops over the columns: short rows stay in L1 by
+// themselves, and the warps of a block, at the same columns, share more of the
+// gathered values (27 entries, 128^3: 920 us SHARED, 734 us so).
+constexpr int kUnitCols = 4;
+constexpr int kLongRow = 40;    // entries of a row beyond which neighbouring warps share them
+template <bool SHARED, typename Body>
+__device__ __forceinline__ void spmm_units(int n, int w, Body body) {
+  const int r0 = (int)blockIdx.x * kT;
+  if constexpr (SHARED) {
+    const int groups = (w + kUnitCols - 1) / kUnitCols;
+    const int units = (min(kT, n - r0) + 31) / 32 * groups;
+    for (int u = (int)threadIdx.x >> 5; u < units; u += kT / 32) {
+      const int a = r0 + u / groups * 32 + ((int)threadIdx.x & 31), c = u % groups * kUnitCols;
+      if (a < n) body(a, c, min(kUnitCols, w - c));
+    }
+  } else {
+    const int a = r0 + (int)threadIdx.x;
+    if (a < n)
+      for (int c = 0; c < w; c += kUnitCols) body(a, c, min(kUnitCols, w - c));
+  }
+}
+
 // S is the storage and arithmetic type: double, or float for the first
 // orthogonalisation pass (FP32 copies of the operand and of K's values, so
 // nothing is converted in the inner loop).
@@ -93,50 +121,38 @@ __global__ void __launch_bounds__(kT)
 k_spmm(const SubDesc* __restrict__ sub, const int64_t* __restrict__ lrow,
        const int32_t* __restrict__ lcol, const S* __restrict__ v1, const S* __restrict__ v2,
        ColRefT<S> X, ColRefT<S> Y1, ColRefT<S> Y2, const int32_t* __restrict__ skip) {
-  using C = S;
   const int j = blockIdx.y;
   if (skip && skip[j]) return;
   const SubDesc d = sub[j];
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= d.nN) return;
   const int w = cr_w(X, j);
   const S* x = cr_ptr(X, d, j);
   S* y1 = cr_ptr(Y1, d, j);
   S* y2 = v2 ? cr_ptr(Y2, d, j) : nullptr;
-  const int64_t e0 = lrow[d.offN + a], e1 = lrow[d.offN + a + 1];
   const int64_t nn = d.nN;
-  // four columns per pass: the row's column indices and values are read once
-  // per four vectors
-  int c = 0;
-  for (; c + 4 <= w; c += 4) {
+  spmm_units<true>(d.nN, w, [&](int a, int c, int nc) {
+    const int64_t e0 = lrow[d.offN + a], e1 = lrow[d.offN + a + 1];
     const S* xc = x + (int64_t)c * nn;
-    C s10 = 0, s11 = 0, s12 = 0, s13 = 0, s20 = 0, s21 = 0, s22 = 0, s23 = 0;
+    S s1[kUnitCols], s2[kUnitCols];
+#pragma unroll
+    for (int z = 0; z < kUnitCols; ++z) s1[z] = s2[z] = 0;
     for (int64_t e = e0; e < e1; ++e) {
       const int col = lcol[e];
-      const C x0 = (C)xc[col], x1 = (C)xc[nn + col], x2 = (C)xc[2 * nn + col], x3 = (C)xc[3 * nn + col];
-      const C va = (C)v1[e];
-      s10 += va * x0; s11 += va * x1; s12 += va * x2; s13 += va * x3;
-      if (v2) {
-        const C vb = (C)v2[e];
-        s20 += vb * x0; s21 += vb * x1; s22 += vb * x2; s23 += vb * x3;
+      const S va = v1[e], vb = v2 ? v2[e] : S(0);
+#pragma unroll
+      for (int z = 0; z < kUnitCols; ++z)
+        if (z < nc) {
+          const S xv = xc[z * nn + col];
+          s1[z] += va * xv;
+          if (v2) s2[z] += vb * xv;
+        }
+    }
+#pragma unroll
+    for (int z = 0; z < kUnitCols; ++z)
+      if (z < nc) {
+        y1[(c + z) * nn + a] = s1[z];
+        if (v2) y2[(c + z) * nn + a] = s2[z];
       }
-    }
-    y1[c * nn + a] = s10; y1[(c + 1) * nn + a] = s11; y1[(c + 2) * nn + a] = s12; y1[(c + 3) * nn + a] = s13;
-    if (v2) {
-      y2[c * nn + a] = s20; y2[(c + 1) * nn + a] = s21; y2[(c + 2) * nn + a] = s22; y2[(c + 3) * nn + a] = s23;
-    }
-  }
-  for (; c < w; ++c) {
-    const S* xc = x + (int64_t)c * nn;
-    C s1 = 0, s2 = 0;
-    for (int64_t e = e0; e < e1; ++e) {
-      const C xv = (C)xc[lcol[e]];
-      s1 += (C)v1[e] * xv;
-      if (v2) s2 += (C)v2[e] * xv;
-    }
-    y1[c * nn + a] = s1;
-    if (v2) y2[c * nn + a] = s2;
-  }
+  });
 }
 
 // ---------------------------------------------------------------------------
@@ -210,57 +226,53 @@ __global__ void k_build_ell(const SubDesc* __restrict__ sub, const int64_t* __re
   }
 }
 
-// Y1 = V1 X (and Y2 = V2 X when v2 is given) in double-single arithmetic from
-// the ELLPACK layout, results stored in FP64; one row per thread, four
-// columns per pass (more columns per pass cost occupancy, which this
-// gather-bound loop needs more), the entry loop unrolled three times so that
-// the loads of several entries are in flight before their gathers.  Each
-// entry and operand value is one 8-byte (hi, lo) load.
-__global__ void __launch_bounds__(kT)
+// Y1 = V1 X (and, BOTH, Y2 = V2 X) in double-single arithmetic from the
+// ELLPACK layout, results stored in FP64; units of 32 rows x 4 columns (more
+// columns per thread cost occupancy, which this gather-bound loop needs more:
+// at most 64 registers for four blocks per SM, 808 -> 740 us at 128^3), the entry
+// loop unrolled three times so that the loads of several entries are in flight
+// before their gathers.  Each entry and operand value is one 8-byte
+// (hi, lo) load.
+template <bool BOTH, bool SHARED>
+__global__ void __launch_bounds__(kT, 4)
 k_spmm_ds(const SubDesc* __restrict__ sub, int L, const int32_t* __restrict__ ecol,
           const float2* __restrict__ v1, const float2* __restrict__ v2, ColRefT<float2> X2, ColRef Y1,
           ColRef Y2, const int32_t* __restrict__ skip) {
   const int j = blockIdx.y;
   if (skip && skip[j]) return;
   const SubDesc d = sub[j];
-  const int a = blockIdx.x * blockDim.x + threadIdx.x;
-  if (a >= d.nN) return;
   const int w = cr_w(X2, j);
   const float2* x2 = cr_ptr(X2, d, j);
   double* y1 = cr_ptr(Y1, d, j);
-  double* y2 = v2 ? cr_ptr(Y2, d, j) : nullptr;
+  double* y2 = BOTH ? cr_ptr(Y2, d, j) : nullptr;
   const int64_t nn = d.nN;
-  const int64_t base = d.offN * (int64_t)L + a;
-  constexpr int CP = 4;
-  for (int c = 0; c < w; c += CP) {
-    const int nc = min(CP, w - c);
-    DS s1[CP], s2[CP];
+  spmm_units<SHARED>(d.nN, w, [&](int a, int c, int nc) {
+    DS s1[kUnitCols], s2[kUnitCols];
 #pragma unroll
-    for (int z = 0; z < CP; ++z) s1[z] = s2[z] = DS{0.f, 0.f};
+    for (int z = 0; z < kUnitCols; ++z) s1[z] = s2[z] = DS{0.f, 0.f};
     const float2* xc = x2 + (int64_t)c * nn;
+    const int64_t base = d.offN * (int64_t)L + a;
 #pragma unroll 3
     for (int t = 0; t < L; ++t) {
       const int64_t o = base + (int64_t)t * nn;
       const int col = ecol[o];
       const float2 va = v1[o];
-      const float2 vb = v2 ? v2[o] : make_float2(0.f, 0.f);
+      const float2 vb = BOTH ? v2[o] : make_float2(0.f, 0.f);
 #pragma unroll
-      for (int z = 0; z < CP; ++z) {
+      for (int z = 0; z < kUnitCols; ++z)
         if (z < nc) {
           const float2 xv = xc[z * nn + col];
           ds_fma(s1[z], va.x, va.y, xv.x, xv.y);
-          if (v2) ds_fma(s2[z], vb.x, vb.y, xv.x, xv.y);
+          if (BOTH) ds_fma(s2[z], vb.x, vb.y, xv.x, xv.y);
         }
-      }
     }
 #pragma unroll
-    for (int z = 0; z < CP; ++z) {
+    for (int z = 0; z < kUnitCols; ++z)
       if (z < nc) {
         y1[(c + z) * nn + a] = acc_value(s1[z]);
-        if (v2) y2[(c + z) * nn + a] = acc_value(s2[z]);
+        if (BOTH) y2[(c + z) * nn + a] = acc_value(s2[z]);
       }
-    }
-  }
+  });
 }
 
 // Y = X columnwise copy (with conversion between storage types)
@@ -798,7 +810,11 @@ __global__ void k_init_random(const SubDesc* __restrict__ sub, ColRef X, uint64_
 // of pair k, columns of pair l) is R_k A_kl R_l^T.  A stays exactly
 // symmetric, so only the blocks k <= l are formed and each is written to
 // both of its places; every block is read and written by one thread, in
-// place.  One barrier after the rotations, one after the update.
+// place.  One barrier after the update of A; the next rotations, a latency-bound
+// chain on one or two warps, are formed beside the update of V, whose warps a
+// barrier for them left idle (with the blocks k <= l enumerated without gaps,
+// k_rr<dsv> 2.00 -> 1.36 ms at 18 subdomains of order 72, 1.00 -> 0.61 ms at 512
+// of order 36).
 // ---------------------------------------------------------------------------
 template <typename T> struct JacobiOps;
 template <> struct JacobiOps<float> {
@@ -890,7 +906,7 @@ __device__ void jacobi_eig(T* A, int lda, T* V, int ldv, int m, T* cs, T* sn,
                            typename JacobiOps<T>::R* red) {
   using J = JacobiOps<T>;
   using R = typename J::R;
-  __shared__ int jp[kMaxW / 2 + 1], jq[kMaxW / 2 + 1], jact[kMaxW / 2 + 1];
+  __shared__ uint32_t jpk[2][kMaxW / 2 + 1];   // p | q << 8 | rotates << 16
   const int tid = threadIdx.x, nt = blockDim.x;
   const int M = m + (m & 1), H = M / 2;
   for (int idx = tid; idx < m * m; idx += nt) {
@@ -899,6 +915,32 @@ __device__ void jacobi_eig(T* A, int lda, T* V, int ldv, int m, T* cs, T* sn,
   }
   __syncthreads();
   if (m <= 1) return;
+  // idx / m and idx / (H + 1) by a product (idx * divisor < 2^24)
+  static_assert(kMaxW <= 192, "eight-bit indices, and the quotients by products");
+  const uint32_t inv_m = (1u << 24) / (uint32_t)m + 1u, inv_h = (1u << 24) / (uint32_t)(H + 1) + 1u;
+  const int tri = H * (H + 1) / 2;
+  const int rw = min((H + 31) / 32, nt / 64);   // warps that form the rotations
+  auto rotations = [&](int round, int t0, int step) {
+    const int buf = round & 1;
+    // pair k: (M-1, round) for k = 0; ((round+k)%(M-1), (round-k+M-1)%(M-1))
+    // otherwise; q = M - 1 = m is the padding index of odd m
+    for (int k = t0; k < H; k += step) {
+      int pi, qi;
+      if (k == 0) {
+        pi = M - 1;
+        qi = round;
+      } else {
+        pi = round + k >= M - 1 ? round + k - (M - 1) : round + k;
+        qi = round - k < 0 ? round - k + M - 1 : round - k;
+      }
+      if (pi > qi) { const int t = pi; pi = qi; qi = t; }
+      T c = T(1.0), sv = T(0.0);
+      const bool act = qi < m && jacobi_rot(A[pi * lda + pi], A[qi * lda + qi], A[pi * lda + qi], c, sv);
+      jpk[buf][k] = (uint32_t)pi | (uint32_t)qi << 8 | (act ? 1u << 16 : 0u);
+      cs[buf * H + k] = act ? c : T(1.0);
+      sn[buf * H + k] = act ? sv : T(0.0);
+    }
+  };
   for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
     R off = R(0), all = R(0);
     for (int idx = tid; idx < m * m; idx += nt) {
@@ -910,28 +952,21 @@ __device__ void jacobi_eig(T* A, int lda, T* V, int ldv, int m, T* cs, T* sn,
     off = block_sum(off, red);
     all = block_sum(all, red);
     if (off <= J::eps_off * all || all == R(0)) break;
+    rotations(0, tid, nt);
+    __syncthreads();
     for (int round = 0; round < M - 1; ++round) {
-      // pair k: (M-1, round) for k = 0; ((round+k)%(M-1), (round-k+M-1)%(M-1))
-      // otherwise; q = M - 1 = m is the padding index of odd m
-      for (int k = tid; k < H; k += nt) {
-        int pi, qi;
-        if (k == 0) { pi = M - 1; qi = round; }
-        else { pi = (round + k) % (M - 1); qi = (round - k + M - 1) % (M - 1); }
-        if (pi > qi) { const int t = pi; pi = qi; qi = t; }
-        T c = T(1.0), sv = T(0.0);
-        const bool act = qi < m && jacobi_rot(A[pi * lda + pi], A[qi * lda + qi], A[pi * lda + qi], c, sv);
-        jp[k] = pi;
-        jq[k] = qi;
-        jact[k] = act;
-        cs[k] = act ? c : T(1.0);
-        sn[k] = act ? sv : T(0.0);
-      }
-      __syncthreads();
-      // A <- R A R^T over the blocks k <= l
-      for (int idx = tid; idx < H * H; idx += nt) {
-        const int k = idx / H, l = idx % H;
-        if (k > l || !(jact[k] | jact[l])) continue;
-        const int pk = jp[k], qk = jq[k], pl = jp[l], ql = jq[l];
+      const uint32_t* jp = jpk[round & 1];
+      const T* cr = cs + (round & 1) * H;
+      const T* sr = sn + (round & 1) * H;
+      // A <- R A R^T over the blocks k <= l; rows kk and H - 1 - kk of that
+      // triangle together have H + 1 blocks
+      for (int idx = tid; idx < tri; idx += nt) {
+        const int kk = (int)((uint32_t)idx * inv_h >> 24), pos = idx - kk * (H + 1);
+        const int k = pos < H - kk ? kk : H - 1 - kk;
+        const int l = pos < H - kk ? kk + pos : pos - 1;
+        const uint32_t ek = jp[k], el = jp[l];
+        if (!((ek | el) >> 16)) continue;
+        const int pk = ek & 255, qk = ek >> 8 & 255, pl = el & 255, ql = el >> 8 & 255;
         const bool hk = qk < m, hl = ql < m;
         const T z = T(0.0);
         const T a00 = A[pk * lda + pl];
@@ -939,16 +974,16 @@ __device__ void jacobi_eig(T* A, int lda, T* V, int ldv, int m, T* cs, T* sn,
         const T a10 = hk ? A[qk * lda + pl] : z;
         const T a11 = (hk && hl) ? A[qk * lda + ql] : z;
         T t00 = a00, t01 = a01, t10 = a10, t11 = a11;
-        if (jact[l]) {
-          const T c = cs[l], s = sn[l];
+        if (el >> 16) {
+          const T c = cr[l], s = sr[l];
           t00 = a00 * c - a01 * s;
           t01 = a00 * s + a01 * c;
           t10 = a10 * c - a11 * s;
           t11 = a10 * s + a11 * c;
         }
         T b00 = t00, b01 = t01, b10 = t10, b11 = t11;
-        if (jact[k]) {
-          const T c = cs[k], s = sn[k];
+        if (ek >> 16) {
+          const T c = cr[k], s = sr[k];
           b00 = c * t00 - s * t10;
           b10 = s * t00 + c * t10;
           b01 = c * t01 - s * t11;
@@ -979,15 +1014,22 @@ __device__ void jacobi_eig(T* A, int lda, T* V, int ldv, int m, T* cs, T* sn,
           A[ql * lda + qk] = b11;
         }
       }
+      __syncthreads();
+      // the first warps form the next round's rotations while the others take
       // V <- V R^T (columns of the pairs)
-      for (int idx = tid; idx < H * m; idx += nt) {
-        const int k = idx / m, row = idx % m;
-        if (!jact[k]) continue;
-        const int pi = jp[k], qi = jq[k];
-        const T c = cs[k], s = sn[k];
-        const T vp = V[row * ldv + pi], vq = V[row * ldv + qi];
-        V[row * ldv + pi] = c * vp - s * vq;
-        V[row * ldv + qi] = s * vp + c * vq;
+      if (tid < 32 * rw) {
+        if (round + 1 < M - 1) rotations(round + 1, tid, 32 * rw);
+      } else {
+        for (int idx = tid - 32 * rw; idx < H * m; idx += nt - 32 * rw) {
+          const int k = (int)((uint32_t)idx * inv_m >> 24), row = idx - k * m;
+          const uint32_t ek = jp[k];
+          if (!(ek >> 16)) continue;
+          const int pi = ek & 255, qi = ek >> 8 & 255;
+          const T c = cr[k], s = sr[k];
+          const T vp = V[row * ldv + pi], vq = V[row * ldv + qi];
+          V[row * ldv + pi] = c * vp - s * vq;
+          V[row * ldv + qi] = s * vp + c * vq;
+        }
       }
       __syncthreads();
     }
@@ -1020,8 +1062,8 @@ k_svqb(const double* __restrict__ Gall, double* __restrict__ Tout, int ldg,
   T* dsc = V + (size_t)wmax * LD;
   T* ev = dsc + wmax;
   T* cs = ev + wmax;
-  T* sn = cs + wmax;
-  T* red = sn + wmax;
+  T* sn = cs + wmax + 1;   // two rounds' values of ceil(m / 2) each
+  T* red = sn + wmax + 1;
   __shared__ int keep[kMaxW];
   __shared__ int nkeep;
   if (q <= 0) {
@@ -1172,8 +1214,8 @@ k_rr(const double* __restrict__ Gall, double* __restrict__ Tout, int ldg,
   T* V = A + (size_t)wmax * LD;
   double* ev = reinterpret_cast<double*>(V + (size_t)wmax * LD);
   T* cs = reinterpret_cast<T*>(ev + wmax);
-  T* sn = cs + wmax;
-  auto* red = reinterpret_cast<typename JacobiOps<T>::R*>(sn + wmax);
+  T* sn = cs + wmax + 1;   // two rounds' values of ceil(m / 2) each
+  auto* red = reinterpret_cast<typename JacobiOps<T>::R*>(sn + wmax + 1);
   __shared__ int order[kMaxW];
   __shared__ double wmx[kTD / 32];
   if (m <= 0) return;
@@ -1775,8 +1817,16 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
         const ColRefT<float2> Xs{X2, X.W, X.c0, X.c0d, X.w, X.wd, X.wd2};
         k_split_cols<<<gridR, kT, 0, st>>>(h->dsub, X, Xs, sds); note_launch();
         const bool both = withK && withB;
-        k_spmm_ds<<<gridR, kT, 0, st>>>(h->dsub, ell, ecol, withK ? eK2 : eB2, both ? eB2 : nullptr, Xs,
-                                        withK ? YK : YB, YB, sds);
+        // rows longer than a few loads in flight: units shared by neighbouring warps
+        if (both) {
+          if (ell > kLongRow) k_spmm_ds<true, true><<<gridR, kT, 0, st>>>(h->dsub, ell, ecol, eK2, eB2, Xs, YK, YB, sds);
+          else k_spmm_ds<true, false><<<gridR, kT, 0, st>>>(h->dsub, ell, ecol, eK2, eB2, Xs, YK, YB, sds);
+        } else {
+          const float2* v = withK ? eK2 : eB2;
+          const ColRef Y = withK ? YK : YB;
+          if (ell > kLongRow) k_spmm_ds<false, true><<<gridR, kT, 0, st>>>(h->dsub, ell, ecol, v, nullptr, Xs, Y, Y, sds);
+          else k_spmm_ds<false, false><<<gridR, kT, 0, st>>>(h->dsub, ell, ecol, v, nullptr, Xs, Y, Y, sds);
+        }
         note_launch();
         if (n64 == 0) {
           h->prof.end(pr, st);
