@@ -29,6 +29,17 @@ __device__ __forceinline__ void ds_fma(DS& acc, float ah, float al, float xh, fl
   acc.l = __fadd_rn(acc.l, __fadd_rn(err, e));
 }
 
+// acc += a * x for a float a
+__device__ __forceinline__ void ds_fma1(DS& acc, float a, float xh, float xl) {
+  const float p = __fmul_rn(a, xh);
+  const float e = __fmaf_rn(a, xl, __fmaf_rn(a, xh, -p));
+  const float s = __fadd_rn(acc.h, p);
+  const float bv = __fsub_rn(s, acc.h);
+  const float err = __fadd_rn(__fsub_rn(acc.h, __fsub_rn(s, bv)), __fsub_rn(p, bv));
+  acc.h = s;
+  acc.l = __fadd_rn(acc.l, __fadd_rn(err, e));
+}
+
 // FP64 -> (hi, lo) floats with integer operations only (the FP64 pipe,
 // which also executes conversions, is the scarce unit): hi keeps the sign,
 // the exponent and the top 23 mantissa bits (truncation), lo the next 23

@@ -1335,15 +1335,28 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
 // blocks' lower triangles (w >= blk - 1, so the triangle lies in the band).
 // One thread block per diagonal block; thread c forms column c by forward
 // substitution in arithmetic A (double-single for FP32 bands: FP64 runs at
-// 1/64 of the FP32 rate here) and rounds it to T.
+// 1/64 of the FP32 rate here) and rounds it to T.  Four rows at a time: four
+// independent sums hide the latency of a double-single sum that one or two
+// rows left bare, and share each loaded value of X.
 // ---------------------------------------------------------------------------
+template <typename A, typename T>
+__device__ __forceinline__ void blkinv_fma(A& s, T l, const A& x) {
+  if constexpr (std::is_same_v<A, dsv> && std::is_same_v<T, float>) {
+    DS v{s.h, s.l};
+    ds_fma1(v, l, x.h, x.l);
+    s = dsv(v.h, v.l);
+  } else {
+    s += factor_value<A>(l) * x;
+  }
+}
 template <typename T, typename A, int B>
 constexpr size_t blkinv_smem() {
-  return sizeof(A) * (B * B + B) + sizeof(T) * B * B;
+  return sizeof(A) * (B * B + B) + sizeof(T) * B * (B + 4);
 }
 template <typename T, typename A, int B>
 __global__ void __launch_bounds__(B < 32 ? 32 : B)
 k_band_blkinv(T* __restrict__ base, const BandDesc* __restrict__ descs) {
+  constexpr int LT = B + 4;
   const BandDesc d = descs[blockIdx.y];
   const int kb = (int)blockIdx.x * B;
   if (kb >= d.n || d.blk != B) return;
@@ -1352,27 +1365,36 @@ k_band_blkinv(T* __restrict__ base, const BandDesc* __restrict__ descs) {
   extern __shared__ __align__(128) unsigned char smem_raw[];
   A* Xs = reinterpret_cast<A*>(smem_raw);   // B x B
   A* Rs = Xs + B * B;                       // reciprocal pivots
-  T* Ls = reinterpret_cast<T*>(Rs + B);     // B x B
+  T* Lt = reinterpret_cast<T*>(Rs + B);     // L(r, t) at t * LT + r
   const int nt = blockDim.x, c = threadIdx.x;
 #pragma unroll 8
   for (int i = c; i < B * B; i += nt) {
     const int r = i / B, cc = i % B;
-    Ls[i] = (r < b && cc <= r) ? L[(int64_t)r * ld + cc - r] : T(0);
+    Lt[cc * LT + r] = (r < b && cc <= r) ? L[(int64_t)r * ld + cc - r] : T(0);
   }
-  if (c < b) Rs[c] = recip_arith<A>(L[(int64_t)c * ld]);
+  if (c < B) Rs[c] = c < b ? recip_arith<A>(L[(int64_t)c * ld]) : A();
   __syncthreads();
   if (c < B) {
     const int w0 = c & ~31;   // this warp's columns are zero above row w0
-    for (int r = w0; r < b; ++r) {
-      A s0 = A(), s1 = A();
-      int t = w0;
-      for (; t + 1 < r; t += 2) {
-        s0 += factor_value<A>(Ls[r * B + t]) * Xs[t * B + c];
-        s1 += factor_value<A>(Ls[r * B + t + 1]) * Xs[(t + 1) * B + c];
+    for (int r0 = w0; r0 < b; r0 += 4) {
+      A s[4] = {};
+#pragma unroll 2
+      for (int t = w0; t < r0; ++t) {
+        T l[4];
+        load_n<4>(Lt + t * LT + r0, l);
+        const A x = Xs[t * B + c];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) blkinv_fma<A>(s[i], l[i], x);
       }
-      if (t < r) s0 += factor_value<A>(Ls[r * B + t]) * Xs[t * B + c];
-      const A one = r == c ? to_arith<A>(1.0) : A();
-      Xs[r * B + c] = (one - (s0 + s1)) * Rs[r];
+      A x[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+#pragma unroll
+        for (int q = 0; q < i; ++q) blkinv_fma<A>(s[i], Lt[(r0 + q) * LT + r0 + i], x[q]);
+        const A one = r0 + i == c ? to_arith<A>(1.0) : A();
+        x[i] = (one - s[i]) * Rs[r0 + i];
+        Xs[(r0 + i) * B + c] = x[i];
+      }
     }
     for (int r = c; r < b; ++r) L[(int64_t)r * ld + c - r] = (T)to_double(Xs[r * B + c]);
   }
