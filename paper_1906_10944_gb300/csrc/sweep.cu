@@ -1588,14 +1588,26 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
       for (int c0 = 0; c0 < nrhs; c0 += 32) {
         a.c0 = c0;
         a.kc = std::min(32, nrhs - c0);
-        // two column tiles per block while the batch fills the GPU anyway
-        const int units = (a.kc + 7) / 8;
-        bool two = units > 1 && (int64_t)live * units > sms;
-        if (two)
-          two = (blk == 64 ? mma_smem<64, 2>(max_w, 1, 2) : blk == 32 ? mma_smem<32, 2>(max_w, 1, 2)
-                                                                     : mma_smem<16, 2>(max_w, 1, 2)) <= kSmemMax;
-        const int parts = two ? (units + 1) / 2 : units;
-        const int C = clusters(parts);
+        // one or two column tiles of 8 per block: two take 1.5 times as long per
+        // block and need half as many (64 bands of order 6859, half width 381,
+        // 12 columns: 662 us in two parts of one tile on single blocks, 562 us in
+        // one part of two on clusters of 2; 27 of order 9261, half width 463:
+        // 593 and 645 us)
+        int parts = (a.kc + 7) / 8;
+        double len1;
+        int C = clusters(parts, &len1);
+        bool two = parts > 1 && (blk == 64   ? mma_smem<64, 2>(max_w, 1, 2)
+                                 : blk == 32 ? mma_smem<32, 2>(max_w, 1, 2)
+                                             : mma_smem<16, 2>(max_w, 1, 2)) <= kSmemMax;
+        if (two) {
+          double len2;
+          const int C2 = clusters((parts + 1) / 2, &len2);
+          two = 1.5 * len2 < len1;
+          if (two) {
+            C = C2;
+            parts = (parts + 1) / 2;
+          }
+        }
         geneo_status_t rc;
         if (two)
           rc = blk == 64 ? run_mma<64, 2>(base, a, C, parts, tc_passes)
