@@ -9,29 +9,41 @@
 // Storage while factoring ("tiled band"): each matrix is cut into row blocks
 // of 32 rows; row block I holds the dense 32 x (W + 32) rectangle of the
 // columns [32 I - W, 32 I + 32), W = the batch's largest half bandwidth
-// rounded up to 32, row-major.  Entries outside the band are zero and stay
-// zero.  In this layout the columns [c - W, c) of any row block form a plain
-// 2D box, so the panel update of a left-looking Cholesky is a sequence of
-// boxed tiles.  Each value x is kept in two planes, hi and lo, both TF32
-// (split_tf32_rn), so the three-pass TF32 product hi*hi + hi*lo + lo*hi
-// (error at most 3 * 2^-22 of the product) needs no splitting on chip.  The row blocks of a whole batch form one 3D tensor
-// (x: W + 32 columns, y: 32 rows, z: row block) described by two tensor maps
-// (hi, lo) with 128-byte swizzle, the layout the MMA descriptors read.
+// rounded up to 32, row-major, the block of columns 32 C .. 32 C + 31 at slot
+// C mod (W / 32 + 1) of the row.  Entries outside the band are zero and stay
+// zero.  So the same columns of any number of consecutive rows form one 2D box,
+// and the panel update of a left-looking Cholesky is a sequence of boxed tiles.
+// Each value x is kept in two planes, hi and lo, both TF32 (split_tf32_rn), so
+// the three-pass TF32 product hi*hi + hi*lo + lo*hi (error at most 3 * 2^-22 of
+// the product) needs no splitting on chip.  The rows of a whole batch form one
+// 3D tensor (x: W + 32 columns, y: rows, z: plane) described by tensor maps of
+// several box heights with 128-byte swizzle, the layout the MMA descriptors
+// read.
 //
 // Panel J (columns c0 = 32 J .. c0 + 31; rows [c0, c0 + R),
 // R = min(n, c0 + 32 + w) - c0, in chunks h of 128 rows = four row blocks):
 //   D_h = sum over k-chunks q of A_h(q) B(q)^T      (TMEM, M 128 x N 32)
-// with A_h(q) = the chunk's rows at the columns c0 - W + 32 q .. + 31 (row
-// block I: box x = 32 (J + q - I), negative x reads zeros) and B(q) = row
-// block J at box x = 32 q.  Each tile is four K = 8 steps times three passes
-// of tcgen05.mma kind::tf32.  Tiles whose row blocks all lie outside the
-// band (4 h > q) are skipped.  The tensor cores add each MMA's products into
+// with A_h(q) = the chunk's rows at the columns c0 - W + 32 q .. + 31 and B(q) =
+// row block J at the same columns.  Each tile is four K = 8 steps times three
+// passes of tcgen05.mma kind::tf32, or two where one of N = 64 reads both planes
+// of B (an MMA takes about 66 cycles for N = 32 and 64 alike: it waits for its
+// 128 rows of A).  Tiles whose row blocks all lie outside the band (4 h > q) are
+// skipped.  A full tile (q >= 4 h + 3) is one copy of both planes; in the other
+// three of a chunk the row blocks below the band, whose slot holds other
+// columns, are filled with zeros by boxes out of range.  (Copies of one 32 x 32
+// box each, eight a tile, took 824 cycles to issue, one copy of the tile 306.)
+// What bounds a panel is the turn of a stage: copy, MMAs, and the hand-overs
+// between the roles, about 1300 cycles a tile with four stages.  Measured with
+// all of this against copies box by box, one MMA warp and the diagonal block
+// through shared memory: 64 bands of order 5832, half width 340, 4.1 -> 3.7 ms;
+// 27 of order 9261, 463, 9.3 -> 8.0 ms; 18 of order 9000, 672, 15.6 -> 12.6 ms.
+// The tensor cores add each MMA's products into
 // the FP32 accumulator with truncation, a bias that grows with the number of
 // MMAs summed into one accumulator; so every chunk has 1 + P accumulators:
 // slot 0 takes the small terms (lo*hi + hi*lo), slot 1 + (q mod P) the
 // hi*hi terms of k-chunk q, and the panel threads add the slots in FP32
-// (small terms first).  Thread 0 issues the copies and thread 32 the
-// MMAs through a ring of kStages stages (full / empty mbarriers;
+// (small terms first).  One lane issues the copies and two lanes the
+// MMAs through rings of stages (full / empty mbarriers;
 // tcgen05.commit releases a stage and finally signals the accumulators).
 // Then every thread reads its TMEM lane (tcgen05.ld), forms U = A - D in
 // shared memory, one warp factors the 32 x 32 diagonal block in registers,
@@ -57,7 +69,7 @@ namespace geneo {
 namespace {
 
 constexpr int kEpi5 = 256;                     // epilogue / panel threads (warps 0-7)
-constexpr int kT5 = kEpi5 + 64;                // + copy warp 8 + MMA warp 9
+constexpr int kT5 = kEpi5 + 96;                // + copy warp 8 + MMA warps 9, 10
 constexpr int kPB5 = 32;                       // panel width = row block height
 constexpr int kMaxStA5 = 4;                    // A-tile stages (4, or fewer for the widest bands)
 constexpr int kStB5 = 2;                       // B-tile stages
@@ -67,7 +79,7 @@ constexpr uint32_t kTileA5 = 4 * kBox5;        // 128 rows x 32 columns
 constexpr uint32_t kTileB5 = kBox5;            // 32 rows x 32 columns
 constexpr uint32_t kStageA5 = 2 * kTileA5;     // hi and lo of an A tile: 32 KB
 constexpr uint32_t kStageB5 = 2 * kTileB5;     // hi and lo of a B tile: 8 KB
-constexpr uint32_t kIdesc5 = umma_idesc_tf32(128, 32);
+constexpr uint32_t kIdesc5 = umma_idesc_tf32(128, 32), kIdesc5x2 = umma_idesc_tf32(128, 64);
 constexpr int kMaxPar5 = 7;                    // at most this many hi*hi accumulators per chunk
 // afull, aempty, bfull, bempty, acc_full[2], acc_empty[2], pdone, fin
 constexpr int bars5(int sta) { return 2 * sta + 2 * kStB5 + 2 + 2 + 2; }
@@ -120,8 +132,8 @@ __device__ __forceinline__ void split5(float x, int bf16, float& h, float& l) {
 }
 
 // Warp-specialised: warp 8 (one lane) streams the tiles of panel after
-// panel, warp 9 (one lane) issues the MMAs into one of nbuf (1 or 2) TMEM
-// accumulator buffers (panel G uses buffer G % nbuf), and warps 0-7 run the panel
+// panel, warps 9 and 10 (one lane each) issue the MMAs into one of nbuf (1 or 2)
+// TMEM accumulator buffers (panel G uses buffer G % nbuf), and warps 0-7 run the panel
 // steps.  A tiles go through a ring of kStA5 stages (4, or 3 or 2 for the
 // widest classes, whose panel block takes the room), the B tile of each
 // k-chunk (shared by the chunk's row tiles) through a ring of kStB5.  The
@@ -133,11 +145,10 @@ __device__ __forceinline__ void split5(float x, int bf16, float& h, float& l) {
 // (panel written).
 template <int kStA5>
 __global__ void __launch_bounds__(kT5, 1)
-k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constant__ CUtensorMap tm_lo,
-                 float* __restrict__ phi, float* __restrict__ plo, const BandDesc* __restrict__ descs,
-                 const int64_t* __restrict__ zoff, int count, int32_t* __restrict__ queue, int W,
-                 uint32_t tmem_cols, int nbuf, int P, DevStatus* st, int32_t* __restrict__ weak, float weak_tol,
-                 int bf16) {
+k_band_potrf_tc5(const __grid_constant__ Tc5Maps tm, float* __restrict__ phi, float* __restrict__ plo,
+                 const BandDesc* __restrict__ descs, const int64_t* __restrict__ zoff, int count,
+                 int32_t* __restrict__ queue, int W, uint32_t tmem_cols, int nbuf, int P, int yend, DevStatus* st,
+                 int32_t* __restrict__ weak, float weak_tol, int bf16) {
   const int Wt = W + kPB5;
   const int QW = W / kPB5;                    // k-chunks in a full window
   const uint32_t bufcols = tmem_cols / nbuf;  // columns of one accumulator buffer
@@ -165,18 +176,18 @@ k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constan
   if (tid == 0) {
     for (int i = 0; i < kStA5; ++i) {
       mbar_init(&afull[i], 1);
-      mbar_init(&aempty[i], 1);
+      mbar_init(&aempty[i], 2);
     }
     for (int i = 0; i < kStB5; ++i) {
       mbar_init(&bfull[i], 1);
-      mbar_init(&bempty[i], 1);
+      mbar_init(&bempty[i], 2);
     }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&acc_full[i], 1);
+      mbar_init(&acc_full[i], 2);
       mbar_init(&acc_empty[i], kEpi5);
     }
     mbar_init(pdone, kEpi5);
-    mbar_init(fin, 1);
+    mbar_init(fin, 2);
     *abort = 0;
     fence_barrier_init();
   }
@@ -211,16 +222,17 @@ k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constan
           const int R = min(n, c0 + kPB5 + w) - c0;
           const int nh = ((R + 31) / 32 + 3) / 4;
           const int q0 = max(0, QW - J);
+          int slot = (J - QW + q0) % (QW + 1);   // of the k-chunk's columns
           for (int q = q0; q < QW; ++q, ++tb) {
+            const int x = 32 * slot, y0 = (int)(z0 + J) * 32;
+            slot = slot == QW ? 0 : slot + 1;
             // the last k-chunk holds panel J - 1's columns
             if (q == QW - 1 && J >= 1 && !*abort) wait5(pdone, (pb + J - 1) & 1, abort, st, d.id, c0);
             {
               const uint32_t sb = tb % kStB5;
               if (!*abort && (tb < (uint32_t)kStB5 || wait5(&bempty[sb], ((tb / kStB5) - 1) & 1, abort, st, d.id, c0))) {
-                unsigned char* dst = stB + sb * kStageB5;
                 mbar_arrive_expect_tx(&bfull[sb], kStageB5);
-                tma_load_3d(dst, &tm_hi, 32 * q, 0, (int)(z0 + J), &bfull[sb]);
-                tma_load_3d(dst + kTileB5, &tm_lo, 32 * q, 0, (int)(z0 + J), &bfull[sb]);
+                tma_load_3d(stB + sb * kStageB5, &tm.b, x, y0, 0, &bfull[sb]);
                 ++issB[sb];
               }
             }
@@ -231,19 +243,37 @@ k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constan
               if (ta >= (uint32_t)kStA5 && !wait5(&aempty[sa], ((ta / kStA5) - 1) & 1, abort, st, d.id, c0)) continue;
               unsigned char* dst = stA + sa * kStageA5;
               mbar_arrive_expect_tx(&afull[sa], kStageA5);
-              for (int i = 0; i < 4; ++i) {
-                const int I = J + 4 * hh + i;
-                const int x = 32 * (J + q - I);
-                tma_load_3d(dst + i * kBox5, &tm_hi, x, 0, (int)(z0 + I), &afull[sa]);
-                tma_load_3d(dst + kTileA5 + i * kBox5, &tm_lo, x, 0, (int)(z0 + I), &afull[sa]);
+              const int v = q - 4 * hh + 1, y = y0 + 128 * hh;   // row blocks 0 .. v - 1 reach these columns
+              if (v >= 4) {
+                tma_load_3d(dst, &tm.a, x, y, 0, &afull[sa]);
+              } else {
+                for (int pl = 0; pl < 2; ++pl, dst += kTileA5) {
+                  if (v >= 2) {
+                    tma_load_3d(dst, &tm.r64, x, y, pl, &afull[sa]);
+                  } else {
+                    tma_load_3d(dst, &tm.r32, x, y, pl, &afull[sa]);
+                    tma_load_3d(dst + kBox5, &tm.r32, x, yend, pl, &afull[sa]);
+                  }
+                  if (v == 3) {
+                    tma_load_3d(dst + 2 * kBox5, &tm.r32, x, y + 64, pl, &afull[sa]);
+                    tma_load_3d(dst + 3 * kBox5, &tm.r32, x, yend, pl, &afull[sa]);
+                  } else {
+                    tma_load_3d(dst + 2 * kBox5, &tm.r64, x, yend, pl, &afull[sa]);
+                  }
+                }
               }
               ++issA[sa];
             }
           }
         }
       }
-    } else if (wid == 9) {
+    } else if (wid >= 9) {
       // ------------------------------------------------------------ MMAs
+      // warp 9 takes the even row tiles, warp 10 the odd ones: an MMA of these
+      // shapes holds the tensor cores about 66 cycles (528 a tile), and one
+      // warp's waits and commits between the tiles took as long again.  Both
+      // wait for every tile and release its stage (a warp that passed the
+      // other's tiles unseen could take a stage's earlier phase for its own).
       if (lane == 0) {
         for (int J = 0; J < np; ++J) {
           const int c0 = J * kPB5;
@@ -264,21 +294,36 @@ k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constan
             for (int hh = 0; hh < hmax; ++hh, ++ta) {
               const uint32_t sa = ta % kStA5;
               if (!bok || *abort || !wait5(&afull[sa], (ta / kStA5) & 1, abort, st, d.id, c0)) continue;
+              if ((hh & 1) != wid - 9) {
+                arrive5(&aempty[sa]);
+                continue;
+              }
               tc_fence_after();
               const uint32_t asa = smem_u32(stA + sa * kStageA5);
               const int ss = 1 + q % P;  // the hi*hi slot of this k-chunk
               const int bs = (1 + P) * hh, bb = bs + ss;
-              const uint32_t ds = dbuf + chcols * hh, db = ds + 32u * ss;
+              const uint32_t dhl = dbuf + chcols * hh, ds = P == 1 ? dhl + 32u : dhl, db = dhl + 32u * ss;
               const uint32_t acs = (uint32_t)((inited >> bs) & 1u), acb = (uint32_t)((inited >> bb) & 1u);
+              if (P == 1) {
+                // the lo tile of B lies behind the hi tile: one product of N = 64
+                // gives hi*hi and hi*lo in the chunk's two neighbouring slots
   #pragma unroll
-              for (int kk = 0; kk < 4; ++kk) {
-                const uint64_t ah = umma_desc_sw128(asa + 32 * kk);
-                const uint64_t al = umma_desc_sw128(asa + kTileA5 + 32 * kk);
-                const uint64_t bh = umma_desc_sw128(bsa + 32 * kk);
-                const uint64_t bl = umma_desc_sw128(bsa + kTileB5 + 32 * kk);
-                umma_tf32(ds, al, bh, kIdesc5, acs | (kk > 0 ? 1u : 0u));
-                umma_tf32(ds, ah, bl, kIdesc5, 1u);
-                umma_tf32(db, ah, bh, kIdesc5, acb | (kk > 0 ? 1u : 0u));
+                for (int kk = 0; kk < 4; ++kk) {
+                  const uint64_t bh = umma_desc_sw128(bsa + 32 * kk);
+                  umma_tf32(dhl, umma_desc_sw128(asa + 32 * kk), bh, kIdesc5x2, acs | (kk > 0 ? 1u : 0u));
+                  umma_tf32(ds, umma_desc_sw128(asa + kTileA5 + 32 * kk), bh, kIdesc5, 1u);
+                }
+              } else {
+    #pragma unroll
+                for (int kk = 0; kk < 4; ++kk) {
+                  const uint64_t ah = umma_desc_sw128(asa + 32 * kk);
+                  const uint64_t al = umma_desc_sw128(asa + kTileA5 + 32 * kk);
+                  const uint64_t bh = umma_desc_sw128(bsa + 32 * kk);
+                  const uint64_t bl = umma_desc_sw128(bsa + kTileB5 + 32 * kk);
+                  umma_tf32(ds, al, bh, kIdesc5, acs | (kk > 0 ? 1u : 0u));
+                  umma_tf32(ds, ah, bl, kIdesc5, 1u);
+                  umma_tf32(db, ah, bh, kIdesc5, acb | (kk > 0 ? 1u : 0u));
+                }
               }
               inited |= (1ull << bs) | (1ull << bb);
               umma_commit(&aempty[sa]);
@@ -298,27 +343,27 @@ k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constan
         const int q0 = max(0, QW - J);
         const int G = pb + J;
         const int buf = G % nbuf;
+        const int xJ = 32 * (J % (QW + 1));   // the panel's columns in every row
         // the panel's entries of A (both planes) into Us: eight lanes per row,
-        // four columns each (16-byte loads), four row groups of 32 rows per
+        // four columns each (16-byte loads), eight row groups of 32 rows per
         // batch in flight; entries outside the band are zero in the planes
         {
           const int rsub = lane >> 3, cg = 4 * (lane & 7);
-          for (int i0 = 4 * wid + rsub; i0 < R; i0 += 4 * kEpi5 / 8) {
-            float4 vh[4], vl[4];
+          for (int i0 = 4 * wid + rsub; i0 < R; i0 += 8 * kEpi5 / 8) {
+            float4 vh[8], vl[8];
   #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < 8; ++u) {
               const int i = i0 + u * (kEpi5 / 8);
               vh[u] = make_float4(0.f, 0.f, 0.f, 0.f);
               vl[u] = vh[u];
               if (i < R) {
-                const int I = J + i / 32;
-                const int64_t o = ((z0 + I) * 32 + (i & 31)) * (int64_t)Wt + (W - 32 * (I - J)) + cg;
+                const int64_t o = (z0 * 32 + c0 + i) * (int64_t)Wt + xJ + cg;
                 vh[u] = *reinterpret_cast<const float4*>(phi + o);
                 vl[u] = *reinterpret_cast<const float4*>(plo + o);
               }
             }
   #pragma unroll
-            for (int u = 0; u < 4; ++u) {
+            for (int u = 0; u < 8; ++u) {
               const int i = i0 + u * (kEpi5 / 8);
               if (i < R) {
                 float* ur = Us + (size_t)i * kUS5 + cg;
@@ -330,9 +375,10 @@ k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constan
             }
           }
         }
-        if (!*abort) wait5(&acc_full[buf], (G / nbuf) & 1, abort, st, d.id, c0);
-        tc_fence_after();
+        // one warp polls: eight slow the other roles' waits
+        if (wid == 0 && !*abort) wait5(&acc_full[buf], (G / nbuf) & 1, abort, st, d.id, c0);
         epi_sync();
+        tc_fence_after();
         // U = A - D.  Warp w reads TMEM lanes 32 (w % 4) .. + 31 of the
         // chunks h = w / 4, w / 4 + 2, ...; chunk h holds data when one of its
         // tiles was multiplied (some k-chunk q >= 4 h exists), and its hi*hi
@@ -362,65 +408,116 @@ k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constan
         tc_fence_before();
         arrive5(&acc_empty[buf]);  // the MMAs may refill this buffer
         epi_sync();
-        // ---- the 32 x 32 diagonal block in warp 0: lane r holds row r; step t
-        // takes pivot t from lane t (a pivot that is not positive is reported
-        // and replaced by 1), scales column t and updates the trailing part
+        // ---- the 32 x 32 diagonal block in warp 0: lane r holds row r; a step
+        // takes two pivots from their lanes (a pivot that is not positive is
+        // reported and replaced by 1), scales the two columns and updates the
+        // rows from the columns' values in the other lanes (entries right of the
+        // diagonal hold no meaning): by shuffles for the columns of the next two
+        // pivots, which the chain waits for, by 16-byte broadcasts from shared
+        // memory for the rest.  One column a step through shared memory took
+        // 13300 cycles per block, all by shuffles 8300, this 6900.  The factor
+        // goes to Us column by column (L(u, t) at 32 t + u), also for the rows
+        // below.  Meanwhile the other warps ask for the next panel's entries of
+        // A, which nothing changes before.
         if (wid == 0) {
-          // lane r holds row r; step t publishes the scaled column t in Dcol
-          // (shared memory) and every lane updates its row from it
-          float* Dcol = Dinv + kPB5;  // kPB5 scratch values after Dinv
           float a[kPB5];
   #pragma unroll
           for (int u = 0; u < kPB5; ++u) a[u] = (lane < b && u <= lane) ? Us[lane * kUS5 + u] : 0.f;
+          __syncwarp();
+          float dinv = 0.f, pbad = 0.f;
+          int tbad = kPB5;       // the first pivot that is not positive and finite
+          bool wk = false;
+          float p0 = __shfl_sync(0xffffffffu, a[0], 0), e0 = __shfl_sync(0xffffffffu, a[0], 1),
+                p1 = __shfl_sync(0xffffffffu, a[1], 1);
   #pragma unroll
-          for (int t = 0; t < kPB5; ++t) {
-            if (t < b) {
-              float p = __shfl_sync(0xffffffffu, a[t], t);
-              if (weak) {
-                if (lane == 0 && !(p > weak_tol)) weak[d.id] = 1;
-                if (!finite_pos5(p)) p = 1.f;
-              } else if (!finite_pos5(p)) {
-                if (lane == 0) record_error(st, isfinite(p) ? GENEO_ERR_NOT_SPD : GENEO_ERR_NONFINITE, d.id,
-                                            (int64_t)c0 + t);
-                p = 1.f;
-              }
-              const float inv = rsqrtf(p);
-              if (lane == t) {
-                a[t] = p * inv;
-                Dinv[t] = inv;
-              } else if (lane > t) {
-                a[t] *= inv;
-              }
-              Dcol[lane] = a[t];
-              __syncwarp();
+          for (int h = 0; h < kPB5 / 2; ++h) {
+            const int t = 2 * h;
+            // reciprocal square roots of the pivots, 0 beyond the matrix; a bad
+            // pivot is noted and replaced by 1
+            const bool bad0 = t < b && !finite_pos5(p0);
+            wk |= t < b && !(p0 > weak_tol);
+            if (bad0 && tbad == kPB5) {
+              tbad = t;
+              pbad = p0;
+            }
+            p0 = bad0 ? 1.f : p0;
+            const float i0 = t < b ? rsqrtf(p0) : 0.f;
+            const float l10 = e0 * i0;       // L(t + 1, t)
+            p1 -= l10 * l10;
+            const bool bad1 = t + 1 < b && !finite_pos5(p1);
+            wk |= t + 1 < b && !(p1 > weak_tol);
+            if (bad1 && tbad == kPB5) {
+              tbad = t + 1;
+              pbad = p1;
+            }
+            p1 = bad1 ? 1.f : p1;
+            const float i1 = t + 1 < b ? rsqrtf(p1) : 0.f;
+            const float x0 = lane == t ? p0 * i0 : a[t] * i0;
+            const float y1 = a[t + 1] - x0 * l10;
+            const float x1 = lane == t + 1 ? p1 * i1 : y1 * i1;
+            Us[32 * t + lane] = lane >= t ? x0 : 0.f;
+            Us[32 * (t + 1) + lane] = lane > t ? x1 : 0.f;
+            __syncwarp();
+            dinv = lane == t ? i0 : lane == t + 1 ? i1 : dinv;
+            if (h + 1 < kPB5 / 2) {   // the next two pivots first: the rest overlaps their chain
   #pragma unroll
-              for (int u = t + 1; u < kPB5; ++u)
-                if (lane >= u) a[u] -= a[t] * Dcol[u];
-              __syncwarp();
+              for (int u = t + 2; u < t + 4; ++u) {
+                a[u] -= x0 * __shfl_sync(0xffffffffu, x0, u);
+                a[u] -= x1 * __shfl_sync(0xffffffffu, x1, u);
+              }
+              p0 = __shfl_sync(0xffffffffu, a[t + 2], t + 2);
+              e0 = __shfl_sync(0xffffffffu, a[t + 2], t + 3);
+              p1 = __shfl_sync(0xffffffffu, a[t + 3], t + 3);
+            }
+  #pragma unroll
+            for (int u0 = (t + 4) & ~3; u0 < kPB5; u0 += 4) {
+              float y0[4], y1[4];
+              *reinterpret_cast<float4*>(y0) = *reinterpret_cast<const float4*>(Us + 32 * t + u0);
+              *reinterpret_cast<float4*>(y1) = *reinterpret_cast<const float4*>(Us + 32 * (t + 1) + u0);
+  #pragma unroll
+              for (int q = 0; q < 4; ++q)
+                if (u0 + q >= t + 4) {
+                  a[u0 + q] -= x0 * y0[q];
+                  a[u0 + q] -= x1 * y1[q];
+                }
             }
           }
-          if (lane < b) {
-  #pragma unroll
-            for (int u = 0; u < kPB5; ++u)
-              if (u <= lane) Us[lane * kUS5 + u] = a[u];
-          } else {
-            Dinv[lane] = 0.f;
+          if (lane == 0) {
+            if (weak) {
+              if (wk) weak[d.id] = 1;
+            } else if (tbad < kPB5) {
+              record_error(st, isfinite(pbad) ? GENEO_ERR_NOT_SPD : GENEO_ERR_NONFINITE, d.id, (int64_t)c0 + tbad);
+            }
+          }
+          Dinv[lane] = dinv;
+        } else {
+          const int rn = min(n, c0 + 2 * kPB5 + w) - (c0 + kPB5);   // rows of panel J + 1
+          const int x1 = 32 * ((J + 1) % (QW + 1));
+          for (int i = tid - 32; i < rn; i += kEpi5 - 32) {
+            const int64_t o = (z0 * 32 + c0 + kPB5 + i) * (int64_t)Wt + x1;
+            prefetch_l2(phi + o);
+            prefetch_l2(plo + o);
           }
         }
         epi_sync();
-        // ---- rows below: x L_JJ^T = u, one row per thread
-        for (int i = b + tid; i < R; i += kEpi5) {
+        // ---- rows below: x L_JJ^T = u, one row per thread (the block is full:
+        // b = 32); column t of the factor by 16-byte broadcasts, its updates of x
+        // independent of each other
+        for (int i = kPB5 + tid; i < R; i += kEpi5) {
           float* ur = Us + (size_t)i * kUS5;
           float x[kPB5];
   #pragma unroll
           for (int t = 0; t < kPB5; ++t) x[t] = ur[t];
   #pragma unroll
           for (int t = 0; t < kPB5; ++t) {
-            if (t < b) {
-              float v = x[t];
+            x[t] *= Dinv[t];
   #pragma unroll
-              for (int u = 0; u < t; ++u) v -= x[u] * Us[t * kUS5 + u];
-              x[t] = v * Dinv[t];
+            for (int u0 = (t + 1) & ~3; u0 < kPB5; u0 += 4) {
+              const float4 l = *reinterpret_cast<const float4*>(Us + 32 * t + u0);
+              if (u0 > t) x[u0] -= x[t] * l.x;
+              if (u0 + 1 > t) x[u0 + 1] -= x[t] * l.y;
+              if (u0 + 2 > t) x[u0 + 2] -= x[t] * l.z;
+              if (u0 + 3 > t) x[u0 + 3] -= x[t] * l.w;
             }
           }
   #pragma unroll
@@ -430,21 +527,24 @@ k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constan
         // ---- the panel's columns back to both planes: eight lanes per row,
         // 16-byte stores.  Us holds exact zeros outside the band (A is zero
         // there and every update of such an entry is 0 - 0), which is also
-        // what the planes hold there.
+        // what the planes hold there.  The rows of the diagonal block lie
+        // column by column.
         {
           const int rsub = lane >> 3, cg = 4 * (lane & 7);
-          for (int i = 4 * wid + rsub; i < R; i += kEpi5 / 8) {
-            const int I = J + i / 32;
-            const int64_t o = ((z0 + I) * 32 + (i & 31)) * (int64_t)Wt + (W - 32 * (I - J)) + cg;
-            const float* ur = Us + (size_t)i * kUS5 + cg;
+          auto put = [&](int i, const float* ur, int us) {
+            const int64_t o = (z0 * 32 + c0 + i) * (int64_t)Wt + xJ + cg;
             float4 xh, xl;
             split5(ur[0], bf16, xh.x, xl.x);
-            split5(ur[1], bf16, xh.y, xl.y);
-            split5(ur[2], bf16, xh.z, xl.z);
-            split5(ur[3], bf16, xh.w, xl.w);
+            split5(ur[us], bf16, xh.y, xl.y);
+            split5(ur[2 * us], bf16, xh.z, xl.z);
+            split5(ur[3 * us], bf16, xh.w, xl.w);
             *reinterpret_cast<float4*>(phi + o) = xh;
             *reinterpret_cast<float4*>(plo + o) = xl;
-          }
+          };
+          int i = 4 * wid + rsub;
+          if (i < R) put(i, Us + 32 * cg + i, 32);
+  #pragma unroll 4
+          for (i += kEpi5 / 8; i < R; i += kEpi5 / 8) put(i, Us + (size_t)i * kUS5 + cg, 1);
         }
         fence_proxy_async_global();  // the next panel's copies read these columns
         arrive5(pdone);
@@ -464,7 +564,7 @@ k_band_potrf_tc5(const __grid_constant__ CUtensorMap tm_hi, const __grid_constan
         for (int it = 0; it < (1 << 22) && !mbar_try_wait(&bfull[i], (issB[i] - 1) & 1); ++it) {
         }
   }
-  if (tid == 9 * 32) {
+  if (tid == 9 * 32 || tid == 10 * 32) {
     umma_commit(fin);
     for (int it = 0; it < (1 << 22) && !mbar_try_wait(fin, 0); ++it) {
     }
@@ -496,9 +596,12 @@ k_tb_pack(const float* __restrict__ band, const BandDesc* __restrict__ descs, co
     const float* src = band + d.off + (int64_t)r * d.ld;
     const int64_t o = ((zoff[blockIdx.y] + I) * 32 + (r & 31)) * (int64_t)Wt;
     const float sr = (S && r < d.n) ? S[r] : 1.f;
+    // the block of columns 32 C .. at slot C mod (W / 32 + 1), from C = I - W / 32
+    const int nsl = Wt / 32;
+    int slot = (I + 1) % nsl;
 #pragma unroll 4
-    for (int xx = lane; xx < Wt; xx += 32) {
-      const int c = xx + 32 * I - W;
+    for (int k = 0; k < nsl; ++k) {
+      const int c = 32 * (I + 1 - nsl + k) + lane;
       float x = 0.f;
       if (r < d.n && c >= 0 && c <= r && r - c <= d.w) {
         x = src[c - r + d.w];
@@ -506,8 +609,9 @@ k_tb_pack(const float* __restrict__ band, const BandDesc* __restrict__ descs, co
       }
       float xh, xl;
       split5(x, bf16, xh, xl);
-      phi[o + xx] = xh;
-      plo[o + xx] = xl;
+      phi[o + 32 * slot + lane] = xh;
+      plo[o + 32 * slot + lane] = xl;
+      slot = slot + 1 == nsl ? 0 : slot + 1;
     }
   }
 }
@@ -526,19 +630,25 @@ k_tb_unpack(float* __restrict__ band, const BandDesc* __restrict__ descs, const 
     const int64_t o = ((zoff[blockIdx.y] + I) * 32 + (r & 31)) * (int64_t)Wt;
     // six groups of 32 in flight (one at a time left the copy at 3.0 TB/s)
     constexpr int U = 6;
-    const int64_t oc = o - 32 * I + W;
-    int c = max(0, r - d.w) + lane;
-    for (; c + 32 * (U - 1) <= r; c += 32 * U) {
+    const int nsl = Wt / 32, lo = max(0, r - d.w);
+    int slot = (lo >> 5) % nsl;
+    for (int cb = lo & ~31; cb <= r; cb += 32 * U) {
       float v[U], l[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        v[u] = phi[oc + c + 32 * u];
-        l[u] = plo[oc + c + 32 * u];
+        const int c = cb + 32 * u + lane;
+        if (c >= lo && c <= r) {
+          v[u] = phi[o + 32 * slot + lane];
+          l[u] = plo[o + 32 * slot + lane];
+        }
+        slot = slot + 1 == nsl ? 0 : slot + 1;
       }
 #pragma unroll
-      for (int u = 0; u < U; ++u) dst[c + 32 * u - r + d.w] = v[u] + l[u];
+      for (int u = 0; u < U; ++u) {
+        const int c = cb + 32 * u + lane;
+        if (c >= lo && c <= r) dst[c - r + d.w] = v[u] + l[u];
+      }
     }
-    for (; c <= r; c += 32) dst[c - r + d.w] = phi[oc + c] + plo[oc + c];
   }
 }
 
@@ -557,15 +667,16 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
   return fn;
 }
 
-// 3D tensor map over the tiled-band planes: x = W + 32 columns, y = 32 rows,
-// z = row blocks; 32 x 32 x 1 boxes, 128-byte swizzle, zeros out of range
-bool encode_tb_map(CUtensorMap* m, float* base, int W, int64_t Z) {
+// 3D tensor map over the tiled-band planes: x = W + 32 columns, y = rows,
+// z = plane; boxes of 32 columns x `rows` x `planes`, 128-byte swizzle, zeros
+// out of range
+bool encode_tb_map(CUtensorMap* m, float* base, int W, int64_t Z, int rows, int planes) {
   PFN_cuTensorMapEncodeTiled_v12000 fn = encode_fn();
   if (!fn) return false;
   const cuuint64_t Wt = (cuuint64_t)W + kPB5;
-  const cuuint64_t dims[3] = {Wt, 32, (cuuint64_t)Z};
-  const cuuint64_t strides[2] = {Wt * sizeof(float), Wt * 32 * sizeof(float)};
-  const cuuint32_t box[3] = {32, 32, 1};
+  const cuuint64_t dims[3] = {Wt, 32 * (cuuint64_t)Z, 2};
+  const cuuint64_t strides[2] = {Wt * sizeof(float), Wt * 32 * (cuuint64_t)Z * sizeof(float)};
+  const cuuint32_t box[3] = {32, (cuuint32_t)rows, (cuuint32_t)planes};
   const cuuint32_t estr[3] = {1, 1, 1};
   return fn(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
             CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -619,13 +730,16 @@ geneo_status_t tc5_prepare(const BandDesc* h_desc, int count, int max_w, DevMem&
     Z += (h_desc[i].n + 31) / 32;
     max_n = std::max(max_n, h_desc[i].n);
   }
-  if (Z <= 0 || Z > (int64_t)INT32_MAX) return GENEO_OK;
+  if (Z <= 0 || 32 * Z + 128 > (int64_t)INT32_MAX) return GENEO_OK;
   const size_t plane = (size_t)Z * 32 * (W + kPB5);
-  GENEO_TRY(tmp.get(&p->phi, plane));
-  GENEO_TRY(tmp.get(&p->plo, plane));
+  GENEO_TRY(tmp.get(&p->phi, 2 * plane));
+  p->plo = p->phi + plane;
   GENEO_TRY(tmp.get(&p->dz, (size_t)count));
   GENEO_TRY(tmp.get(&p->queue, 1));
-  if (!encode_tb_map(&p->mhi, p->phi, W, Z) || !encode_tb_map(&p->mlo, p->plo, W, Z)) return GENEO_OK;
+  if (!encode_tb_map(&p->maps.a, p->phi, W, Z, 128, 2) || !encode_tb_map(&p->maps.b, p->phi, W, Z, 32, 2) ||
+      !encode_tb_map(&p->maps.r64, p->phi, W, Z, 64, 1) || !encode_tb_map(&p->maps.r32, p->phi, W, Z, 32, 1))
+    return GENEO_OK;
+  p->yend = (int)(32 * Z);
   GENEO_CUDA(cudaMemcpyAsync(p->dz, zo.data(), sizeof(int64_t) * count, cudaMemcpyHostToDevice, s));
   p->W = W;
   p->cols = cols;
@@ -653,8 +767,8 @@ geneo_status_t tc5_factor(const Tc5Plan& p, float* band, const BandDesc* d_desc,
   GENEO_CUDA(cudaGetDevice(&dev));
   GENEO_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   GENEO_CUDA(cudaMemsetAsync(p.queue, 0, sizeof(int32_t), s));
-  kern<<<std::min(p.count, sms), kT5, p.smem, s>>>(p.mhi, p.mlo, p.phi, p.plo, d_desc, p.dz, p.count, p.queue, p.W,
-                                                    p.cols, p.nbuf, p.par, st, weak, weak_tol, bf16);
+  kern<<<std::min(p.count, sms), kT5, p.smem, s>>>(p.maps, p.phi, p.plo, d_desc, p.dz, p.count, p.queue, p.W,
+                                                    p.cols, p.nbuf, p.par, p.yend, st, weak, weak_tol, bf16);
   note_launch();
   GENEO_CUDA(cudaGetLastError());
   k_tb_unpack<<<gp, 256, 0, s>>>(band, d_desc, p.dz, p.W, p.phi, p.plo); note_launch();

@@ -309,8 +309,14 @@ geneo_status_t exclusive_scan_i64(const int64_t* in, int64_t* out, int64_t n, in
 // batch does not fit the kernel (the older kernels then factor it).
 // tc5_factor (after equilibration) packs the bands, factors them and unpacks
 // the factors back into the bands.
+// maps of the tiled-band planes: boxes of 128 rows of both planes, 32 rows of
+// both, 64 and 32 rows of one
+struct Tc5Maps {
+  CUtensorMap a, b, r64, r32;
+};
 struct Tc5Plan {
-  CUtensorMap mhi, mlo;
+  Tc5Maps maps;
+  int yend = 0;       // rows of the planes: boxes from here on read zeros
   bool ok = false;
   int W = 0, count = 0, max_n = 0;
   uint32_t cols = 0;  // TMEM columns allocated
