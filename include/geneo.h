@@ -204,7 +204,7 @@ typedef struct {
  *  autotune   1 (default): at the end of the first setup of each batch
  *             shape (precision, largest A_j band width and order, number of
  *             subdomains) in the process, the preconditioner's local solve
- *             is timed at each pipeline depth on a scratch vector and the
+ *             is timed at each pipeline depth (2 to 4 row slots) on a scratch vector and the
  *             fastest is kept for every later apply (reported in
  *             geneo_coarse_info_t.local_solve_stages); 0: the depth follows
  *             from shared memory alone.

@@ -5,7 +5,8 @@
 // (Section 4.4) and the coarse matrix A_H (Section 4.5) are all banded in the
 // natural (lexicographic) dof order of a box subdomain, so one banded kernel
 // family serves all three.  One thread block owns one matrix; the batch is
-// the grid.  Storage: lower band by rows (BandDesc in common.cuh).
+// the grid (FP64 batches smaller than the GPU: every panel over all SMs, below).
+// Storage: lower band by rows (BandDesc in common.cuh).
 //
 // Factorisation (right-looking, block width NB): per step the NB x NB
 // diagonal block is factored by one warp, the panel rows below are solved
@@ -14,7 +15,8 @@
 // are not positive are reported (GENEO_ERR_NOT_SPD) and replaced by 1 so the
 // kernel always finishes.
 //
-// Solves (L L^T x = b, in place): the factor is streamed block row by block
+// The solves run in sweep.cu; what follows is the kernel for bands too wide for
+// its row blocks.  L L^T x = b, in place: the factor is streamed block row by block
 // row (SNB rows, one contiguous chunk) into shared memory by bulk copies on
 // an mbarrier pipeline.  The forward sweep is left-looking (each new row is
 // a dot product with the last w solved rows, kept in a shared ring), the
@@ -252,7 +254,8 @@ k_band_panel_diag(T* __restrict__ base, const BandDesc* __restrict__ descs, int 
           p = T(1);
         }
         // one reciprocal square root instead of a square root and a division:
-        // both are long dependent chains on the FP64 pipe (66 -> 30 us a panel)
+        // both are long dependent chains on the FP64 pipe (66 -> 41 us
+        // a panel of 27 bands of half width 463, 46 -> 20 us of narrower ones)
         const T r = rsqrt(p);
         a[t >> 2] = lane == t ? p * r : lane > t ? a[t >> 2] * r : T(0);
         col[t & 1][lane] = a[t >> 2];
@@ -1014,7 +1017,7 @@ geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w,
   // FP64 bands too few for one SM each: every panel's work spread over the GPU.
   // Both sides in units of 32^3 / 2 multiply-adds: one block per matrix runs the
   // widest alone on its SM; spread, a panel's three launches cost about 75 us
-  // (measured: 20 + 24 + 3 x 4 beside the update) whatever the batch
+  // (measured: 20 to 41 + 24 to 28, and the gaps) whatever the batch
   if constexpr (sizeof(T) == 8) {
     if (!weak && max_n > 256 && max_w >= 96) {
       const double panel = 0.5 * (double)max_w * max_w * kPN;          // multiply-adds of one panel's update

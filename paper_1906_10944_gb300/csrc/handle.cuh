@@ -51,7 +51,7 @@ struct geneo_handle_s {
   std::vector<uint8_t> a64;        // [N] 1: A_j factored in FP64
   int nK64 = 0;                    // the same count for K_j (setup only)
   int factor_classes = 0;          // FP32: factorisation batches (size classes) of K_j and A_j
-  int local_stages = 0;            // pipeline depth of the local solve picked by the autotuner
+  int local_stages = 0;            // row slots of the local solve picked by the autotuner
 
   // coarse space
   int dimH = 0, wH = 0;

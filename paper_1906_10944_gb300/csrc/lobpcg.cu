@@ -89,7 +89,7 @@ ColRefT<S> cref(S* base, int W, int c0, const int32_t* c0d, int w, const int32_t
 // SHARED: a block's kT rows and w columns are cut into units of 32 rows x 4
 // columns, one warp each, the column groups of a row chunk on neighbouring
 // warps, so that all but the first take the entries from L1 (one thread per row
-// reads them again from L2 or HBM for every four columns: elasticity 38^3, 81
+// reads them again from L2 or HBM for every four columns: elasticity 38x31x24, 81
 // entries a row, 442 MB for each of six passes; k_spmm_ds 558 -> 546 us).
 // Otherwise one thread per row loops over the columns: short rows stay in L1 by
 // themselves, and the warps of a block, at the same columns, share more of the

@@ -10,8 +10,8 @@
 //   4. per global dof k (gather form over the subdomains whose D contains k):
 //      z_k = sum_j (u_j[k] + Z_j[k, :] y_j); z_k = r_k on global Dirichlet dofs.
 // PCG (Section 5): x0 = 0, stop when ||r||_2 <= tol ||b||_2; all dot
-// products are two-stage fixed-order reductions, so iterates are bitwise
-// reproducible run to run.
+// products are two-stage fixed-order reductions (the last block sums the
+// partials), so iterates are bitwise reproducible run to run.
 #include <algorithm>
 #include <cmath>
 #include <map>
@@ -400,7 +400,7 @@ __global__ void k_update_p(int64_t n, const double* __restrict__ scal, const dou
 // slots, and the scalar updates are folded into the kernels that use them,
 // so an iteration needs four launches besides the preconditioner instead of
 // seven.  Slots (parity p = iteration & 1): RZ[p] = 8 + p, PQ[p] = 10 + p,
-// RR[p] = 12 + p; flag 6 as in k_finish.
+// RR[p] = 12 + p; flag 6 as in finish_step.
 // ---------------------------------------------------------------------------
 constexpr int kRZ = 8, kPQ = 10, kRR = 12;
 
@@ -526,10 +526,9 @@ double condition_estimate_fixed(const double* a, const double* b, int m, double*
   return ext[1] / ext[0];
 }
 
-// Autotuner of the preconditioner's local solve (the one-right-hand-side
-// band solve with the vector resident in shared memory): each pipeline
-// depth (2, 3, 4 stages; deeper stages take more shared memory and so fewer
-// blocks per SM) is timed on this batch, on a scratch copy of the subdomain
+// Autotuner of the preconditioner's local solve (the one-right-hand-side band
+// sweep): each depth of its copy pipeline (2, 3 or 4 row slots; more slots take
+// more shared memory and may leave fewer blocks per SM) is timed on this batch, on a scratch copy of the subdomain
 // vectors, and the fastest is kept for the process, keyed by (precision,
 // largest band width, largest order, batch size).  The depths are timed in
 // turn, four rounds after a warm-up launch of each, one launch per CUDA-event

@@ -147,7 +147,7 @@ k_dot_cols(int64_t n, const double* __restrict__ A, const double* __restrict__ B
 }
 
 // per column (block c): the sum of its partials, then the scalar step `what`
-// (as k_finish in solve.cu); inactive columns keep alpha = 0
+// (as finish_step in solve.cu); inactive columns keep alpha = 0
 __global__ void k_finish_cols(const double* __restrict__ part, double* __restrict__ scal, int what,
                               double* __restrict__ hist_a, double* __restrict__ hist_b, int hcap, int it) {
   __shared__ double red[kT / 32];

@@ -16,7 +16,9 @@
 //  forward: the owner has summed L(k, j) y_j over all older j while the chain
 //    ran elsewhere; when y_{k-1} arrives it adds that product, applies the
 //    inverted diagonal block and stores y_k into the ring of solved rows of
-//    every block of the cluster (st.async on the receivers' mbarriers).
+//    every block of the cluster.  A value is its own flag: the receiver clears
+//    the slot to a NaN pattern no computation gives and polls for anything else
+//    (an mbarrier per message cost a link about 170 cycles more).
 //  backward: the owner of k gathers the other blocks' partial sums
 //    sum_r L(r, k)^T x_r from its mailbox, applies the transposed inverse,
 //    then computes its contribution to block k - 1 first and sends it on;
@@ -26,6 +28,14 @@
 // column phase) thread; several, FP32 factors: m16n8k8 TF32 MMAs in one or
 // three passes; several, FP64 factors: FP64 or double-single
 // multiply-adds, a register tile of NC columns per thread.
+//
+// Measured against one thread block per matrix in 16-row steps of forward
+// substitution: one column of 64 FP32 bands of order 5832, half width 340,
+// 785 -> 267 us; a solve with the 8 bands of a 32^3 grid 24.4 -> 6.7 ms; an FP64
+// apply at 64^3 2.9 -> 1.4 ms; the eigensolver's sweeps at 48^3 in FP64 (11
+// columns, 27 bands) 653 -> 138 ms, where the FP64 pipe bounds them.  With more
+// matrices than SMs HBM bounds the one-column sweep (512 bands of a 128^3 grid,
+// 1.69 ms for 9.23 GB: 5.5 TB/s).
 //
 // All sums run in a fixed order.  Every wait is bounded; a wait that gives up
 // records GENEO_ERR_TIMEOUT and the block goes on without waiting.
@@ -543,8 +553,6 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
       csync<kThreads>();
     }
   };
-  // receivers of this lane's solved value: the blocks rank + 1 + ph + PH i
-  // (NC = 1; the lanes of a row share them) or all others
   const uint32_t win_at = smem_u32(win);
 
   // ------------------------------------------------------------- forward
@@ -856,7 +864,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
 // ---------------------------------------------------------------------------
 // Sixteen warps: a link is a chain of short steps (shared loads, splits, a few
 // MMAs, a barrier), and twice the warps halve each warp's share of all but the
-// barrier (elasticity 38^3, half width about 500, 24 columns: the 56 sweeps of
+// barrier (elasticity 38x31x24, half width about 500, 24 columns: the 56 sweeps of
 // the eigensolver 81 ms with eight warps, 54 ms with sixteen).
 template <int B>
 __host__ __device__ constexpr int mma_warps() {
@@ -1554,8 +1562,9 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
   SweepArgs a{d_desc, xbase, xoff, count, max_w, max_n, 0, nrhs, nrhs_dev, skip_dev, st, s, slots};
   const int sms = sm_count();
   // C thread blocks per matrix: the waves of blocks times the length of one
-  // matrix's sweep, relative to C = 1 as measured at half widths 307-463 (FP32
-  // one column 1, 0.57, 0.35, 0.36; MMA 1, 0.54, 0.44; FP64 1, 0.54, 0.45); a
+  // matrix's sweep, relative to C = 1 (rel: between what the kernels measured at
+  // half widths 307-463: FP32 one column 1, 0.57, 0.35, 0.36; MMA 1, 0.54, 0.44;
+  // FP64 1, 0.54, 0.45); a
   // block is solved from the ceil(w / blk) before it, which bounds what C can
   // share, and each thread block has at least two
   auto clusters = [&](int units, double* len = nullptr) {
