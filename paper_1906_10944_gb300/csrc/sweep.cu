@@ -1411,7 +1411,7 @@ k_band_blkinv(T* __restrict__ base, const BandDesc* __restrict__ descs) {
 // ---------------------------------------------------------------------------
 // Launches.
 // ---------------------------------------------------------------------------
-constexpr size_t kSmemMax = 227 * 1024;
+constexpr size_t kSmemMax = 227 * 1024, kSmemPair = 113 * 1024;   // one and two blocks per SM
 
 template <typename T, typename A, int NC, int B>
 size_t sweep_smem(int w, int C, int nslot) {
@@ -1454,6 +1454,7 @@ struct SweepArgs {
   const int32_t *nrhs_dev, *skip;
   DevStatus* st;
   cudaStream_t s;
+  int live;    // matrices of the whole solve set
   int slots;   // wanted row slots (2-4), 0 = as many as fit
 };
 
@@ -1488,6 +1489,10 @@ geneo_status_t run_sweep(const T* base, const SweepArgs& a, int C, int parts, in
     if (nslot > 0 || C == 1) break;
   }
   if (nslot == 0) return GENEO_ERR_ARG;
+  if (sizeof(T) == 8 && NC == 1 && B == 16 && C == 1 && a.live > sm_count())   // two blocks per SM (sweep_block)
+    while (nslot > HB && sweep_smem<T, A, NC, B>(a.w, C, nslot) > kSmemPair &&
+           sweep_smem<T, A, NC, B>(a.w, C, HB) <= kSmemPair)
+      --nslot;
   return launch_cluster(k_sweep<T, A, NC, B, KC>, 32 * sweep_warps<NC, B>() + 32, dim3(a.count * C, parts), C, sweep_smem<T, A, NC, B>(a.w, C, nslot),
                         a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev, a.skip, cpp, C, nslot,
                         ring_blocks(a.w, B, C), a.st);
@@ -1520,10 +1525,16 @@ geneo_status_t run_mma(const float* base, const SweepArgs& a, int C, int parts, 
 // 466 us with 32 rows and a second block streaming in, 283 us with 64 and none;
 // the other blocks of the cluster work while the rows arrive).  0: too wide,
 // the factor stays as it is for the streamed kernels of band.cu.
-int sweep_block(int w, bool f64) {
+// FP64 bands too wide for 32 rows and the next 32 streaming in, more of them
+// than SMs (one-column local solves): 16 rows, so that two thread blocks share an
+// SM and one computes while the other's rows arrive.
+int sweep_block(int w, bool f64, int64_t count) {
   if (f64) {
-    if (w >= 31 && sweep_smem<double, double, 8, 32>(w, 1, 2) <= kSmemMax) return 32;
-    if (sweep_smem<double, double, 8, 16>(w, 1, 1) <= kSmemMax) return 16;
+    if (count > sm_count() && sweep_smem<double, double, 1, 32>(w, 1, 4) > kSmemMax &&
+        sweep_smem<double, double, 1, 16>(w, 1, 1) <= kSmemPair && sweep_smem<double, double, 4, 16>(w, 1, 1) <= kSmemMax)
+      return 16;
+    if (w >= 31 && sweep_smem<double, double, 4, 32>(w, 1, 2) <= kSmemMax) return 32;
+    if (sweep_smem<double, double, 4, 16>(w, 1, 1) <= kSmemMax) return 16;
     if (sweep_smem<double, double, 4, 8>(w, 1, 1) <= kSmemMax) return 8;
     return 0;
   }
@@ -1559,7 +1570,7 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
                            double* xbase, const int64_t* xoff, int nrhs, const int32_t* nrhs_dev,
                            const int32_t* skip_dev, DevStatus* st, cudaStream_t s, int tc_passes, int slots,
                            int live) {
-  SweepArgs a{d_desc, xbase, xoff, count, max_w, max_n, 0, nrhs, nrhs_dev, skip_dev, st, s, slots};
+  SweepArgs a{d_desc, xbase, xoff, count, max_w, max_n, 0, nrhs, nrhs_dev, skip_dev, st, s, live, slots};
   const int sms = sm_count();
   // C thread blocks per matrix: the waves of blocks times the length of one
   // matrix's sweep, relative to C = 1 (rel: between what the kernels measured at
@@ -1637,7 +1648,9 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
     // is the waves times the columns formed times the sweep's relative length
     // (27 FP64 bands of order 9261, half width 463, 11 columns: 12.2 ms in three
     // parts of 4, 11.3 in two of 6 on clusters of 2)
-    const bool fit8 = blk != 8 || sweep_smem<double, A, 8, 8>(max_w, 1, 1) <= kSmemMax;
+    const bool fit8 = (blk == 32   ? sweep_smem<double, A, 8, 32>(max_w, 1, 2)
+                       : blk == 16 ? sweep_smem<double, A, 8, 16>(max_w, 1, 1)
+                                   : sweep_smem<double, A, 8, 8>(max_w, 1, 1)) <= kSmemMax;
     const int most = fit8 ? 8 : 4;
     int parts = (nrhs + most - 1) / most, C = 1;
     double least = 1e300;
