@@ -410,6 +410,7 @@ struct SolveClass {
   BandDesc* d = nullptr;       // the class's descriptors (device), largest sweep first
   int count = 0, blk = 0, max_w = 0, max_n = 0;
   double cost = 0.0;           // bytes of one forward and backward sweep over the class
+  double longest = 0.0;        // and over its largest matrix
   int lane = 0;
 };
 struct SolveSet {

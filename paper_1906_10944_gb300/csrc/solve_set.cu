@@ -13,6 +13,7 @@
 // loaded stream.  Inside a class the subdomains are ordered by cost, largest
 // first, so that the longest sweeps start first.
 #include <algorithm>
+#include <cmath>
 #include <numeric>
 #include <vector>
 
@@ -67,6 +68,7 @@ geneo_status_t add_part(const void* base, bool f64, bool ds, const BandDesc* d_d
       c.max_w = std::max(c.max_w, b.w);
       c.max_n = std::max(c.max_n, b.n);
       c.cost += sweep_bytes(b, esz);
+      c.longest = std::max(c.longest, sweep_bytes(b, esz));
     }
     GENEO_TRY(mem.get(&c.d, g.size()));
     GENEO_CUDA(cudaMemcpyAsync(c.d, g.data(), sizeof(BandDesc) * g.size(), cudaMemcpyHostToDevice, s));
@@ -124,13 +126,24 @@ geneo_status_t solve_set_run(const SolveSet& ss, const SolveStreams& pool, doubl
     GENEO_CUDA(cudaEventRecord(pool.fork, s));
     for (int l = 1; l < ss.lanes; ++l) GENEO_CUDA(cudaStreamWaitEvent(pool.s[l - 1], pool.fork, 0));
   }
-  // the classes run side by side: each sizes its clusters for all of them
-  int live = 0;
-  for (const SolveClass& c : ss.cls) live += c.count;
-  if (active > 0) live = std::min(live, active);
+  // the classes run side by side: each sizes its clusters for all of them, as so
+  // many matrices of its own largest length (counted one by one, the small boxes
+  // of an uneven batch left the large ones a thread block each)
+  int all = 0;
+  double total = 0.0;
+  for (const SolveClass& c : ss.cls) {
+    all += c.count;
+    total += c.cost;
+  }
+  if (active > 0 && active < all) {
+    total *= (double)active / all;
+    all = active;
+  }
   geneo_status_t rc = GENEO_OK;
   for (const SolveClass& c : ss.cls) {
     const cudaStream_t cs = c.lane == 0 ? s : pool.s[c.lane - 1];
+    const int live = std::max(std::min(c.count, all),
+                              (int)std::min((double)all, std::ceil(total / std::max(c.longest, 1.0))));
     rc = run_class(c, xbase, xoff, nrhs, nrhs_dev, skip_dev, st, cs, tc_passes, slots, live);
     if (rc != GENEO_OK) break;
   }
