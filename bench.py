@@ -359,10 +359,10 @@ def ds_peak():
 # + dram__bytes_write.sum) on the 64^3 case, whose 64 subdomains have the same
 # size as the 128^3 ones; it is scaled to a launch of the timed workload by the
 # ratio of traffic to algorithmic bytes (both grow with the band entries
-# read).  Command and figures: profiles/k_band_solve_res_darcy3d_64.md.
+# read).  Command and figures: profiles/k_sweep_darcy3d_64.md.
 MEASURED_TRAFFIC = {
-    ("local_solve", "mixed"): {"kernel": "k_band_solve_res<float, 3>", "capture": "darcy3d_64",
-                               "dram_bytes_per_launch": 1.0333e9, "algorithmic_bytes_per_launch": 1.008916e9},
+    ("local_solve", "mixed"): {"kernel": "k_sweep<float, float, 1, 64, 1>", "capture": "darcy3d_64",
+                               "dram_bytes_per_launch": 0.9963e9, "algorithmic_bytes_per_launch": 1.008916e9},
 }
 
 
