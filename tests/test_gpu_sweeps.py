@@ -24,7 +24,9 @@ from gpu_helpers import run_gpu
 pytestmark = pytest.mark.gpu
 
 # (elements, parts, overlap): local half bandwidths about 5, 12, 16, 33, 64, 68, 90
-# and 190, orders with every kind of remainder, 1 to 144 subdomains
+# and 190, orders with every kind of remainder, 2 to 144 subdomains; the last two,
+# flat boxes of half bandwidth about 930 and 1840, take the 16- and 8-row blocks of
+# FP64 and the 32- and 16-row blocks of FP32
 GEOMETRIES = [
     ((12, 10), (4, 3), 1),
     ((96, 90), (12, 12), 1),
@@ -34,6 +36,8 @@ GEOMETRIES = [
     ((134, 66), (2, 1), 1),
     ((18, 16, 15), (2, 2, 2), 1),
     ((26, 23, 22), (2, 2, 2), 2),
+    ((60, 30, 6), (2, 1, 1), 1),
+    ((90, 40, 5), (2, 1, 1), 1),
 ]
 
 
