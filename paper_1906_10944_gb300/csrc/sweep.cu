@@ -45,6 +45,7 @@
 #include "common.cuh"
 #include "ds.cuh"
 #include "ptx.cuh"
+#include "sweep_index.h"
 
 namespace geneo {
 namespace {
@@ -144,21 +145,6 @@ __device__ __forceinline__ void split_tf32(float x, uint32_t& hi, uint32_t& lo) 
   lo = __float_as_uint(l);
 }
 
-// row blocks before a block that its owner reads: those the band reaches, and
-// all that the other blocks of the cluster solve between two of its own (so
-// that every value sent is waited for)
-__host__ __device__ __forceinline__ int reach_blocks(int w, int B, int C) {
-  const int r = (w + B - 1) / B;
-  return r > C - 1 ? r : C - 1;
-}
-// blocks of B rows in the ring of solved rows (and of partial sums): the
-// reach, and the slots of block k itself and of the C - 1 blocks that may
-// arrive before the owner of k reads on (rounded up to 32 rows, the columns
-// the multiply-add sweep takes at a time)
-__host__ __device__ __forceinline__ int ring_blocks(int w, int B, int C) {
-  const int r = reach_blocks(w, B, C) + C, m = B < 32 ? 32 / B : 1;
-  return m > 1 ? (r + 2 * m - 1) / m * m : r;
-}
 __device__ __forceinline__ float shfl_xor(float v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ double shfl_xor(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
 __device__ __forceinline__ dsv shfl_xor(dsv v, int o) {
@@ -246,9 +232,9 @@ struct RowStream {
 // Shared memory ahead of the slots.
 struct Bars {
   uint64_t full[kMaxSlots], empty[kMaxSlots];
-  uint64_t pad[48];   // loads of the entries left of the first row's band (not used) stay inside
+  uint64_t pad[48];   // and the entries left of the first slot's first band row (kSlotLead)
 };
-static_assert(sizeof(Bars) == 512, "slot alignment");
+static_assert(sizeof(Bars) == kSlotLead && kSlotLead % 128 == 0, "slot alignment");
 
 // barrier of the compute warps
 template <int N = kThreads>
@@ -1042,7 +1028,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
     const int ra = 16 * mt + g, rb8 = ra + 8;     // this lane's rows of the block
     const int half = 16 * mt / SR;
     // shared address of L(kb + ra, kl) in the band (row ra + 8: row8 on)
-    const uint32_t la = rs.slot_at(half) + (uint32_t)(((ra - half * SR) * ld + w - kb - ra + kl) * 4);
+    const uint32_t la = rs.slot_at(half) + (uint32_t)(slot_offset(kk, ra, kl, w, ld, B, SR) * 4);
     const bool va = ra < b, vb = rb8 < b;
     if (C > 1)  // the slots of the blocks that arrive before this one reads on
       for (int i = tid; i < (C - 1) * B * NC; i += kThreads) {
@@ -1050,7 +1036,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
         unset(win + (size_t)(i / ((C - 1) * B)) * YS + (q >= rwb ? q - rwb : q) * B + i % B);
       }
     clear();
-    const int jlo = max(0, min((kb - w + B) / B - 1, kk - C + 1));
+    const int jlo = forward_first(kk, w, B, C);
     int rb = rbk - (kk - jlo);
     if (rb < 0) rb += rwb;
     for (int j = jlo; j < kk; ++j) {
@@ -1064,7 +1050,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
         }
         ready = j + 1;
       }
-      if (G == 1 || (j - jlo) % G == gkp) {
+      if ((G == 1 || (j - jlo) % G == gkp) && block_in_band(kk, j, w, B)) {
         const bool fullb = b == B && j * B >= kb + B - 1 - w;
         const uint32_t lj = la + (uint32_t)(j * B * 4), wj = win_at + (uint32_t)((g * YS + rb * B + kl) * 4);
         const int ca = kb + ra - w - j * B - kl, cb = ca + 8;   // first columns in band, from kl
