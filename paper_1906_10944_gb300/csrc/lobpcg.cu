@@ -22,11 +22,12 @@
 // orthogonalisation pass runs in FP32 and the second, the block products,
 // the Gram matrices and the Rayleigh-Ritz sweeps in double-single arithmetic
 // (about 46 bits; the products and Gram matrices of the subdomains whose K_j
-// needed FP64 stay FP64); with FP64 factors all of it is FP64.  The K^{-1} solves use the factor's
+// needed FP64 stay FP64); with FP64 factors all of it is FP64 (Jacobi angles start
+// in FP32 and are refined to FP64 rounding).  The K^{-1} solves use the factor's
 // precision.
 //
 // Dense small problems (at most kMaxW = 104 columns) are solved by parallel
-// cyclic Jacobi in shared memory, one thread block per subdomain.
+// cyclic Jacobi in shared memory, one to four thread blocks per subdomain.
 #include <algorithm>
 #include <chrono>
 #include <type_traits>
@@ -34,6 +35,7 @@
 
 #include "ds.cuh"
 #include "handle.cuh"
+#include "jacobi_rotation.h"
 
 namespace geneo {
 namespace {
@@ -852,35 +854,24 @@ __device__ __forceinline__ bool jacobi_rot(T app, T aqq, T apq, T& c, T& s) {
   s = t * c;
   return s != T(0);
 }
-// FP64: the divisions and square roots of the formula above are dependent
-// chains on a pipe of 1/64 of the FP32 rate, a third of k_rr<double> (2.25 ms
-// a launch at 27 subdomains, m = 39).  The tangent is formed in FP32 and
-// improved by one Newton step on a_pq t^2 + (a_qq - a_pp) t - a_pq = 0 whose
-// residual is FP64 (error of the order of the FP32 error squared); c = (1 +
-// t^2)^(-1/2) is FP64, so c^2 + s^2 = 1 holds to FP64 rounding.
+// FP64: starting values in FP32, refined to FP64 rounding (jacobi_rotation.h),
+// without branches but for pivots out of FP32's range.
 template <>
 __device__ __forceinline__ bool jacobi_rot<double>(double app, double aqq, double apq, double& c, double& s) {
   using J = JacobiOps<double>;
-  const double a = fabs(apq);
-  if (!(a > J::tiny && a * a > J::eps_rot * J::eps_rot * fabs(app * aqq))) return false;
-  const double dd = aqq - app;
-  const float af = (float)apq, df = (float)dd;
+  const double a = fabs(apq), dd = aqq - app;
+  const bool big = a > J::tiny && a * a > J::eps_rot * J::eps_rot * fabs(app * aqq);
+  const float af = jacobi_f32_inf(apq), df = jacobi_f32_inf(dd);
+  const float theta = __fdividef(df, 2.f * af), ta = fabsf(theta), q = fmaf(theta, theta, 1.f);
+  const float t0 = __fdividef(theta >= 0.f ? 1.f : -1.f, ta < 1e9f ? ta + q * rsqrtf(q) : 2.f * ta);
   double t;
-  if (fabsf(af) > 1e-30f && fabsf(af) < 1e30f && fabsf(df) < 1e30f) {
-    const float theta = df / (2.f * af);
-    float t0 = copysignf(1.f, theta) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f)));
-    if (fabsf(theta) > 1e15f) t0 = 0.5f / theta;
-    const double td = (double)t0;
-    const double f = fma(fma(apq, td, dd), td, -apq);
-    const float fp = fmaf(2.f * af, t0, df);
-    t = fp != 0.f ? td - (double)((float)f / fp) : td;
-  } else {
-    const double theta = dd / (2.0 * apq);
-    t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
+  jacobi_refine(dd, apq, t0, rsqrtf(fmaf(t0, t0, 1.f)), __fdividef(1.f, fmaf(2.f * af, t0, df)), t, c);
+  if (big && !jacobi_in_range(theta, af)) {
+    t = jacobi_tangent_formula(dd, apq);
+    c = rsqrt(fma(t, t, 1.0));
   }
-  c = rsqrt(fma(t, t, 1.0));
   s = t * c;
-  return s != 0.0;
+  return big && s != 0.0;
 }
 // Double-single: the angle in FP32 from the double-single difference of the
 // pivots.  An angle good to FP32 leaves a_pq about 1e-7 of its size instead of
