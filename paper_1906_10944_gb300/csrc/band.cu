@@ -25,6 +25,7 @@
 // The factor is read once per sweep; b and x once each.
 #include "common.cuh"
 #include "ds.cuh"
+#include "pivot.h"
 #include "ptx.cuh"
 
 namespace geneo {
@@ -256,8 +257,8 @@ k_band_panel_diag(T* __restrict__ base, const BandDesc* __restrict__ descs, int 
         // one reciprocal square root instead of a square root and a division:
         // both are long dependent chains on the FP64 pipe (66 -> 41 us
         // a panel of 27 bands of half width 463, 46 -> 20 us of narrower ones)
-        const T r = rsqrt(p);
-        a[t >> 2] = lane == t ? p * r : lane > t ? a[t >> 2] * r : T(0);
+        const T r = rsqrt(p), d = pivot_root(p, r);
+        a[t >> 2] = lane == t ? d : lane > t ? pivot_quotient(a[t >> 2], d, r) : T(0);
         col[t & 1][lane] = a[t >> 2];
       }
       __syncthreads();
