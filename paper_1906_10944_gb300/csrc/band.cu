@@ -960,16 +960,6 @@ k_band_solve(const T* __restrict__ base, const BandDesc* __restrict__ descs,
       mbar_wait_bounded(&bars[v % kStages], (uint32_t)((v / kStages) & 1), st, d.id, v);
 }
 
-inline int sm_count() {
-  static int sms[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
-  if (!sms[dev] && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 152;
-  }
-  return sms[dev];
-}
 constexpr int kNB = 32;
 constexpr size_t kSmemCap = 200 * 1024;
 

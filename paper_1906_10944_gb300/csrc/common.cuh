@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -297,6 +298,21 @@ inline cudaError_t allow_smem(K kern) {
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&v, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
   return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, v - (int)a.sharedSizeBytes);
+}
+
+// SMs of the current device (any thread), looked up once per device; 152, a GB300's,
+// where that fails.
+inline int sm_count() {
+  static std::atomic<int> sms[64];
+  int dev = 0, v = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
+  if ((v = sms[dev].load(std::memory_order_relaxed)) > 0) return v;
+  if (cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || v <= 0) {
+    cudaGetLastError();
+    return 152;
+  }
+  sms[dev].store(v, std::memory_order_relaxed);
+  return v;
 }
 
 // --------------------------------------------------------------------------

@@ -1459,10 +1459,11 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
   // splits used 72 of 152 SMs: 812 us per FP64 Gram matrix, 328 us in 16; 64
   // subdomains in 5 splits are 320 blocks, a second wave for the last 16 of
   // them: 200 us per double-single Gram matrix, 164 us in 14)
+  const int sms = sm_count();
   int nrs = kMinRS;
   double nrs_cost = 1e300;
   for (int r = kMinRS; r <= kMaxRS; ++r) {
-    const double cost = (double)ceil_div(N * r, 2 * 152) / r + 0.002 * r;
+    const double cost = (double)ceil_div(N * r, 2 * sms) / r + 0.002 * r;
     if (cost < nrs_cost) {
       nrs_cost = cost;
       nrs = r;
@@ -1537,10 +1538,10 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
 
   // threads of the Jacobi kernels: one block per SM at most, so more warps hide
   // its latencies; with several blocks per SM, 256
-  const int td = N <= 152 ? kTD : kT;
+  const int td = N <= sms ? kTD : kT;
   // blocks per matrix: as many as idle SMs allow, up to four (beyond that the
   // rotation of A is all that is left)
-  const dim3 gj(N, std::max(1, std::min(4, 152 / std::max(N, 1))));
+  const dim3 gj(N, std::max(1, std::min(4, sms / std::max(N, 1))));
   const bool f32 = h->fp32;
   // Rayleigh-Ritz sweeps in double-single arithmetic in the FP32 mode
   auto rr_launch = [&](const double* Gm, double* Tt, int ld, const int32_t* s_, const int32_t* q_,

@@ -682,7 +682,7 @@ geneo_status_t alloc_solver(geneo_handle_s* h) {
 
 static geneo_status_t apply_dot(geneo_handle_s* h, const double* r, double* z, cudaStream_t s, const Dot& dot) {
   const int N = h->N;
-  if (N < 304) {   // fewer than two blocks per SM
+  if (N < 2 * sm_count()) {   // fewer than two blocks per SM
     const int gy = std::max(1, std::min(ceil_div(h->maxnD, kT), 4));
     k_restrict_wide<<<dim3(N, gy + ceil_div(h->maxm, kRq)), kT, 0, s>>>(h->dsub, h->Dlist, r, h->Z, h->u, h->cH, gy);
   } else {

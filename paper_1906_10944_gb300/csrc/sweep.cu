@@ -1469,17 +1469,6 @@ struct SweepArgs {
   int slots;   // wanted row slots (2-4), 0 = as many as fit
 };
 
-inline int sm_count() {
-  static int sms[64] = {0};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
-  if (!sms[dev] && cudaDeviceGetAttribute(&sms[dev], cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
-    cudaGetLastError();
-    return 152;
-  }
-  return sms[dev];
-}
-
 // slots that fit beside the rest, capped at `want` (0 = kMaxSlots); 0 = none
 template <typename F>
 int fit_slots(F bytes, int need, int want) {
