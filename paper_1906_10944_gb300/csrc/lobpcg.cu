@@ -1454,16 +1454,17 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
   if (W3 > kMaxW) return GENEO_ERR_ARG;
   const int64_t rows = h->sumN;
   double *S, *KS, *BS, *P, *Tmp, *G, *Gp, *Tm, *nu, *rn;
-  // row splits of the Gram matrices: the fewest waves of two blocks per SM per
-  // split, and few splits to sum (18 subdomains of 38x31x24 elasticity in four
-  // splits used 72 of 152 SMs: 812 us per FP64 Gram matrix, 328 us in 16; 64
-  // subdomains in 5 splits are 320 blocks, a second wave for the last 16 of
-  // them: 200 us per double-single Gram matrix, 164 us in 14)
+  // row splits r of the Gram matrices: waves of two blocks per SM, each block as
+  // long as its 1/r of a subdomain's rows and what it costs whatever its rows
+  // (0.004 of a subdomain: partial sums written and read again, prologue).  Gram
+  // family of a setup at 512 subdomains (128^3) 58.1 ms in 4 splits, 56.9 in 7, 59.7
+  // in 13, which the waves alone would take; at 64 (64^3) 12.2 in 4, 10.3 in 9, 10.0
+  // in 14; at 18 (elasticity 38x31x24) 74.5 in 4, 33.8 in 14 and 16.
   const int sms = sm_count();
   int nrs = kMinRS;
   double nrs_cost = 1e300;
   for (int r = kMinRS; r <= kMaxRS; ++r) {
-    const double cost = (double)ceil_div(N * r, 2 * sms) / r + 0.002 * r;
+    const double cost = (double)ceil_div(N * r, 2 * sms) * (1.0 / r + 0.004);
     if (cost < nrs_cost) {
       nrs_cost = cost;
       nrs = r;
