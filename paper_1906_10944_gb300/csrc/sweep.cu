@@ -90,20 +90,16 @@ __device__ __forceinline__ void st_cluster(uint32_t dst, dsv v) {
   const uint64_t b = ((uint64_t)__float_as_uint(v.l) << 32) | __float_as_uint(v.h);
   asm volatile("st.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(dst), "l"(b) : "memory");
 }
-__device__ __forceinline__ void unset(float* p) {
-  asm volatile("st.relaxed.cluster.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(p)), "r"(kUnset32) : "memory");
-}
-__device__ __forceinline__ void unset64(void* p) {
-  asm volatile("st.relaxed.cluster.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(p)), "l"(kUnset64) : "memory");
-}
-__device__ __forceinline__ void unset(double* p) { unset64(p); }
-__device__ __forceinline__ void unset(dsv* p) { unset64(p); }
+__device__ __forceinline__ void unset(float* p) { *reinterpret_cast<uint32_t*>(p) = kUnset32; }
+__device__ __forceinline__ void unset(double* p) { *reinterpret_cast<uint64_t*>(p) = kUnset64; }
+__device__ __forceinline__ void unset(dsv* p) { *reinterpret_cast<uint64_t*>(p) = kUnset64; }
 // A slot is cleared by its owner and filled again by another block: what orders
-// the two is a message from the owner (release, after the block barrier that
-// follows the clears) that the other block has polled (acquire, before the block
-// barrier that precedes its stores).  Both fences cover shared memory only; a
-// solve of eight columns at 64^3 takes 46.3 ms with them and 45.3 ms without, one
-// column at 32^3 7.0 ms either way.
+// the two is a message from the owner (release, after a block barrier that follows
+// the clears) that the other block has polled (acquire, after the polls and before
+// the block barrier that precedes its stores).  Both fences cover shared memory
+// only.  With and without them: eight columns, 64 bands of order 6859, half width
+// 381, 491 and 486 us a sweep; 12 columns 574 and 560; one column, 64 bands of 5832,
+// 340, 231 and 230.
 __device__ __forceinline__ void release_cluster() {
   asm volatile("fence.release.sync_restrict::shared::cta.cluster;" ::: "memory");
 }
@@ -143,10 +139,7 @@ __device__ __forceinline__ bool wait_set(A* v, At at, In in, DevStatus* st, int 
         all &= !is_unset(v[i]);
       }
     }
-    if (all) {
-      acquire_cluster();
-      return true;
-    }
+    if (all) return true;
   }
   record_error(st, GENEO_ERR_TIMEOUT, id, where);
   return false;
@@ -253,7 +246,7 @@ struct RowStream {
 // Shared memory ahead of the slots.
 struct Bars {
   uint64_t full[kMaxSlots], empty[kMaxSlots];
-  uint64_t pad[48];   // and the entries left of the first slot's first band row (kSlotLead)
+  uint64_t pad[48];
 };
 static_assert(sizeof(Bars) == kSlotLead && kSlotLead % 128 == 0, "slot alignment");
 
@@ -632,6 +625,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
       const A t = reduce(acc);
       if (mine) zb[row * NC + col] = in ? rhs - t : A();
     }
+    if (C > 1) acquire_cluster();
     csync<kThreads>();
     if (C > 1) release_cluster();
     // y = M z, M the inverted diagonal block (its lower triangle)
@@ -734,6 +728,7 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
       }
       zb[row * NC + col] = row < b ? z : A();
     }
+    if (C > 1) acquire_cluster();
     csync<kThreads>();
     if (C > 1) release_cluster();
     const uint32_t sa0 = smem_u32(S0), sa1 = smem_u32(S1) + (uint32_t)(32 * (ld - 1) * (int)sizeof(T));
@@ -914,7 +909,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
 
   extern __shared__ __align__(128) unsigned char smem_raw[];
   Bars* bars = reinterpret_cast<Bars*>(smem_raw);
-  float* slots = reinterpret_cast<float*>(smem_raw + sizeof(Bars));
+  float* slots = reinterpret_cast<float*>(smem_raw + slot_lead(C));
   float* win = slots + (size_t)nslot * SR * ld;        // NC columns of YS: solved rows, then partial sums
   float* red = win + (size_t)NC * YS;                  // KP x NC x RB
   float* zb = red + (size_t)KP * NC * RB;              // NC x ZS
@@ -1069,11 +1064,12 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
           if (ok)
             ok = wait_set<E>(v, [&](int e) { return win + (size_t)(ph + e * P) * YS + rb * B + row; },
                              [&](int e) { return ph + e * P < k; }, st, d.id, j);
+          acquire_cluster();
           csync<kThreads>();
         }
         ready = j + 1;
       }
-      if ((G == 1 || (j - jlo) % G == gkp) && block_in_band(kk, j, w, B)) {
+      if (G == 1 || (j - jlo) % G == gkp) {
         const bool fullb = b == B && j * B >= kb + B - 1 - w;
         const uint32_t lj = la + (uint32_t)(j * B * 4), wj = win_at + (uint32_t)((g * YS + rb * B + kl) * 4);
         const int ca = kb + ra - w - j * B - kl, cb = ca + 8;   // first columns in band, from kl
@@ -1194,6 +1190,7 @@ k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, 
         zb[c * ZS + row] = row < b ? d2f_bits(xc[e]) - s : 0.f;
       }
     }
+    if (C > 1) acquire_cluster();
     csync<kThreads>();
     if (C > 1) release_cluster();
     // x = M^T z: A(m = column, k = row t) = M(t, m)
@@ -1433,7 +1430,7 @@ size_t sweep_smem(int w, int C, int nslot) {
 template <int B, int NT>
 size_t mma_smem(int w, int C, int nslot) {
   const size_t SR = B < 32 ? B : 32, NC = 8 * NT, KP = mma_warps<B>() / (B / 16);
-  return sizeof(Bars) + sizeof(float) * (nslot * SR * band_ld(w) + NC * ((size_t)ring_blocks(w, B, C) * B + 1) +
+  return slot_lead(C) + sizeof(float) * (nslot * SR * band_ld(w) + NC * ((size_t)ring_blocks(w, B, C) * B + 1) +
                                          KP * NC * (B + 4) + NC * (B + 1) + (C > 1 ? (size_t)C * NC * B : 0));
 }
 

@@ -27,16 +27,15 @@ int main() {
         for (int kk = 0; kk < nb; ++kk) {
           const int first = forward_first(kk, w, B, C);
           for (int j = first; j < kk; ++j) {
-            if (!block_in_band(kk, j, w, B)) continue;
             for (int r = 0; r < B; r += SR) {
-              const long at = kSlotLead + 4L * slot_offset(kk, r, j * B, w, ld, B, SR);
+              const long at = slot_lead(C) + 4L * slot_offset(kk, r, j * B, w, ld, B, SR);
               if (at < lowest) lowest = at;
               if (at < 0) ++bad;
             }
           }
           for (int j = 0; j < kk; ++j) {
             const bool holds = j * B + B - 1 >= kk * B - w;   // a column in the first row's band
-            if (holds && (j < first || !block_in_band(kk, j, w, B))) ++missed;
+            if (holds && j < first) ++missed;
           }
           // every block that arrives between two blocks of an owner is waited for
           if (kk >= C - 1 && first > kk - C + 1) ++missed;
