@@ -40,6 +40,7 @@
 // All sums run in a fixed order.  Every wait is bounded; a wait that gives up
 // records GENEO_ERR_TIMEOUT and the block goes on without waiting.
 #include <algorithm>
+#include <atomic>
 #include <type_traits>
 
 #include "common.cuh"
@@ -1466,6 +1467,35 @@ struct SweepArgs {
   int slots;   // wanted row slots (2-4), 0 = as many as fit
 };
 
+// Clusters of C = 1 << i thread blocks, one block per SM, that the current device
+// runs at the same time (any thread), looked up once per device.  A cluster lies in
+// one GPC: of 152 SMs, 76 clusters of 2, 36 of 4 and 15 of 8.
+inline int cluster_count(int i) {
+  static std::atomic<int> fit[64][4];
+  const int C = 1 << i;
+  int dev = 0, n = 0;
+  if (C == 1 || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return std::max(sm_count() / C, 1);
+  if ((n = fit[dev][i].load(std::memory_order_relaxed)) > 0) return n;
+  const auto kern = k_sweep<float, float, 1, 64, 1>;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(C);
+  cfg.blockDim = dim3(32 * sweep_warps<1, 64>() + 32);
+  cfg.dynamicSmemBytes = kSmemPair + 1024;   // more than half of an SM's
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)C;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (allow_smem(kern) != cudaSuccess || cudaOccupancyMaxActiveClusters(&n, kern, &cfg) != cudaSuccess || n <= 0) {
+    cudaGetLastError();
+    return std::max(sm_count() / C, 1);
+  }
+  fit[dev][i].store(n, std::memory_order_relaxed);
+  return n;
+}
+
 // slots that fit beside the rest, capped at `want` (0 = kMaxSlots); 0 = none
 template <typename F>
 int fit_slots(F bytes, int need, int want) {
@@ -1568,20 +1598,22 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
                            const int32_t* skip_dev, DevStatus* st, cudaStream_t s, int tc_passes, int slots,
                            int live) {
   SweepArgs a{d_desc, xbase, xoff, count, max_w, max_n, 0, nrhs, nrhs_dev, skip_dev, st, s, live, slots};
-  const int sms = sm_count();
   // C thread blocks per matrix: the waves of blocks times the length of one
   // matrix's sweep, relative to C = 1 (rel: between what the kernels measured at
   // half widths 307-463: FP32 one column 1, 0.57, 0.35, 0.36; MMA 1, 0.54, 0.44;
   // FP64 1, 0.54, 0.45); a
   // block is solved from the ceil(w / blk) before it, which bounds what C can
-  // share, and each thread block has at least two
+  // share, and each thread block has at least two.  (Waves of SMs / C clusters sent
+  // 16 to 19 matrices to C = 8 in what are two waves: one column of 18 FP32 bands of
+  // order 9000, half width 672, 402 us, and 312 on C = 4; FP64, 6859 and 381, 2245
+  // and 1119.)
   auto clusters = [&](int units, double* len = nullptr) {
     const double rel[4] = {1.0, 0.56, 0.40, 0.38};
     int best = 1;
     double least = 1e300;
     for (int i = 0, C = 1; C <= kMaxC; ++i, C *= 2) {
       if (C > 1 && (C * blk > max_w + blk - 1 || (max_n > 0 && max_n < 2 * C * blk))) break;
-      const int64_t per_wave = std::max(sms / C, 1), waves = ((int64_t)live * units + per_wave - 1) / per_wave;
+      const int64_t per_wave = cluster_count(i), waves = ((int64_t)live * units + per_wave - 1) / per_wave;
       if (waves * rel[i] < least - 1e-9) {
         least = waves * rel[i];
         best = C;
