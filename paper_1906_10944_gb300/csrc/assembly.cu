@@ -461,12 +461,11 @@ geneo_status_t refactor_fp64(geneo_handle_s* h, const AssemblyOut& a, const int3
   std::vector<BandDesc> rd;
   int64_t tot = 0;
   int blk_mask = 0;
-  const int64_t solved = isK ? 0 : std::count_if(flag.begin(), flag.end(), [](int32_t f) { return f != 0; });
   for (int j = 0; j < N; ++j) {
     if (!flag[j]) continue;
     const SubDesc& d = h->hsub[j];
     const int n = isK ? d.nN : d.nD, w = band_w(isK ? d.wK : d.wA);
-    rd.push_back(BandDesc{tot, n, w, j, band_ld(w), sweep_block(w, true, solved), -1});
+    rd.push_back(BandDesc{tot, n, w, j, band_ld(w), sweep_block(w, true), -1});
     blk_mask |= rd.back().blk;
     tot += (int64_t)n * band_ld(w);
     r->maxw = std::max(r->maxw, w);
@@ -759,7 +758,7 @@ geneo_status_t assemble_local(geneo_handle_s* h, const geneo_problem_t* p, Assem
     const SubDesc& d = h->hsub[j];
     const int wK = band_w(d.wK), wA = band_w(d.wA);
     bk[j] = BandDesc{d.bandK, d.nN, wK, j, band_ld(wK), sweep_block(wK, !h->fp32), equil ? dK : -1};
-    ba[j] = BandDesc{d.bandA, d.nD, wA, j, band_ld(wA), sweep_block(wA, !h->fp32, N), equil ? dA : -1};
+    ba[j] = BandDesc{d.bandA, d.nD, wA, j, band_ld(wA), sweep_block(wA, !h->fp32), equil ? dA : -1};
     dK += equil ? scl_elems(d.nN) : 0;
     dA += equil ? scl_elems(d.nD) : 0;
     maskK |= bk[j].blk;

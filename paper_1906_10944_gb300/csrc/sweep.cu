@@ -1420,7 +1420,7 @@ k_band_blkinv(T* __restrict__ base, const BandDesc* __restrict__ descs) {
 // ---------------------------------------------------------------------------
 // Launches.
 // ---------------------------------------------------------------------------
-constexpr size_t kSmemMax = 227 * 1024, kSmemPair = 113 * 1024;   // one and two blocks per SM
+constexpr size_t kSmemMax = 227 * 1024;
 
 template <typename T, typename A, int NC, int B>
 size_t sweep_smem(int w, int C, int nslot) {
@@ -1480,7 +1480,7 @@ inline int cluster_count(int i) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(C);
   cfg.blockDim = dim3(32 * sweep_warps<1, 64>() + 32);
-  cfg.dynamicSmemBytes = kSmemPair + 1024;   // more than half of an SM's
+  cfg.dynamicSmemBytes = 114 * 1024;   // more than half of an SM's
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = (unsigned)C;
@@ -1516,10 +1516,6 @@ geneo_status_t run_sweep(const T* base, const SweepArgs& a, int C, int parts, in
     if (nslot > 0 || C == 1) break;
   }
   if (nslot == 0) return GENEO_ERR_ARG;
-  if (sizeof(T) == 8 && NC == 1 && B == 16 && C == 1 && a.live > sm_count())   // two blocks per SM (sweep_block)
-    while (nslot > HB && sweep_smem<T, A, NC, B>(a.w, C, nslot) > kSmemPair &&
-           sweep_smem<T, A, NC, B>(a.w, C, HB) <= kSmemPair)
-      --nslot;
   return launch_cluster(k_sweep<T, A, NC, B, KC>, 32 * sweep_warps<NC, B>() + 32, dim3(a.count * C, parts), C, sweep_smem<T, A, NC, B>(a.w, C, nslot),
                         a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev, a.skip, cpp, C, nslot,
                         ring_blocks(a.w, B, C), a.st);
@@ -1552,14 +1548,8 @@ geneo_status_t run_mma(const float* base, const SweepArgs& a, int C, int parts, 
 // 466 us with 32 rows and a second block streaming in, 283 us with 64 and none;
 // the other blocks of the cluster work while the rows arrive).  0: too wide,
 // the factor stays as it is for the streamed kernels of band.cu.
-// FP64 bands too wide for 32 rows and the next 32 streaming in, more of them
-// than SMs (one-column local solves): 16 rows, so that two thread blocks share an
-// SM and one computes while the other's rows arrive.
-int sweep_block(int w, bool f64, int64_t count) {
+int sweep_block(int w, bool f64) {
   if (f64) {
-    if (count > sm_count() && sweep_smem<double, double, 1, 32>(w, 1, 4) > kSmemMax &&
-        sweep_smem<double, double, 1, 16>(w, 1, 1) <= kSmemPair && sweep_smem<double, double, 4, 16>(w, 1, 1) <= kSmemMax)
-      return 16;
     if (w >= 31 && sweep_smem<double, double, 4, 32>(w, 1, 2) <= kSmemMax) return 32;
     if (sweep_smem<double, double, 4, 16>(w, 1, 1) <= kSmemMax) return 16;
     if (sweep_smem<double, double, 4, 8>(w, 1, 1) <= kSmemMax) return 8;
