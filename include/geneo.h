@@ -202,12 +202,13 @@ typedef struct {
  *             tensor-map copies) when the batch's half bandwidth fits that
  *             kernel; 1 always uses the warp-level MMA kernel.
  *  autotune   1 (default): at the end of the first setup of each batch
- *             shape (precision, largest A_j band width and order, number of
- *             subdomains) in the process, the preconditioner's local solve
- *             is timed at each pipeline depth (2 to 4 row slots) on a scratch vector and the
- *             fastest is kept for every later apply (reported in
- *             geneo_coarse_info_t.local_solve_stages); 0: the depth follows
- *             from shared memory alone.
+ *             shape (device, precision, largest A_j band width and order,
+ *             number of subdomains) in the process, the preconditioner's
+ *             local solve is timed at each pipeline depth (2 to 4 row slots)
+ *             on a scratch vector and the fastest is kept for every later
+ *             apply of that shape (reported in
+ *             geneo_coarse_info_t.local_solve_stages; it changes times, not
+ *             results); 0: the depth follows from shared memory alone.
  *  factor_bf16  GENEO_PREC_FP32 only, a precision study: 1 rounds the
  *             equilibrated matrices and every factor panel to BF16 (the
  *             fifth-generation kernel's planes hold BF16 values exactly),

@@ -528,20 +528,25 @@ double condition_estimate_fixed(const double* a, const double* b, int m, double*
 
 // Autotuner of the preconditioner's local solve (the one-right-hand-side band
 // sweep): each depth of its copy pipeline (2, 3 or 4 row slots; more slots take
-// more shared memory and may leave fewer blocks per SM) is timed on this batch, on a scratch copy of the subdomain
-// vectors, and the fastest is kept for the process, keyed by (precision,
-// largest band width, largest order, batch size).  The depths are timed in
+// more shared memory and may leave fewer blocks per SM) is timed on this batch, on
+// a scratch copy of the subdomain vectors, and the fastest is kept for the process,
+// keyed by (device, precision, largest band width, largest order, batch size).
+// Batches that share a key but not their size classes or FP64 factors share the
+// depth, which changes their time and not their result: classes in the key would
+// time every new coefficient field of a mesh again (15 sweeps).  The depths are timed in
 // turn, four rounds after a warm-up launch of each, one launch per CUDA-event
 // pair, and each depth keeps its fastest launch: a single short window per
 // depth is at the mercy of whatever else the GPU does at that moment.  Runs
 // once per key at the end of a setup.
 namespace {
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int, int>, int> g_tune;
+std::map<std::tuple<int, int, int, int, int>, int> g_tune;
 }  // namespace
 
 geneo_status_t tune_local_solve(geneo_handle_s* h) {
-  const auto key = std::make_tuple(h->fp32 ? 1 : 0, h->maxwA, h->maxnD, h->N);
+  int dev = 0;
+  GENEO_CUDA(cudaGetDevice(&dev));
+  const auto key = std::make_tuple(dev, h->fp32 ? 1 : 0, h->maxwA, h->maxnD, h->N);
   {
     std::lock_guard<std::mutex> lock(g_tune_mu);
     auto it = g_tune.find(key);
