@@ -360,6 +360,9 @@ geneo_status_t tc5_factor(const Tc5Plan& p, float* band, const BandDesc* d_desc,
 // Rows per block of the sweeps for a band of half width w >= 15 (stored as
 // FP64 or FP32); 0: too wide for them.
 int sweep_block(int w, bool f64);
+// Looks up what the sweeps' launches need from the current device, so that a solve
+// only launches (a setup calls it).
+void sweep_prepare();
 // the inverses of the diagonal blocks, in place, of every matrix whose blk is
 // in blk_mask (an OR of block sizes, which are powers of two)
 template <typename T>

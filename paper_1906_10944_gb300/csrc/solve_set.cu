@@ -97,6 +97,7 @@ geneo_status_t make_solve_set(const void* base, bool f64, const BandDesc* d_desc
                               cudaStream_t s, SolveSet* out, bool ds64) {
   out->cls.clear();
   out->lanes = 1;
+  sweep_prepare();
   GENEO_TRY(add_part(base, f64, false, d_desc, count, mem, s, out->cls));
   GENEO_TRY(add_part(base64, true, ds64, d_desc64, count64, mem, s, out->cls));
   // The class with the longest sweep first (its chain starts at once, the others

@@ -1562,6 +1562,10 @@ int sweep_block(int w, bool f64) {
   return 0;
 }
 
+void sweep_prepare() {
+  for (int i = 1; i < 4; ++i) cluster_count(i);
+}
+
 template <typename T>
 geneo_status_t band_blkinv(T* base, const BandDesc* d_desc, int count, int max_n, int blk_mask, cudaStream_t s) {
   using A = std::conditional_t<sizeof(T) == 4, dsv, double>;
