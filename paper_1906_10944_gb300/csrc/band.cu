@@ -1006,9 +1006,10 @@ geneo_status_t band_potrf(T* base, const BandDesc* d_desc, int count, int max_w,
     }
   }
   // FP64 bands too few for one SM each: every panel's work spread over the GPU.
-  // Both sides in units of 32^3 / 2 multiply-adds: one block per matrix runs the
-  // widest alone on its SM; spread, a panel's three launches cost about 75 us
-  // (measured: 20 to 41 + 24 to 28, and the gaps) whatever the batch
+  // Both sides in SM clocks per panel, of 2 multiply-adds: one block per matrix runs
+  // the widest alone on its SM; spread, a panel's three launches cost about 75 us
+  // (150e3 clocks at 2.0 GHz; measured: 20 to 41 + 24 to 28, and the gaps) whatever
+  // the batch
   if constexpr (sizeof(T) == 8) {
     if (!weak && max_n > 256 && max_w >= 96) {
       const double panel = 0.5 * (double)max_w * max_w * kPN;          // multiply-adds of one panel's update

@@ -1882,13 +1882,21 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
     GENEO_TRY(solveK(xoffX, sj, skip));
     spmm(true, false, Xr, KXr, KXr, skip);
     GENEO_TRY(gram(Xr, KXr, 1, skip));
-    { const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st); k_svqb<double><<<gj, td, dsm, st>>>(G, Tm, ldg, sj, nullptr, rj, 1e-14, skip, wcur); note_launch(); h->prof.end(prs, st); }
+    {
+      const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st);
+      k_svqb<double><<<gj, td, dsm, st>>>(G, Tm, ldg, sj, nullptr, rj, 1e-14, skip, wcur); note_launch();
+      h->prof.end(prs, st);
+    }
     GENEO_TRY(gemm(Xr, Tm, 0, nullptr, cref(Tmp, W3, 0, nullptr, 0, rj), 1.0, 0.0, skip));
     k_set_i32<<<ceil_div(N, 128), 128, 0, st>>>(sj, rj, N, skip); note_launch();
     k_copy_cols<double, double><<<gridR, kT, 0, st>>>(h->dsub, cref(Tmp, W3, 0, nullptr, 0, sj), Xr, skip); note_launch();
     spmm(false, true, Xr, BXr, BXr, skip);
     GENEO_TRY(gram(Xr, BXr, 1, skip));
-    { const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st); rr_launch(G, Tm, ldg, sj, nullptr, nu, s, skip, wcur); note_launch(); h->prof.end(prs, st); }
+    {
+      const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st);
+      rr_launch(G, Tm, ldg, sj, nullptr, nu, s, skip, wcur); note_launch();
+      h->prof.end(prs, st);
+    }
     GENEO_TRY(gemm(Xr, Tm, 0, nullptr, cref(Tmp, W3, 0, nullptr, 0, sj), 1.0, 0.0, skip));
     k_copy_cols<double, double><<<gridR, kT, 0, st>>>(h->dsub, cref(Tmp, W3, 0, nullptr, 0, sj), Xr, skip); note_launch();
     GENEO_CUDA(cudaGetLastError());
@@ -2005,7 +2013,11 @@ geneo_status_t local_eigensolve(geneo_handle_s* h, AssemblyOut& asmb, DevMem& tm
       // only BQ is new
       spmm(false, true, Qr, BQr, BQr, done);
       GENEO_TRY(gram(Sr, BSr, 1, done));
-      { const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st); rr_launch(G, Tm, ldg, sj, qj, nu, s, done, wcur); note_launch(); h->prof.end(prs, st); }
+      {
+        const int prs = h->prof.begin(GENEO_PROF_SMALL_EIG, 0.0, 0.0, st);
+        rr_launch(G, Tm, ldg, sj, qj, nu, s, done, wcur); note_launch();
+        h->prof.end(prs, st);
+      }
       // P = Q U[s_j:, :], X = S U
       // P only spans the next search block: FP32 arithmetic with FP32 factors
       if (f32) GENEO_TRY(gemm32(Qr, Tm, 0, sj, cref(P, s, 0, nullptr, 0, sj), 1.0, 0.0, done, 0, 0,

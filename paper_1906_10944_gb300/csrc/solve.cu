@@ -710,9 +710,9 @@ static geneo_status_t apply_dot(geneo_handle_s* h, const double* r, double* z, c
     {
       const int pc = h->prof.begin(GENEO_PROF_COARSE_SOLVE, band_solve_flops(h->dimH, h->wH),
                                    2.0 * 8.0 * band_entries(h->dimH, h->wH) + 16.0 * h->dimH, h->aux);
-      GENEO_TRY(band_solve<double>(h->bandH, h->dbandH, 1, sweep_block(band_w(h->wH), true), band_w(h->wH), h->cH, h->xoffH, 1,
-                                   nullptr, nullptr,
-                                   h->dstat, h->aux, h->dimH));
+      const int w = band_w(h->wH);   // as stored
+      GENEO_TRY(band_solve<double>(h->bandH, h->dbandH, 1, sweep_block(w, true), w, h->cH, h->xoffH, 1, nullptr,
+                                   nullptr, h->dstat, h->aux, h->dimH));
       h->prof.end(pc, h->aux);
     }
     GENEO_CUDA(cudaEventRecord(h->ev_join, h->aux));

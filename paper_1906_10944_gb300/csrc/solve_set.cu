@@ -1,17 +1,17 @@
 // Size classes of a batch of band factors for the solves.
 //
 // The local solves of the preconditioner (A_j^{-1}, Section 3) and the block
-// solves of the eigensolver (K_j^{-1}, Section 4.4) run one thread block per
-// subdomain, and band_solve picks one kernel and one shared-memory size for a
-// whole launch from the widest band and the longest vector of the batch.  In
-// a batch of very uneven subdomains one large box would then send every
-// subdomain to the streamed kernels and size every block for itself.  A
-// SolveSet cuts the batch (the FP32 part and the FP64 part separately) into
-// classes of similar half bandwidth, each launched with its own maxima, and
-// runs the classes concurrently: the largest on the caller's stream, the
-// others on the handle's solve streams, assigned longest-first to the least
-// loaded stream.  Inside a class the subdomains are ordered by cost, largest
-// first, so that the longest sweeps start first.
+// solves of the eigensolver (K_j^{-1}, Section 4.4) launch one cluster of thread
+// blocks per subdomain, and band_solve picks one kernel, one cluster size and one
+// shared-memory size for a whole launch from the widest band and the longest vector
+// of the batch.  In a batch of very uneven subdomains one large box would then size
+// every block for itself, and its block height (sweep_block) would be everyone's.  A
+// SolveSet cuts the batch (the FP32 part and the FP64 part separately) into classes
+// of one block height and similar half bandwidth, each launched with its own maxima,
+// and runs the classes concurrently: the one with the longest sweep first and on the
+// caller's stream, the others on the handle's solve streams, each on the stream that
+// is free first.  Inside a class the subdomains are ordered by cost, largest first,
+// so that the longest sweeps start first.
 #include <algorithm>
 #include <cmath>
 #include <numeric>

@@ -38,7 +38,8 @@
 // 1.69 ms for 9.23 GB: 5.5 TB/s).
 //
 // All sums run in a fixed order.  Every wait is bounded; a wait that gives up
-// records GENEO_ERR_TIMEOUT and the block goes on without waiting.
+// records GENEO_ERR_TIMEOUT and the block goes on without waiting.  A slot's clears
+// and fills are ordered by release and acquire fences (release_cluster).
 #include <algorithm>
 #include <atomic>
 #include <type_traits>
@@ -117,7 +118,9 @@ __device__ __forceinline__ uint64_t ld_cluster64(const void* p) {
   asm volatile("ld.relaxed.cluster.shared::cta.b64 %0, [%1];" : "=l"(v) : "r"(smem_u32(p)) : "memory");
   return v;
 }
-__device__ __forceinline__ double ld_cluster(const double* p) { return __longlong_as_double((long long)ld_cluster64(p)); }
+__device__ __forceinline__ double ld_cluster(const double* p) {
+  return __longlong_as_double((long long)ld_cluster64(p));
+}
 __device__ __forceinline__ dsv ld_cluster(const dsv* p) {
   const uint64_t v = ld_cluster64(p);
   return dsv(__uint_as_float((uint32_t)v), __uint_as_float((uint32_t)(v >> 32)));
@@ -388,8 +391,8 @@ __device__ __forceinline__ T chains(const T (&a)[W]) {
 }
 
 // ---------------------------------------------------------------------------
-// Multiply-add sweep (T factor storage, A arithmetic, NC columns).  Eight
-// warps of RPW = B / 8 rows each (backward: columns); the PH = 32 / RPW lanes
+// Multiply-add sweep (T factor storage, A arithmetic, NC columns).  NW = four or
+// eight warps of RPW = B / NW rows each (backward: columns); the PH = 32 / RPW lanes
 // that share a row take RPW consecutive columns (rows) of every 32, so a
 // warp's 32 band addresses fall in distinct banks (ld - 1 is odd), and the
 // row's sum ends in two to five shuffles instead of a block barrier.
@@ -871,19 +874,16 @@ k_sweep(const T* __restrict__ base, const BandDesc* __restrict__ descs, double* 
 // MMAs, a barrier), and twice the warps halve each warp's share of all but the
 // barrier (elasticity 38x31x24, half width about 500, 24 columns: the 56 sweeps of
 // the eigensolver 81 ms with eight warps, 54 ms with sixteen).
-template <int B>
-__host__ __device__ constexpr int mma_warps() {
-  return 16;
-}
+constexpr int kMmaWarps = 16;
 template <int B, int NT, int PASSES>
-__global__ void __launch_bounds__(32 * mma_warps<B>() + 32, 1)
+__global__ void __launch_bounds__(32 * kMmaWarps + 32, 1)
 k_sweep_mma(const float* __restrict__ base, const BandDesc* __restrict__ descs, double* __restrict__ xbase,
             const int64_t* __restrict__ xoff, int col0, int kcap, const int32_t* __restrict__ nrhs_dev,
             const int32_t* __restrict__ skip, int C, int nslot, int rwb, DevStatus* st) {
   using RS = RowStream<float, B>;
   constexpr int SR = RS::SR;
   constexpr int NC = 8 * NT;
-  constexpr int NW = mma_warps<B>(), kThreads = 32 * NW;
+  constexpr int NW = kMmaWarps, kThreads = 32 * NW;
   constexpr int MT = B / 16, KP = NW / MT;      // row tiles, k-parts
   constexpr int ST = B / 8;                     // k-steps per block
   constexpr int SPW = ST / KP > 0 ? ST / KP : 1;  // k-steps per warp and block
@@ -1430,7 +1430,7 @@ size_t sweep_smem(int w, int C, int nslot) {
 }
 template <int B, int NT>
 size_t mma_smem(int w, int C, int nslot) {
-  const size_t SR = B < 32 ? B : 32, NC = 8 * NT, KP = mma_warps<B>() / (B / 16);
+  const size_t SR = B < 32 ? B : 32, NC = 8 * NT, KP = kMmaWarps / (B / 16);
   return slot_lead(C) + sizeof(float) * (nslot * SR * band_ld(w) + NC * ((size_t)ring_blocks(w, B, C) * B + 1) +
                                          KP * NC * (B + 4) + NC * (B + 1) + (C > 1 ? (size_t)C * NC * B : 0));
 }
@@ -1459,7 +1459,7 @@ struct SweepArgs {
   const BandDesc* d;
   double* x;
   const int64_t* xoff;
-  int count, w, max_n, c0, kc;
+  int count, w, c0, kc;
   const int32_t *nrhs_dev, *skip;
   DevStatus* st;
   cudaStream_t s;
@@ -1516,9 +1516,9 @@ geneo_status_t run_sweep(const T* base, const SweepArgs& a, int C, int parts, in
     if (nslot > 0 || C == 1) break;
   }
   if (nslot == 0) return GENEO_ERR_ARG;
-  return launch_cluster(k_sweep<T, A, NC, B, KC>, 32 * sweep_warps<NC, B>() + 32, dim3(a.count * C, parts), C, sweep_smem<T, A, NC, B>(a.w, C, nslot),
-                        a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev, a.skip, cpp, C, nslot,
-                        ring_blocks(a.w, B, C), a.st);
+  return launch_cluster(k_sweep<T, A, NC, B, KC>, 32 * sweep_warps<NC, B>() + 32, dim3(a.count * C, parts), C,
+                        sweep_smem<T, A, NC, B>(a.w, C, nslot), a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev,
+                        a.skip, cpp, C, nslot, ring_blocks(a.w, B, C), a.st);
 }
 
 template <int B, int NT>
@@ -1530,14 +1530,9 @@ geneo_status_t run_mma(const float* base, const SweepArgs& a, int C, int parts, 
     if (nslot > 0 || C == 1) break;
   }
   if (nslot == 0) return GENEO_ERR_ARG;
-  const size_t smem = mma_smem<B, NT>(a.w, C, nslot);
-  const dim3 grid(a.count * C, parts);
-  const int rwb = ring_blocks(a.w, B, C);
-  if (passes == 1)
-    return launch_cluster(k_sweep_mma<B, NT, 1>, 32 * mma_warps<B>() + 32, grid, C, smem, a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev,
-                          a.skip, C, nslot, rwb, a.st);
-  return launch_cluster(k_sweep_mma<B, NT, 3>, 32 * mma_warps<B>() + 32, grid, C, smem, a.s, base, a.d, a.x, a.xoff, a.c0, a.kc, a.nrhs_dev,
-                        a.skip, C, nslot, rwb, a.st);
+  return launch_cluster(passes == 1 ? k_sweep_mma<B, NT, 1> : k_sweep_mma<B, NT, 3>, 32 * kMmaWarps + 32,
+                        dim3(a.count * C, parts), C, mma_smem<B, NT>(a.w, C, nslot), a.s, base, a.d, a.x, a.xoff, a.c0,
+                        a.kc, a.nrhs_dev, a.skip, C, nslot, ring_blocks(a.w, B, C), a.st);
 }
 
 }  // namespace
@@ -1591,7 +1586,7 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
                            double* xbase, const int64_t* xoff, int nrhs, const int32_t* nrhs_dev,
                            const int32_t* skip_dev, DevStatus* st, cudaStream_t s, int tc_passes, int slots,
                            int live) {
-  SweepArgs a{d_desc, xbase, xoff, count, max_w, max_n, 0, nrhs, nrhs_dev, skip_dev, st, s, live, slots};
+  SweepArgs a{d_desc, xbase, xoff, count, max_w, 0, nrhs, nrhs_dev, skip_dev, st, s, live, slots};
   // C thread blocks per matrix: the waves of blocks times the length of one
   // matrix's sweep, relative to C = 1 (rel: between what the kernels measured at
   // half widths 307-463: FP32 one column 1, 0.57, 0.35, 0.36; MMA 1, 0.54, 0.44;
@@ -1669,8 +1664,10 @@ geneo_status_t sweep_solve(const T* base, const BandDesc* d_desc, int count, int
     // the columns cut into parts of cpp per block (kernels for 3, 4 and 8); the
     // FP64 and double-single pipes are full with one block per SM, so the time
     // is the waves times the columns formed times the sweep's relative length
-    // (27 FP64 bands of order 9261, half width 463, 11 columns: 12.2 ms in three
-    // parts of 4, 11.3 in two of 6 on clusters of 2)
+    // (27 FP64 bands of order 9261, half width 463, single blocks: 8.9 ms for 3
+    // columns, 11.4 for 4, 21.9 for 8, and 0.52 and 0.40 of that on clusters of 2 and
+    // 4; so 11 columns take 8.9 ms in four parts of 3, 11.4 in three of 4 or in two
+    // of 6 on clusters of 2)
     const bool fit8 = (blk == 32   ? sweep_smem<double, A, 8, 32>(max_w, 1, 2)
                        : blk == 16 ? sweep_smem<double, A, 8, 16>(max_w, 1, 1)
                                    : sweep_smem<double, A, 8, 8>(max_w, 1, 1)) <= kSmemMax;
