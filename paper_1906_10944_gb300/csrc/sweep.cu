@@ -31,11 +31,11 @@
 //
 // Measured against one thread block per matrix in 16-row steps of forward
 // substitution: one column of 64 FP32 bands of order 5832, half width 340,
-// 785 -> 267 us; a solve with the 8 bands of a 32^3 grid 24.4 -> 6.7 ms; an FP64
+// 785 -> 267 us; a solve with the 8 bands of a 32^3 grid 24.4 -> 7.1 ms; an FP64
 // apply at 64^3 2.9 -> 1.4 ms; the eigensolver's sweeps at 48^3 in FP64 (11
 // columns, 27 bands) 653 -> 138 ms, where the FP64 pipe bounds them.  With more
 // matrices than SMs HBM bounds the one-column sweep (512 bands of a 128^3 grid,
-// 1.69 ms for 9.23 GB: 5.5 TB/s).
+// 1.74 ms for 9.23 GB: 5.3 TB/s).
 //
 // All sums run in a fixed order.  Every wait is bounded; a wait that gives up
 // records GENEO_ERR_TIMEOUT and the block goes on without waiting.  A slot's clears
